@@ -71,11 +71,12 @@ enum {
                                tensor-core matrix pass vs double-float FFT pass (both within the
                                mixed accuracy); synchronises the device */
     IDP_KEY_DST_SHAPE = 5,  /* block shape of the full-volume sine passes (results are the same
-                               bits for every shape): 0 by size (default), 8 = 8 lines per block,
-                               -8 = 8 lines on 128 threads (M = 128 only), 32 = 32 lines (M = 128
-                               only), 16 = 16 lines (M = 256 only), 4 = 4 lines on 128 threads
-                               (M = 256 and 512 only); a shape that does not apply to a length
-                               falls back to 0 */
+                               bits for every shape): 0 by size (default), 32 = most lines per
+                               block, 16 = half of them, 8 or 4 = few lines on many threads each;
+                               a shape that does not apply to a length (-8 among them) falls back
+                               to 0.  Double-float passes (tensor-core modes): 8 lines; 8 lines on
+                               128 threads (-8, M = 128); 32 lines (M = 128); 16 lines (M = 256);
+                               4 lines on 128 threads (M = 256 and 512) */
     IDP_KEY_STALL_TEST = 3, /* test hook for failure handling (mixed precision only): the next
                                tensor-core pass issues no products, so its bounded wait expires
                                (after ~5 ms); the kernel records the failure, frees its tensor
@@ -119,12 +120,11 @@ enum {
                                       differences form R) and the transforms of the boundary layers run
                                       in double-float arithmetic (48 significant bits).  Setting it
                                       allocates the pieces of the sine matrices and FP32 temporaries. */
-    IDP_PRECISION_DF32 = 2,        /* the FFT-based transforms (sine transforms of rho, R and the final
-                                      inverse, and the 3-D boundary convolutions) in double-float
-                                      arithmetic (a value is a pair of FP32 numbers, ~48 significant
-                                      bits) on the FP32 pipe, FP64 arrays in and out; the transform
-                                      producing u1 and all stencils stay FP64.  Results agree with
-                                      FP64 to a few 1e-13 relative. */
+    IDP_PRECISION_DF32 = 2,        /* the 3-D boundary convolutions (and the direct sine sums of lengths
+                                      without an FFT) in double-float arithmetic (a value is a pair of
+                                      FP32 numbers, ~48 significant bits) on the FP32 pipe, FP64 arrays
+                                      in and out; the sine transforms and all stencils as in FP64.
+                                      Results agree with FP64 to a few 1e-13 relative. */
     IDP_PRECISION_MIXED_TF32X3 = 3 /* as MIXED_BF16X3, with the operands split into two TF32 pieces
                                       (hi + lo, ~22 significant bits) and three products (hi*hi,
                                       hi*lo, lo*hi; tcgen05 kind::tf32), FP32 accumulation */

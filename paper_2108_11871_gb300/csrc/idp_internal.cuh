@@ -49,20 +49,19 @@ struct DstPass {
     int n0, n1, n2;
     int axis;
     int M;
-    const Tw *tw;          // twiddles for the complex FFT of length M/2
-    const double2 *half;   // half-step twiddles for length M/2 (e^{-i pi k/(M/2)})
-    const Tw *halfr;       // the same in ratio form
-    const double *sin2;    // 2 sin(pi j / M), j = 0..M/2
+    // fixed-point tables (q64.cuh): the factors of the complex FFT of
+    // length K = M/2 pass by pass, e^{-i pi k/K} (k = 0..K/2), sin(pi j/M) (j = 0..K-1)
+    const int4 *qtab;
+    int in_dd;             // the input holds double-float pairs
+    int lines;   // lines per block: 0 = by size, 8 = fewest, 16, 32 = most
     // double-float variant (dd = 1): arithmetic on the FP32 pipe; in/out/add
     // may hold FP64 values or double-float pairs (in_dd / out_dd / add_dd)
     int dd;
-    int in_dd, out_dd, add_dd;
+    int out_dd, add_dd;
     const ddr *tabd;       // tab as double-float pairs (if not null, used instead of tab)
-    const TwD *twd;
-    const ddc *halfd;
-    const ddr *sin2d;
-    int lines;   // lines per block: 0 = by size (8 for launches of < 2 blocks per SM), 8 = always 8,
-                 // -8 = 8 lines on 128 threads (M = 128), 32 (M = 128), 16 (M = 256)
+    const TwD *twd;        // twiddles for the complex FFT of length M/2
+    const ddc *halfd;      // half-step twiddles for length M/2 (e^{-i pi k/(M/2)})
+    const ddr *sin2d;      // 2 sin(pi j / M), j = 0..M/2
     const void *sinm;      // lengths without an FFT: the sine matrix S[i][e] = sin(pi (i+1)(e+1)/M),
                            // e fastest, FP64 (dd = 0) or double-float pairs (dd = 1): direct sums
 };
@@ -71,10 +70,12 @@ struct DstPass {
 // launch of its stream be placed on the GPU while it runs (pdl_enter at its start),
 // and waits for the previous launch to complete and flush before it reads
 // anything (also in pdl_enter).  For a kernel launched otherwise both are no-ops.
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 __device__ __forceinline__ void pdl_enter()
 {
-    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
-    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    pdl_launch();
+    pdl_wait();
 }
 template <class Kern, class... Args>
 cudaError_t launch_pdl(Kern kern, dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args)
@@ -94,6 +95,11 @@ cudaError_t launch_pdl(Kern kern, dim3 grid, dim3 block, size_t smem, cudaStream
 
 cudaError_t launch_dst_pass(const DstPass &a, cudaStream_t st);
 cudaError_t dst_set_attributes();
+cudaError_t launch_dst_dd(const DstPass &a, cudaStream_t st);
+cudaError_t dst_dd_set_attributes();
+bool q_supported(int L);                    // lengths with a fixed-point FFT (q64.cuh)
+int q_table_radix(int L, int Ns, int RM);   // the radix of its pass after span Ns
+int dst_table_radix(int K);                 // RM of the sine passes' FFT of length K
 cudaError_t boundary_set_attributes();
 
 // ---- mixed-precision sine pass on the tensor cores (mixed.cu) ---------------

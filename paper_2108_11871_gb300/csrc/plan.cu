@@ -117,6 +117,37 @@ TwD make_twd(const Tw &t)
     return d;
 }
 
+// a factor in [-1, 1] in the two-word fixed-point form of q64.cuh: ch 2^-31 + cl 2^-62
+int2 fixed_factor(long double c)
+{
+    const long double top = 2147483647.0L, a = c * 2147483648.0L;
+    const long double h = std::min(top, std::nearbyint(a));
+    return make_int2((int)h, (int)std::min(top, std::nearbyint((a - h) * 2147483648.0L)));
+}
+// cos and sin of pi m / L to the precision of that form (argument reduced to the first octant)
+void cossinpi(int64_t m, int64_t L, long double &c, long double &s)
+{
+    const long double pi = 3.14159265358979323846264338327950288L;
+    m %= 2 * L;
+    if (m < 0) m += 2 * L;
+    int64_t r = m % L;                     // angle pi r / L in [0, pi)
+    const bool neg = m >= L, obtuse = 2 * r > L;
+    if (obtuse) r = L - r;
+    const bool swap = 4 * r > L;
+    const long double t = swap ? pi * (long double)(L - 2 * r) / (long double)(2 * L) : pi * (long double)r / (long double)L;
+    c = swap ? std::sin(t) : std::cos(t);
+    s = swap ? std::cos(t) : std::sin(t);
+    if (obtuse) c = -c;
+    if (neg) { c = -c; s = -s; }
+}
+int4 fixed_unit(int64_t m, int64_t L)      // e^{-i pi m / L}
+{
+    long double c, s;
+    cossinpi(m, L, c, s);
+    const int2 x = fixed_factor(c), y = fixed_factor(-s);
+    return make_int4(x.x, x.y, y.x, y.y);
+}
+
 std::mutex g_attr_mu;
 std::atomic<uint64_t> g_serial{1};
 std::vector<int> g_attr_done;
@@ -171,8 +202,8 @@ struct idp_plan_s {
     StencilCoef coef{};
 
     std::map<int, DevFft> fft;        // by complex length
-    std::map<int, double *> sin2;     // by M: 2 sin(pi j / M), j = 0..M/2
-    std::map<int, ddr *> sin2d;       // double-float form
+    std::map<int, ddr *> sin2d;       // by M: 2 sin(pi j / M), j = 0..M/2, double-float pairs
+    std::map<int, int4 *> qdst;       // by M: fixed-point tables of the sine passes
     std::map<int, double *> sinm;     // by M (lengths without an FFT): sine matrices for direct sums
     std::map<int, ddr *> sinmd;       // double-float form
     int exact = 0;                    // created by idp_create_plan_exact
@@ -386,28 +417,59 @@ int get_fft(idp_plan p, int L, FftTables *out)
     return IDP_OK;
 }
 
-int get_sin2(idp_plan p, int M, const double **out)
+// 2 sin(pi j / M), j <= M/2, as double-float pairs
+int get_sin2d(idp_plan p, int M, const ddr **out)
 {
-    auto it = p->sin2.find(M);
-    if (it != p->sin2.end()) {
-        *out = it->second;
-        return IDP_OK;
+    auto it = p->sin2d.find(M);
+    if (it == p->sin2d.end()) {
+        std::vector<ddr> s(M / 2 + 1);
+        for (int j = 0; j <= M / 2; ++j) s[j] = host_dd(2.0 * sinpi_frac(j, M));
+        ddr *d = nullptr;
+        int rc;
+        if ((rc = p->alloc(&d, M / 2 + 1))) return rc;
+        IDP_CK(cudaMemcpy(d, s.data(), sizeof(ddr) * s.size(), cudaMemcpyHostToDevice));
+        it = p->sin2d.emplace(M, d).first;
     }
-    std::vector<double> s(M / 2 + 1);
-    std::vector<ddr> sd(M / 2 + 1);
-    for (int j = 0; j <= M / 2; ++j) {
-        s[j] = 2.0 * sinpi_frac(j, M);
-        sd[j] = host_dd(s[j]);
+    *out = it->second;
+    return IDP_OK;
+}
+
+// factors of the fixed-point FFT of length L, pass by pass (q64.cuh), radices up to RM
+std::vector<int4> q_factors(int L, int RM)
+{
+    std::vector<int4> q;
+    for (int Ns = 1; Ns < L;) {
+        const int R = q_table_radix(L, Ns, RM);
+        if (Ns > 1)
+            for (int r = 1; r < R; ++r)
+                for (int k = 0; k < Ns; ++k) q.push_back(fixed_unit(2 * (int64_t)r * k, (int64_t)R * Ns));
+        Ns *= R;
     }
-    double *d = nullptr;
-    ddr *dd = nullptr;
-    int rc;
-    if ((rc = p->alloc(&d, M / 2 + 1)) || (rc = p->alloc(&dd, M / 2 + 1))) return rc;
-    IDP_CK(cudaMemcpy(d, s.data(), sizeof(double) * (M / 2 + 1), cudaMemcpyHostToDevice));
-    IDP_CK(cudaMemcpy(dd, sd.data(), sizeof(ddr) * (M / 2 + 1), cudaMemcpyHostToDevice));
-    p->sin2[M] = d;
-    p->sin2d[M] = dd;
-    *out = d;
+    return q;
+}
+
+// the tables of the sine passes of M panels: see DstPass
+int get_dst_tables(idp_plan p, int M, const int4 **out)
+{
+    auto it = p->qdst.find(M);
+    if (it == p->qdst.end()) {
+        const int K = M / 2;
+        std::vector<int4> q = q_factors(K, dst_table_radix(K));
+        for (int k = 0; k <= K / 2; ++k) q.push_back(fixed_unit(k, K));
+        int2 sn[2];
+        for (int j = 0; j < K; ++j) {
+            long double c, s;
+            cossinpi(j, M, c, s);
+            sn[j & 1] = fixed_factor(s);
+            if (j & 1) q.push_back(make_int4(sn[0].x, sn[0].y, sn[1].x, sn[1].y));
+        }
+        int4 *d = nullptr;
+        int rc;
+        if ((rc = p->alloc(&d, (int64_t)q.size()))) return rc;
+        IDP_CK(cudaMemcpy(d, q.data(), sizeof(int4) * q.size(), cudaMemcpyHostToDevice));
+        it = p->qdst.emplace(M, d).first;
+    }
+    *out = it->second;
     return IDP_OK;
 }
 
@@ -675,22 +737,23 @@ int transform(idp_plan p, View3 in, double *work, View3 out, const double *tab, 
         int rc;
         if (has_fft_dst(p->M[s])) {
             if ((rc = get_fft(p, p->M[s] / 2, &t))) return rc;
-            a.tw = t.fwd;
-            a.half = t.half;
-            a.halfr = t.halfr;
-            if ((rc = get_sin2(p, p->M[s], &a.sin2))) return rc;
+            if ((rc = get_dst_tables(p, p->M[s], &a.qtab))) return rc;
         } else if ((rc = get_sinm(p, p->M[s], &a.sinm, dd ? 1 : 0))) {   // direct sums
             return rc;
         }
-        if (dd) {
-            // double-float arithmetic; intermediate passes keep double-float pairs
+        // the tensor-core modes keep double-float passes (their results are compared
+        // bit for bit where a rounding to FP32 follows); precision DF32 runs the
+        // fixed-point FFT, and double-float only in the direct sums
+        a.in_dd = (q == 0) ? in_dd0 : 0;
+        if (dd && (tensor_mode(p) || !has_fft_dst(p->M[s]))) {
             a.dd = 1;
-            a.in_dd = (q == 0) ? in_dd0 : 1;
-            a.out_dd = (q == na - 1) ? 0 : 1;
-            a.add_dd = 0;
+            if (tensor_mode(p)) {   // intermediate passes keep double-float pairs
+                if (q > 0) a.in_dd = 1;
+                a.out_dd = q < na - 1;
+            }
             a.twd = t.fwdd;
             a.halfd = t.halfd;
-            if (has_fft_dst(p->M[s])) a.sin2d = p->sin2d[p->M[s]];
+            if (has_fft_dst(p->M[s]) && (rc = get_sin2d(p, p->M[s], &a.sin2d))) return rc;
         }
         Mark mk(p, IDP_KERNEL_DST, st);
         IDP_CK(launch_dst_pass(a, st));
@@ -717,18 +780,15 @@ int dst_box(idp_plan p, double *x, int b0, int b1, int b2, int M2, int M1, cudaS
         const bool ddm = p->mixed == IDP_PRECISION_DF32 || tensor_mode(p);
         if (has_fft_dst(Ms[q])) {
             if ((rc = get_fft(p, Ms[q] / 2, &t))) return rc;
-            a.tw = t.fwd;
-            a.half = t.half;
-            a.halfr = t.halfr;
-            if ((rc = get_sin2(p, Ms[q], &a.sin2))) return rc;
+            if ((rc = get_dst_tables(p, Ms[q], &a.qtab))) return rc;
         } else if ((rc = get_sinm(p, Ms[q], &a.sinm, ddm ? 1 : 0))) {   // direct sums
             return rc;
         }
-        if (ddm) {
+        if (ddm && (tensor_mode(p) || !has_fft_dst(Ms[q]))) {
             a.dd = 1;
             a.twd = t.fwdd;
             a.halfd = t.halfd;
-            if (has_fft_dst(Ms[q])) a.sin2d = p->sin2d[Ms[q]];
+            if (has_fft_dst(Ms[q]) && (rc = get_sin2d(p, Ms[q], &a.sin2d))) return rc;
         }
         Mark mk(p, IDP_KERNEL_DST_PARTS, st);
         IDP_CK(launch_dst_pass(a, st));
@@ -1198,9 +1258,10 @@ int plan_setup(idp_plan p)
     for (int s = 0; s < 3; ++s) {
         if (!p->act[s]) continue;
         FftTables t;
-        const double *sn;
+        const int4 *qt;
+        const ddr *sd;
         const void *sm_;
-        if ((has_fft_dst(p->M[s]) && ((rc = get_fft(p, p->M[s] / 2, &t)) || (rc = get_sin2(p, p->M[s], &sn)))) ||
+        if ((has_fft_dst(p->M[s]) && ((rc = get_fft(p, p->M[s] / 2, &t)) || (rc = get_dst_tables(p, p->M[s], &qt)) || (rc = get_sin2d(p, p->M[s], &sd)))) ||
             (!has_fft_dst(p->M[s]) && (rc = get_sinm(p, p->M[s], &sm_, 0))) ||
             (rc = get_fft(p, p->P[s], &t)) || (rc = get_fft(p, 2 * p->P[s], &t)))
             return rc;

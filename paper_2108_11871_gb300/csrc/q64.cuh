@@ -1,0 +1,218 @@
+// Block fixed-point ("q64") arithmetic for the FP64-class transforms, and the
+// block-cooperative complex FFT built on it.
+//
+// GB300 issues FP64 at 2 lanes per clock and SM (measured: 64 cycles per warp
+// instruction and scheduler), but a 32 x 32 -> 64-bit integer multiply-add at 60 lanes
+// (2.1 cycles).  A radix-4 unit with its three twiddle products takes about 200
+// cycles in 64-bit integers against 1540 in FP64, so the transforms run in
+// integers: the values of one line share a power-of-two scale, chosen from a bound on
+// the line's absolute sum so that no intermediate can overflow, and every value is
+// a signed 64-bit integer in units of that scale.  Additions are exact; a
+// product with a twiddle (62 fractional bits) is off by about one unit at most.  A unit
+// is 2^-58 to 2^-59 of the line's absolute sum, and every output is bounded by that sum.
+#pragma once
+#include <cstdint>
+#include <cuda_runtime.h>
+
+#include "idp_internal.cuh"
+
+namespace idp {
+
+struct __align__(16) qc {
+    long long re, im;
+};
+
+__device__ __forceinline__ long long q_mulw(int a, int b) { return (long long)a * b; }
+__device__ __forceinline__ long long q_madw(int a, int b, long long c) { return (long long)a * b + c; }
+
+__device__ __forceinline__ qc q_add(qc a, qc b) { return qc{a.re + b.re, a.im + b.im}; }
+__device__ __forceinline__ qc q_sub(qc a, qc b) { return qc{a.re - b.re, a.im - b.im}; }
+
+// A factor c in [-1, 1] is ch 2^-31 + cl 2^-62 (|cl| <= 2^30, except c = 1: ch = cl =
+// 2^31 - 1, 2^-62 below 1); a value x is xh 2^31 + xl with 0 <= xl < 2^31:
+//   x c = xh ch + (xh cl + xl ch) 2^-31 + xl cl 2^-62,
+// the last term (below one unit) dropped and the bracket rounded to nearest (a rounding
+// down is a bias, which the lowest modes add up over the line: measured ten times the
+// error of FP64 on noise at M = 512, against the same).  |x| <= 2^61 keeps the bracket
+// (for a complex product, the sum of two of them with c^2 + s^2 = 1) within 63 bits.
+constexpr long long Q_HALF = 1LL << 30;
+__device__ __forceinline__ long long q_rmul(long long x, int ch, int cl)
+{
+    const int xh = (int)(x >> 31), xl = (int)((unsigned)x & 0x7fffffffu);
+    const long long m = q_madw(xl, ch, q_madw(xh, cl, Q_HALF));
+    return q_madw(xh, ch, m >> 31);
+}
+
+__device__ __forceinline__ qc q_cmul(qc a, int4 w)   // w = (ch, cl, sh, sl): a (c + i s)
+{
+    const int xh = (int)(a.re >> 31), xl = (int)((unsigned)a.re & 0x7fffffffu);
+    const int yh = (int)(a.im >> 31), yl = (int)((unsigned)a.im & 0x7fffffffu);
+    // the two halves of the real part are formed apart and subtracted (measured 6 %
+    // faster than negating the factor words)
+    const long long m = q_madw(xl, w.x, q_madw(xh, w.y, Q_HALF)) - q_madw(yl, w.z, q_mulw(yh, w.w));
+    const long long n = q_madw(yl, w.x, q_madw(yh, w.y, q_madw(xl, w.z, q_madw(xh, w.w, Q_HALF))));
+    qc r;
+    r.re = q_madw(xh, w.x, m >> 31) - q_mulw(yh, w.z);
+    r.im = q_madw(yh, w.x, q_madw(xh, w.z, n >> 31));
+    return r;
+}
+
+constexpr int Q_R2H = 1518500250, Q_R2L = -25716447;    // sqrt(1/2)
+constexpr int Q_S3H = 1859775393, Q_S3L = 815355111;    // sqrt(3)/2
+
+// forward DFTs (e^{-2 pi i/R}) in registers, natural order in and out
+__device__ __forceinline__ void q_dft2(qc *v)
+{
+    const qc a = v[0];
+    v[0] = q_add(a, v[1]);
+    v[1] = q_sub(a, v[1]);
+}
+__device__ __forceinline__ void q_dft3(qc *v)
+{
+    const qc t = q_add(v[1], v[2]), d = q_sub(v[1], v[2]);
+    // t / 2, an odd t rounded up or down by the last bit of another value (no bias)
+    const qc m = qc{v[0].re - ((t.re + (v[0].re & 1)) >> 1), v[0].im - ((t.im + (v[0].im & 1)) >> 1)};
+    const long long pr = q_rmul(d.im, Q_S3H, Q_S3L), pi = q_rmul(d.re, Q_S3H, Q_S3L);
+    v[0] = q_add(v[0], t);
+    v[1] = qc{m.re + pr, m.im - pi};
+    v[2] = qc{m.re - pr, m.im + pi};
+}
+__device__ __forceinline__ void q_dft4(qc &a0, qc &a1, qc &a2, qc &a3)
+{
+    const qc c0 = q_add(a0, a2), c1 = q_sub(a0, a2), e0 = q_add(a1, a3), e1 = q_sub(a1, a3);
+    a0 = q_add(c0, e0);
+    a2 = q_sub(c0, e0);
+    a1 = qc{c1.re + e1.im, c1.im - e1.re};
+    a3 = qc{c1.re - e1.im, c1.im + e1.re};
+}
+__device__ __forceinline__ void q_dft8(qc *v)
+{
+    q_dft4(v[0], v[2], v[4], v[6]);   // E_0..3
+    q_dft4(v[1], v[3], v[5], v[7]);   // O_0..3
+    const qc t0 = v[1];
+    const qc t1 = qc{q_rmul(v[3].re + v[3].im, Q_R2H, Q_R2L), q_rmul(v[3].im - v[3].re, Q_R2H, Q_R2L)};
+    const qc t2 = qc{v[5].im, -v[5].re};
+    const qc t3 = qc{q_rmul(v[7].im - v[7].re, Q_R2H, Q_R2L), -q_rmul(v[7].re + v[7].im, Q_R2H, Q_R2L)};
+    const qc e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6];
+    v[0] = q_add(e0, t0);
+    v[4] = q_sub(e0, t0);
+    v[1] = q_add(e1, t1);
+    v[5] = q_sub(e1, t1);
+    v[2] = q_add(e2, t2);
+    v[6] = q_sub(e2, t2);
+    v[3] = q_add(e3, t3);
+    v[7] = q_sub(e3, t3);
+}
+template <int R>
+__device__ __forceinline__ void q_dft(qc *v)
+{
+    if constexpr (R == 2) q_dft2(v);
+    else if constexpr (R == 3) q_dft3(v);
+    else if constexpr (R == 4) q_dft4(v[0], v[1], v[2], v[3]);
+    else q_dft8(v);
+}
+
+// shared-memory place of element e of a line (16-byte elements): the three low bits are
+// XORed with the next three, so that the eight lanes of a quarter-warp hit eight
+// bank groups both in a pass's reads (consecutive e) and in its writes (stride R)
+__device__ __forceinline__ int q_slot(int e) { return e ^ ((e >> 3) & 7); }
+
+// The radices of the passes of length L after a span of Ns: one radix-3 pass first for
+// 3 * 2^m, then radix-4 (or radix-2) until a power of RM (4 or 8) is left, then RM.
+__host__ __device__ constexpr int q_radix(int L, int Ns, int RM)
+{
+    const int rest = L / Ns;
+    if (rest % 3 == 0) return 3;
+    int p = 1;
+    while (p * RM <= rest) p *= RM;
+    const int head = rest / p;
+    if (head == 4) return 4;
+    if (head == 2) return RM == 8 && rest >= 16 ? 4 : 2;   // 16 = 4 * 4, 128 = 4 * 4 * 8
+    return RM;
+}
+__host__ __device__ constexpr int q_passes(int L, int RM, int Ns = 1)
+{
+    return Ns == L ? 0 : 1 + q_passes(L, RM, Ns * q_radix(L, Ns, RM));
+}
+// entries of the factor table of length L, from span Ns on
+__host__ __device__ constexpr int q_tw_count(int L, int RM, int Ns = 1)
+{
+    return Ns == L ? 0 : (Ns > 1 ? (q_radix(L, Ns, RM) - 1) * Ns : 0) + q_tw_count(L, RM, Ns * q_radix(L, Ns, RM));
+}
+
+// One Stockham pass of radix R at span Ns over LB lines (line stride LS elements) by
+// NT threads; tw: the pass's factors w_{R Ns}^{k q}, [q - 1][k].
+template <int L, int Ns, int RM, int LB, int NT, int LS>
+__device__ __forceinline__ void q_pass(const qc *__restrict__ X, qc *__restrict__ Y, const int4 *__restrict__ tw)
+{
+    constexpr int R = q_radix(L, Ns, RM), U = L / R;
+#pragma unroll 1
+    for (int b = threadIdx.x; b < LB * U; b += NT) {
+        const int line = b / U, j = b - line * U, k = j % Ns;
+        const qc *x = X + line * LS;
+        qc v[R];
+#pragma unroll
+        for (int q = 0; q < R; ++q) v[q] = x[q_slot(j + q * U)];
+        if constexpr (Ns > 1) {
+#pragma unroll
+            for (int q = 1; q < R; ++q) v[q] = q_cmul(v[q], tw[(q - 1) * Ns + k]);
+        }
+        q_dft<R>(v);
+        qc *y = Y + line * LS;
+        const int base = (j - k) * R + k;
+#pragma unroll
+        for (int q = 0; q < R; ++q) y[q_slot(base + q * Ns)] = v[q];
+    }
+}
+
+// Forward FFT of LB lines of length L (a multiple of 8) in X, from span Ns on; Y is
+// scratch.  The result is in X if the number of passes is even, else in Y; ends
+// with a block barrier.  tw: the factors of the passes after span Ns, one after the
+// other (none for the first pass at Ns = 1).
+template <int L, int RM, int LB, int NT, int LS, int Ns = 1>
+__device__ __forceinline__ void q_fft(qc *X, qc *Y, const int4 *__restrict__ tw)
+{
+    if constexpr (Ns < L) {
+        constexpr int R = q_radix(L, Ns, RM);
+        q_pass<L, Ns, RM, LB, NT, LS>(X, Y, tw);
+        __syncthreads();
+        q_fft<L, RM, LB, NT, LS, Ns * R>(Y, X, tw + (Ns > 1 ? (R - 1) * Ns : 0));
+    }
+}
+
+// ---- scales --------------------------------------------------------------------
+// A line's scale from two reductions over its FP64 values: the largest exponent field
+// emax, and the sum S of q_weight (the magnitudes in units of 2^(emax - 1043), each
+// rounded up).  With bits = bit length of S, the absolute sum is below 2^(emax - 1043 + bits).
+// (a subnormal value has the exponent field 1 and no leading bit; zeros weigh 1 unit)
+__device__ __forceinline__ int q_expo(double x) { return max((__double2hiint(x) >> 20) & 0x7ff, 1); }
+__device__ __forceinline__ unsigned q_lead(int h) { return (h & 0x7ff00000) ? 0x100000u : 0u; }
+__device__ __forceinline__ unsigned q_weight(double x, int emax)
+{
+    const int h = __double2hiint(x);
+    const unsigned m = ((unsigned)h & 0xfffffu) | q_lead(h);
+    return (m >> min(emax - q_expo(x), 31)) + 1u;
+}
+__device__ __forceinline__ int q_bits(unsigned S) { return max(32 - __clz((int)S), 21); }
+
+// x 2^(1101 - emax - bits) rounded to nearest: below 2^58 in sum over the line
+__device__ __forceinline__ long long q_from(double x, int shift)   // shift = emax + bits - 19
+{
+    const int h = __double2hiint(x);
+    const unsigned m = ((unsigned)h & 0xfffffu) | q_lead(h);
+    const unsigned long long f = (((unsigned long long)m << 32) | (unsigned)__double2loint(x)) << 7;
+    const int r = min(shift - q_expo(x), 63);
+    const long long v = (long long)(((f >> (r - 1)) + 1) >> 1), s = h >> 31;
+    return (v ^ s) - s;
+}
+constexpr int Q_NAN = 1 << 30;   // scale of a line with a NaN or an infinity
+// v 2^-s as FP64; fast: 2^-s and every |v| keep the result normal
+__device__ __forceinline__ bool q_fast(int s) { return s <= 1022 && s >= -960; }
+__device__ __forceinline__ double q_to(long long v, int s, bool fast)
+{
+    const double d = __ll2double_rn(v);
+    if (fast) return __hiloint2double(v ? __double2hiint(d) - (s << 20) : 0, __double2loint(d));
+    return s == Q_NAN ? __longlong_as_double(0x7ff8000000000000LL) : scalbn(d, -s);
+}
+
+}  // namespace idp
