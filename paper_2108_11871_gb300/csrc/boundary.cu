@@ -16,6 +16,7 @@
 #include <type_traits>
 
 #include "fft.cuh"
+#include "q64.cuh"
 
 namespace idp {
 
@@ -243,6 +244,191 @@ __global__ void __launch_bounds__(RfftThreads<R, L>::value) rfft_kernel(const Rf
             double2 *ol = outb + (int64_t)threadIdx.x * osv;
             ol[0] = make_double2(times2_exact(z0.x + z0.y), 0.0);
             ol[(int64_t)L * ose] = make_double2(times2_exact(z0.x - z0.y), 0.0);
+        }
+    }
+}
+
+// ---------------------------------------------------------------- stage 1, fixed point
+// The FP64 form of stage 1 in block fixed point (q64.cuh): every line on its own
+// scale, FP64 in and out.  G threads per line, C of its elements each; LB lines per block.
+// Two shapes: up to 256 threads with 8 or 12 elements each, and, for launches below four of
+// its blocks per SM, whose time is the latency of one block, fewer lines on up to four
+// times the threads per line (65^2: 28 us per solve with the first, 22 with the second).
+template <int L_, bool THIN>
+struct QLineCfg {
+    static constexpr int L = L_;
+    static constexpr int G0 = L % 3 == 0 ? L / 12 : L / 8, G1 = 4 * G0 > 64 ? 64 : 4 * G0;
+    static constexpr int G = THIN ? G1 : G0, C = L / G, W = G < 32 ? G : 32;
+    static constexpr int LBw = (THIN || L % 3 == 0 ? 128 : 256) / G;
+    static constexpr int LB = LBw < 32 ? LBw : 32, T = LB * G;
+    static constexpr int LS = L + 1, BUF = LB * LS, RM = 8, TW = q_tw_count(L, RM);
+    static constexpr size_t SMEM = sizeof(qc) * (2 * BUF + TW);
+    static_assert((G & (G - 1)) == 0 && T % 32 == 0, "power-of-two groups, whole warps");
+    static_assert(sizeof(int) * (L + LB) <= sizeof(qc) * BUF, "the non-zero marks fit the scratch buffer");
+};
+
+template <int L, bool THIN>
+__global__ void __launch_bounds__(QLineCfg<L, THIN>::T) rfft_q_kernel(const RfftPass a)
+{
+    using Cfg = QLineCfg<L, THIN>;
+    constexpr int LB = Cfg::LB, NT = Cfg::T, G = Cfg::G, C = Cfg::C, LS = Cfg::LS;
+    const int M = a.M, N = M - 1;
+    extern __shared__ qc smem_q[];
+    qc *bufA = smem_q, *bufB = smem_q + Cfg::BUF;
+    int4 *tws = reinterpret_cast<int4 *>(bufB + Cfg::BUF);
+    __shared__ int s_emax[LB], s_scale[LB], s_any;
+    __shared__ unsigned s_sum[LB];
+    int nv;
+    int64_t isu, isv, ise, osu, osv, ose;
+    if (a.axis == 2) {
+        nv = a.n1;
+        isu = a.is0; isv = a.is1; ise = a.is2; osu = a.os0; osv = a.os1; ose = a.os2;
+    } else if (a.axis == 1) {
+        nv = a.n2;
+        isu = a.is0; isv = a.is2; ise = a.is1; osu = a.os0; osv = a.os2; ose = a.os1;
+    } else {
+        nv = a.n2;
+        isu = a.is1; isv = a.is2; ise = a.is0; osu = a.os1; osv = a.os2; ose = a.os0;
+    }
+    const int u = blockIdx.y, v0 = blockIdx.x * LB;
+    const int nl = min(LB, nv - v0);
+    const bool contig = (ise == 1);
+    double2 *outb = a.out + (int64_t)u * osu + (int64_t)v0 * osv;
+    // lines that are all zero (rho vanishes near the boundary): zero spectra
+    auto write_zero = [&]() {
+        for (int f = threadIdx.x; f < nl * (L + 1); f += NT) {
+            const int l = f / (L + 1), m = f - l * (L + 1);
+            outb[(int64_t)l * osv + (int64_t)m * ose] = make_double2(0.0, 0.0);
+        }
+    };
+    if (a.lineflag) {
+        if (threadIdx.x == 0) s_any = 0;
+        __syncthreads();
+        if (threadIdx.x < nl && a.lineflag[(int64_t)u * nv + v0 + threadIdx.x]) s_any = 1;
+        __syncthreads();
+        if (!s_any) {
+            write_zero();
+            return;
+        }
+    }
+    // stage 1a: non-zero marks of the block's lines and of their element
+    // positions, in the FFT scratch (free until the FFT)
+    const bool mk = a.fl_row2 != nullptr;
+    int *colnz = reinterpret_cast<int *>(bufB), *rownz = colnz + L;
+    if (threadIdx.x < LB) {
+        s_emax[threadIdx.x] = 1;
+        s_sum[threadIdx.x] = 0;
+    }
+    if (mk)
+        for (int f = threadIdx.x; f < L + LB; f += NT) colnz[f] = 0;
+    for (int f = threadIdx.x; f < Cfg::TW; f += NT) tws[f] = __ldg(a.q + f);
+
+    // 1. load: thread (l, g) takes the elements e = g + i G of line l
+    const int l = contig ? threadIdx.x / G : threadIdx.x % LB;
+    const int g = contig ? threadIdx.x % G : threadIdx.x / LB;
+    const int64_t inb = (int64_t)u * isu + (int64_t)(v0 + l) * isv;
+    double x[C];
+#pragma unroll
+    for (int i = 0; i < C; ++i) {
+        const int e = g + i * G;
+        x[i] = (l < nl && e < N) ? a.in[inb + (int64_t)e * ise] : 0.0;
+    }
+    if (a.copy) {
+#pragma unroll
+        for (int i = 0; i < C; ++i) {
+            const int e = g + i * G;
+            if (l < nl && e < N) a.copy[inb + (int64_t)e * ise] = x[i];
+        }
+    }
+    __syncthreads();   // the scales and marks are reset
+    int emax = 1;
+    bool nz = false;
+#pragma unroll
+    for (int i = 0; i < C; ++i) {
+        emax = max(emax, q_expo(x[i]));
+        // zero test on the bits (+0 and -0 are zero)
+        if ((__double_as_longlong(x[i]) << 1) != 0) {
+            nz = true;
+            if (mk) colnz[g + i * G] = 1;
+        }
+    }
+    if (mk && nz) rownz[l] = 1;
+    // 2. the line's scale (lanes of one line: consecutive ones, or those LB apart)
+    const int d0 = contig ? 1 : LB, d1 = contig ? Cfg::W : 32;
+    for (int d = d0; d < d1; d <<= 1) emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, d));
+    const bool lead = contig ? (threadIdx.x & (Cfg::W - 1)) == 0 : (threadIdx.x & 31) < LB;
+    if (lead) atomicMax(&s_emax[l], emax);
+    const int any = __syncthreads_or(nz);
+    if (mk) {
+        if (threadIdx.x < nl) {
+            const int rf = rownz[threadIdx.x];
+            a.fl_row2[(int64_t)u * nv + v0 + threadIdx.x] = rf;
+            // flags shared by many blocks are read before they are set (a store to
+            // a line that many SMs write is slow; a stale 0 costs one more store)
+            if (rf && !a.fl_sl1[v0 + threadIdx.x]) a.fl_sl1[v0 + threadIdx.x] = 1;
+        }
+        if (any) {
+            if (threadIdx.x == 0 && !a.fl_sl0[u]) a.fl_sl0[u] = 1;
+            for (int e = threadIdx.x; e < N; e += NT)
+                if (colnz[e]) {
+                    int *f1 = a.fl_row1 + (int64_t)u * a.n2 + e;
+                    if (!*f1) *f1 = 1;
+                    if (!a.fl_sl2[e]) a.fl_sl2[e] = 1;
+                }
+        }
+    }
+    if (!any) {
+        write_zero();
+        return;
+    }
+    emax = s_emax[l];
+    unsigned sum = 0;
+#pragma unroll
+    for (int i = 0; i < C; ++i) sum += q_weight(x[i], emax);
+    for (int d = d0; d < d1; d <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
+    if (lead) atomicAdd(&s_sum[l], sum);
+    __syncthreads();
+    const int bits = q_bits(s_sum[l]);
+    if (threadIdx.x < LB) {
+        const int e = s_emax[threadIdx.x];
+        s_scale[threadIdx.x] = e == 0x7ff ? Q_NAN : 1102 - e - q_bits(s_sum[threadIdx.x]);
+    }
+    // 3. into bufA viewed as reals: x_e at position e + 1 of the padded sequence (component
+    //    1 of element e / 2 for even e), zeros elsewhere; the elements from L / 2 on are
+    //    zero and are not read by the first pass
+    {
+        long long *zl = reinterpret_cast<long long *>(bufA + l * LS);
+        const int shift = emax + bits - 20;
+#pragma unroll
+        for (int i = 0; i < C; ++i) {
+            const int q = g + i * G + 1;   // <= L
+            if (q < L) zl[2 * q_slot(q >> 1) + (q & 1)] = q_from(x[i], shift);
+        }
+        if (g == 0) zl[0] = 0;
+    }
+    __syncthreads();
+    // 4. complex FFT of length L
+    q_fft<L, Cfg::RM, LB, NT, LS, 1, true>(bufA, bufB, tws);
+    const qc *Z = q_passes(L, Cfg::RM) % 2 == 0 ? bufA : bufB;
+    // 5. X'_m = 2 X_m, m = 0..L
+    for (int f = threadIdx.x; f < LB * (L / 2); f += NT) {
+        const int ll = f / (L / 2);
+        const int m = f - ll * (L / 2) + 1;   // 1..L/2
+        if (ll >= nl) continue;
+        const qc *zl = Z + ll * LS;
+        const qc zm = zl[q_slot(m)], zc = zl[q_slot(L - m)];
+        const long long Er = zm.re + zc.re, Ei = zm.im - zc.im;
+        const qc P = q_cmul(qc{zm.re - zc.re, zm.im + zc.im}, __ldg(a.qhalf + m));   // W O = P; X' = E - i P
+        const int s = s_scale[ll];
+        const bool fast = q_fast(s);
+        double2 *ol = outb + (int64_t)ll * osv;
+        ol[(int64_t)m * ose] = make_double2(q_to(Er + P.im, s, fast), q_to(Ei - P.re, s, fast));
+        ol[(int64_t)(L - m) * ose] = make_double2(q_to(Er - P.im, s, fast), q_to(-Ei - P.re, s, fast));
+        if (m == 1) {
+            const qc z0 = zl[0];
+            ol[0] = make_double2(q_to((z0.re + z0.im) << 1, s, fast), s == Q_NAN ? q_to(0, s, fast) : 0.0);
+            ol[(int64_t)L * ose] =
+                make_double2(q_to((z0.re - z0.im) << 1, s, fast), s == Q_NAN ? q_to(0, s, fast) : 0.0);
         }
     }
 }
@@ -692,7 +878,15 @@ cudaError_t attrs_len_r()
 {
     cudaError_t e;
     const int sm = (int)smem_lines<L>();
-    if ((e = cudaFuncSetAttribute(rfft_kernel<R, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm))) return e;
+    if constexpr (L <= 512) {
+        if ((e = cudaFuncSetAttribute(rfft_kernel<R, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm))) return e;
+        if ((e = cudaFuncSetAttribute(rfft_q_kernel<L, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)QLineCfg<L, false>::SMEM)))
+            return e;
+        if ((e = cudaFuncSetAttribute(rfft_q_kernel<L, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)QLineCfg<L, true>::SMEM)))
+            return e;
+    }
     if ((e = cudaFuncSetAttribute(face_kernel<R, L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)smem_face<L>())))
         return e;
@@ -762,6 +956,21 @@ int face_blocks_per_sm(int L)
     })
 }
 
+namespace {
+template <int L, bool THIN>
+void launch_rfft_shape(const RfftPass &a, int nu, int nv, cudaStream_t st)
+{
+    using Cfg = QLineCfg<L, THIN>;
+    rfft_q_kernel<L, THIN><<<dim3((nv + Cfg::LB - 1) / Cfg::LB, nu), Cfg::T, Cfg::SMEM, st>>>(a);
+}
+template <int L>
+void launch_rfft_q(const RfftPass &a, int nu, int nv, cudaStream_t st)
+{
+    if ((int64_t)nu * nv >= (int64_t)152 * 4 * QLineCfg<L, false>::LB) launch_rfft_shape<L, false>(a, nu, nv, st);
+    else launch_rfft_shape<L, true>(a, nu, nv, st);
+}
+}  // namespace
+
 cudaError_t launch_rfft_pass(const RfftPass &a, cudaStream_t st)
 {
     int nu, nv;
@@ -769,10 +978,15 @@ cudaError_t launch_rfft_pass(const RfftPass &a, cudaStream_t st)
     else if (a.axis == 1) { nu = a.n0; nv = a.n2; }
     else { nu = a.n1; nv = a.n2; }
     IDP_LEN_SWITCH(a.P ? a.P : a.M, {
-        dim3 grid((nv + LineCfg<L>::LB - 1) / LineCfg<L>::LB, nu);
-        if (a.dd) rfft_kernel<ddr, L><<<grid, RfftThreads<ddr, L>::value, smem_lines<L>(), st>>>(a);
-        else rfft_kernel<double, L><<<grid, RfftThreads<double, L>::value, smem_lines<L>(), st>>>(a);
-        return cudaGetLastError();
+        if constexpr (L <= 512) {
+            dim3 grid((nv + LineCfg<L>::LB - 1) / LineCfg<L>::LB, nu);
+            if (a.fx) launch_rfft_q<L>(a, nu, nv, st);
+            else if (a.dd) rfft_kernel<ddr, L><<<grid, RfftThreads<ddr, L>::value, smem_lines<L>(), st>>>(a);
+            else rfft_kernel<double, L><<<grid, RfftThreads<double, L>::value, smem_lines<L>(), st>>>(a);
+            return cudaGetLastError();
+        } else {
+            return cudaErrorInvalidValue;
+        }
     })
 }
 

@@ -147,6 +147,8 @@ struct RfftPass {
     // its input, zero on entry: rows row2[i0 * n1 + i1] (every entry written),
     // row1[i0 * n2 + i2], slices sl0[i0], sl1[i1], sl2[i2] (set to 1 where non-zero)
     int *fl_row2, *fl_row1, *fl_sl0, *fl_sl1, *fl_sl2;
+    int fx;                // 1: fixed-point arithmetic (dd = 0), FP64 in and out
+    const int4 *q, *qhalf; // its tables for length P: FFT factors, e^{-i pi m/P}, m = 0..P/2
     double *copy;          // optional: the input is also copied here (same strides)
 };
 cudaError_t launch_rfft_pass(const RfftPass &a, cudaStream_t st);

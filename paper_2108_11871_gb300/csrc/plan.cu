@@ -204,6 +204,7 @@ struct idp_plan_s {
     std::map<int, DevFft> fft;        // by complex length
     std::map<int, ddr *> sin2d;       // by M: 2 sin(pi j / M), j = 0..M/2, double-float pairs
     std::map<int, int4 *> qdst;       // by M: fixed-point tables of the sine passes
+    std::map<int, int4 *> qfft;       // by length: fixed-point tables of the complex and real FFTs
     std::map<int, double *> sinm;     // by M (lengths without an FFT): sine matrices for direct sums
     std::map<int, ddr *> sinmd;       // double-float form
     int exact = 0;                    // created by idp_create_plan_exact
@@ -448,13 +449,45 @@ std::vector<int4> q_factors(int L, int RM)
     return q;
 }
 
+// uploads entries made by `fill` once per key
+template <class Fill>
+int cached_table(idp_plan p, std::map<int, int4 *> &cache, int key, Fill fill, const int4 **out)
+{
+    auto it = cache.find(key);
+    if (it == cache.end()) {
+        std::vector<int4> q;
+        fill(q);
+        int4 *d = nullptr;
+        int rc;
+        if ((rc = p->alloc(&d, (int64_t)q.size()))) return rc;
+        IDP_CK(cudaMemcpy(d, q.data(), sizeof(int4) * q.size(), cudaMemcpyHostToDevice));
+        it = cache.emplace(key, d).first;
+    }
+    *out = it->second;
+    return IDP_OK;
+}
+
+// fixed-point tables of a complex FFT of length L (radices up to 8) and, for the real
+// transforms, e^{-i pi m/L}, m = 0..L/2
+int get_fft_tables(idp_plan p, int L, const int4 **q, const int4 **qhalf)
+{
+    const int n = (int)q_factors(L, 8).size();
+    const int4 *d;
+    const int rc = cached_table(p, p->qfft, L, [&](std::vector<int4> &v) {
+        v = q_factors(L, 8);
+        for (int m = 0; m <= L / 2; ++m) v.push_back(fixed_unit(m, L));
+    }, &d);
+    *q = d;
+    *qhalf = d + n;
+    return rc;
+}
+
 // the tables of the sine passes of M panels: see DstPass
 int get_dst_tables(idp_plan p, int M, const int4 **out)
 {
-    auto it = p->qdst.find(M);
-    if (it == p->qdst.end()) {
+    return cached_table(p, p->qdst, M, [&](std::vector<int4> &q) {
         const int K = M / 2;
-        std::vector<int4> q = q_factors(K, dst_table_radix(K));
+        q = q_factors(K, dst_table_radix(K));
         for (int k = 0; k <= K / 2; ++k) q.push_back(fixed_unit(k, K));
         int2 sn[2];
         for (int j = 0; j < K; ++j) {
@@ -463,14 +496,7 @@ int get_dst_tables(idp_plan p, int M, const int4 **out)
             sn[j & 1] = fixed_factor(s);
             if (j & 1) q.push_back(make_int4(sn[0].x, sn[0].y, sn[1].x, sn[1].y));
         }
-        int4 *d = nullptr;
-        int rc;
-        if ((rc = p->alloc(&d, (int64_t)q.size()))) return rc;
-        IDP_CK(cudaMemcpy(d, q.data(), sizeof(int4) * q.size(), cudaMemcpyHostToDevice));
-        it = p->qdst.emplace(M, d).first;
-    }
-    *out = it->second;
-    return IDP_OK;
+    }, out);
 }
 
 // sine matrix S[i][e] = sin(pi (i+1)(e+1) / M), i, e < M - 1, e fastest, for the
@@ -590,6 +616,12 @@ int boundary_dd(idp_plan p)
 {
     return p->d == 3 && (p->mixed == IDP_PRECISION_DF32 || (tensor_mode(p) && p->mixed_bdd)) ? 1 : 0;
 }
+
+// the boundary in fixed point (else FP64 or double-float).  Not in the tensor-core modes: a
+// last-bit change of their FP64 intermediates flips FP32 roundings of the tensor-core
+// inputs, which moves single values of phi by up to 1e-7, within the modes' error of 1e-5
+// but not the same result
+int boundary_fx(idp_plan p) { return !tensor_mode(p) && !boundary_dd(p) ? 1 : 0; }
 
 // Pieces of S_{m,k} = sin(pi (m+1)(k+1)/M) for a tensor-core variant, laid out
 // as the kernel's shared-memory tiles, one contiguous block per (mode tile,
@@ -741,9 +773,8 @@ int transform(idp_plan p, View3 in, double *work, View3 out, const double *tab, 
         } else if ((rc = get_sinm(p, p->M[s], &a.sinm, dd ? 1 : 0))) {   // direct sums
             return rc;
         }
-        // the tensor-core modes keep double-float passes (their results are compared
-        // bit for bit where a rounding to FP32 follows); precision DF32 runs the
-        // fixed-point FFT, and double-float only in the direct sums
+        // the tensor-core modes keep double-float passes (boundary_fx says why); precision
+        // DF32 runs the fixed-point FFT, and double-float only in the direct sums
         a.in_dd = (q == 0) ? in_dd0 : 0;
         if (dd && (tensor_mode(p) || !has_fft_dst(p->M[s]))) {
             a.dd = 1;
@@ -872,6 +903,7 @@ int boundary(idp_plan p, const double *rho, double *dst0, double *dst1, cudaStre
     // double-float arithmetic for the 3-D convolutions in precision DF32 (and, on
     // request, in the tensor-core modes)
     const int dd = boundary_dd(p);
+    const int fx = boundary_fx(p);
     // support flags of rho: set by the first row transform
     IDP_CK(cudaMemsetAsync(p->flags, 0, sizeof(int) * p->nflags, st));
     // stage 1a: along axis 2 -> T0[i0][i1][m2]; stage 1b: along axis 1 -> T1[i0][i2][m1]
@@ -885,6 +917,8 @@ int boundary(idp_plan p, const double *rho, double *dst0, double *dst1, cudaStre
     a2.axis = 2; a2.M = p->M[2]; a2.P = p->P[2];
     if ((rc = get_fft(p, p->P[2], &t))) return rc;
     a2.t = t;
+    a2.fx = a1.fx = fx;
+    if ((rc = get_fft_tables(p, p->P[2], &a2.q, &a2.qhalf))) return rc;
     a2.dd = dd;
     // the pass along axis 2 reads every value of rho once: it also marks which
     // rows and slices are non-zero (zero ones are skipped below; their
@@ -898,6 +932,7 @@ int boundary(idp_plan p, const double *rho, double *dst0, double *dst1, cudaStre
     a1.axis = 1; a1.M = p->M[1]; a1.P = p->P[1];
     if ((rc = get_fft(p, p->P[1], &t))) return rc;
     a1.t = t;
+    if ((rc = get_fft_tables(p, p->P[1], &a1.q, &a1.qhalf))) return rc;
     a1.dd = dd;
     a1.lineflag = p->row1;
     {
@@ -1258,12 +1293,13 @@ int plan_setup(idp_plan p)
     for (int s = 0; s < 3; ++s) {
         if (!p->act[s]) continue;
         FftTables t;
-        const int4 *qt;
+        const int4 *qt, *qh;
         const ddr *sd;
         const void *sm_;
         if ((has_fft_dst(p->M[s]) && ((rc = get_fft(p, p->M[s] / 2, &t)) || (rc = get_dst_tables(p, p->M[s], &qt)) || (rc = get_sin2d(p, p->M[s], &sd)))) ||
             (!has_fft_dst(p->M[s]) && (rc = get_sinm(p, p->M[s], &sm_, 0))) ||
-            (rc = get_fft(p, p->P[s], &t)) || (rc = get_fft(p, 2 * p->P[s], &t)))
+            (rc = get_fft(p, p->P[s], &t)) || (rc = get_fft(p, 2 * p->P[s], &t)) ||
+            (rc = get_fft_tables(p, p->P[s], &qt, &qh)))
             return rc;
     }
     if (p->padded) {

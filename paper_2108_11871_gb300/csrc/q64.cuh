@@ -141,8 +141,9 @@ __host__ __device__ constexpr int q_tw_count(int L, int RM, int Ns = 1)
 }
 
 // One Stockham pass of radix R at span Ns over LB lines (line stride LS elements) by
-// NT threads; tw: the pass's factors w_{R Ns}^{k q}, [q - 1][k].
-template <int L, int Ns, int RM, int LB, int NT, int LS>
+// NT threads; tw: the pass's factors w_{R Ns}^{k q}, [q - 1][k].  HZ: the elements from
+// L / 2 on are zero and not read.
+template <int L, int Ns, int RM, int LB, int NT, int LS, bool HZ = false>
 __device__ __forceinline__ void q_pass(const qc *__restrict__ X, qc *__restrict__ Y, const int4 *__restrict__ tw)
 {
     constexpr int R = q_radix(L, Ns, RM), U = L / R;
@@ -152,7 +153,11 @@ __device__ __forceinline__ void q_pass(const qc *__restrict__ X, qc *__restrict_
         const qc *x = X + line * LS;
         qc v[R];
 #pragma unroll
-        for (int q = 0; q < R; ++q) v[q] = x[q_slot(j + q * U)];
+        for (int q = 0; q < R; ++q) {
+            if (HZ && q * U >= L / 2) v[q] = qc{0, 0};
+            else if (HZ && (q + 1) * U > L / 2) v[q] = j + q * U < L / 2 ? x[q_slot(j + q * U)] : qc{0, 0};
+            else v[q] = x[q_slot(j + q * U)];
+        }
         if constexpr (Ns > 1) {
 #pragma unroll
             for (int q = 1; q < R; ++q) v[q] = q_cmul(v[q], tw[(q - 1) * Ns + k]);
@@ -168,13 +173,13 @@ __device__ __forceinline__ void q_pass(const qc *__restrict__ X, qc *__restrict_
 // Forward FFT of LB lines of length L (a multiple of 8) in X, from span Ns on; Y is
 // scratch.  The result is in X if the number of passes is even, else in Y; ends
 // with a block barrier.  tw: the factors of the passes after span Ns, one after the
-// other (none for the first pass at Ns = 1).
-template <int L, int RM, int LB, int NT, int LS, int Ns = 1>
+// other (none for the first pass at Ns = 1).  HZ (first pass): see q_pass.
+template <int L, int RM, int LB, int NT, int LS, int Ns = 1, bool HZ = false>
 __device__ __forceinline__ void q_fft(qc *X, qc *Y, const int4 *__restrict__ tw)
 {
     if constexpr (Ns < L) {
         constexpr int R = q_radix(L, Ns, RM);
-        q_pass<L, Ns, RM, LB, NT, LS>(X, Y, tw);
+        q_pass<L, Ns, RM, LB, NT, LS, HZ>(X, Y, tw);
         __syncthreads();
         q_fft<L, RM, LB, NT, LS, Ns * R>(Y, X, tw + (Ns > 1 ? (R - 1) * Ns : 0));
     }
