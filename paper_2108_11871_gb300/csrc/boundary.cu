@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(QLineCfg<L, THIN>::T) rfft_q_kernel(const Rfft
     extern __shared__ qc smem_q[];
     qc *bufA = smem_q, *bufB = smem_q + Cfg::BUF;
     int4 *tws = reinterpret_cast<int4 *>(bufB + Cfg::BUF);
-    __shared__ int s_emax[LB], s_scale[LB], s_any;
+    __shared__ int s_emax[LB], s_scale[LB], s_any, s_gmax;
     __shared__ unsigned s_sum[LB];
     int nv;
     int64_t isu, isv, ise, osu, osv, ose;
@@ -319,6 +319,7 @@ __global__ void __launch_bounds__(QLineCfg<L, THIN>::T) rfft_q_kernel(const Rfft
         s_emax[threadIdx.x] = 1;
         s_sum[threadIdx.x] = 0;
     }
+    if (threadIdx.x == 0) s_gmax = 0;
     if (mk)
         for (int f = threadIdx.x; f < L + LB; f += NT) colnz[f] = 0;
     for (int f = threadIdx.x; f < Cfg::TW; f += NT) tws[f] = __ldg(a.q + f);
@@ -391,7 +392,9 @@ __global__ void __launch_bounds__(QLineCfg<L, THIN>::T) rfft_q_kernel(const Rfft
     const int bits = q_bits(s_sum[l]);
     if (threadIdx.x < LB) {
         const int e = s_emax[threadIdx.x];
-        s_scale[threadIdx.x] = e == 0x7ff ? Q_NAN : 1102 - e - q_bits(s_sum[threadIdx.x]);
+        const int eb = e + q_bits(s_sum[threadIdx.x]);
+        s_scale[threadIdx.x] = e == 0x7ff ? Q_NAN : 1102 - eb;
+        atomicMax(&s_gmax, e == 0x7ff ? Q_GNAN : eb);
     }
     // 3. into bufA viewed as reals: x_e at position e + 1 of the padded sequence (component
     //    1 of element e / 2 for even e), zeros elsewhere; the elements from L / 2 on are
@@ -407,6 +410,7 @@ __global__ void __launch_bounds__(QLineCfg<L, THIN>::T) rfft_q_kernel(const Rfft
         if (g == 0) zl[0] = 0;
     }
     __syncthreads();
+    if (a.gmax && threadIdx.x == 0 && *a.gmax < s_gmax) atomicMax(a.gmax, s_gmax);
     // 4. complex FFT of length L
     q_fft<L, Cfg::RM, LB, NT, LS, 1, true>(bufA, bufB, tws);
     const qc *Z = q_passes(L, Cfg::RM) % 2 == 0 ? bufA : bufB;
@@ -653,7 +657,9 @@ struct C2rCfg {
 template <int L>
 size_t smem_c2r() { return 2 * sizeof(double2) * C2rCfg<L>::LB * L; }
 
-template <class R, int L>
+// FX: the parts are the fixed-point sums of face.cu ([chunk][S, D][column][m]): the face is
+// S + D or S - D, added over the chunks in integers
+template <class R, int L, bool FX>
 __global__ void __launch_bounds__(NT) face_invb_kernel(const FaceInvB a)
 {
     using A = Ar<R>;
@@ -665,6 +671,25 @@ __global__ void __launch_bounds__(NT) face_invb_kernel(const FaceInvB a)
     const int c0 = blockIdx.x * TC;
     const int face = blockIdx.y;
     const int ncl = min(TC, a.nc - c0);
+    if constexpr (FX) {
+        const qc *part = reinterpret_cast<const qc *>(a.part);
+        const int g = *a.gmax, base = 1102 - g - a.lgn;
+        for (int f = threadIdx.x; f < TC * L; f += NT) {
+            const int t = f / L, m = f - t * L;
+            qc sum{0, 0}, dif{0, 0};
+            if (t < ncl)
+                for (int ch = 0; ch < a.nchunk; ++ch) {
+                    const qc *x = part + ((int64_t)ch * 2 * a.nc + c0 + t) * L + m;
+                    sum = q_add(sum, x[0]);
+                    dif = q_add(dif, x[(int64_t)a.nc * L]);
+                }
+            const qc v = face ? q_sub(sum, dif) : q_add(sum, dif);
+            const int ek = t < ncl ? a.ek[(int64_t)(c0 + t) * (L / 2 + 1) + (m <= L / 2 ? m : L - m)] : 0;
+            const int s = g >= Q_GNAN ? Q_NAN : base - ek;
+            const bool fast = q_fast(s);
+            bufA[t * L + m] = make_double2(q_to(v.re, s, fast), q_to(v.im, s, fast));
+        }
+    } else {
     const Cx *part = reinterpret_cast<const Cx *>(a.part);
     for (int f = threadIdx.x; f < TC * L; f += NT) {
         const int m = f / TC, t = f - m * TC;
@@ -677,6 +702,7 @@ __global__ void __launch_bounds__(NT) face_invb_kernel(const FaceInvB a)
             }
         }
         bufA[t * L + m] = A::cmake(sr, si);
+    }
     }
     __syncthreads();
     const Cx *Z = cta_fft_t<R, L, TC, NT, true>(bufA, bufB, inv_tw<R>(a.t), false);
@@ -890,7 +916,10 @@ cudaError_t attrs_len_r()
     if ((e = cudaFuncSetAttribute(face_kernel<R, L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)smem_face<L>())))
         return e;
-    if ((e = cudaFuncSetAttribute(face_invb_kernel<R, L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if ((e = cudaFuncSetAttribute(face_invb_kernel<R, L, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)smem_invb<L>())))
+        return e;
+    if ((e = cudaFuncSetAttribute(face_invb_kernel<double, L, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)smem_invb<L>())))
         return e;
     return cudaFuncSetAttribute(face_c2r_kernel<R, L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -926,6 +955,7 @@ cudaError_t attrs_len()
 cudaError_t boundary_set_attributes()
 {
     cudaError_t e;
+    if ((e = face_q_set_attributes())) return e;
     if ((e = attrs_len<16>())) return e;
     if ((e = attrs_len<32>())) return e;
     if ((e = attrs_len<48>())) return e;
@@ -1010,8 +1040,9 @@ cudaError_t launch_face_inv_b(const FaceInvB &a, cudaStream_t st)
 {
     IDP_LEN_SWITCH(2 * (a.Pb ? a.Pb : a.Mb), {
         dim3 grid((a.nc + InvbCfg<L>::TC - 1) / InvbCfg<L>::TC, 2);
-        if (a.dd) face_invb_kernel<ddr, L><<<grid, NT, smem_invb<L>(), st>>>(a);
-        else face_invb_kernel<double, L><<<grid, NT, smem_invb<L>(), st>>>(a);
+        if (a.fx) face_invb_kernel<double, L, true><<<grid, NT, smem_invb<L>(), st>>>(a);
+        else if (a.dd) face_invb_kernel<ddr, L, false><<<grid, NT, smem_invb<L>(), st>>>(a);
+        else face_invb_kernel<double, L, false><<<grid, NT, smem_invb<L>(), st>>>(a);
         return cudaGetLastError();
     })
 }

@@ -149,6 +149,7 @@ struct RfftPass {
     int *fl_row2, *fl_row1, *fl_sl0, *fl_sl1, *fl_sl2;
     int fx;                // 1: fixed-point arithmetic (dd = 0), FP64 in and out
     const int4 *q, *qhalf; // its tables for length P: FFT factors, e^{-i pi m/P}, m = 0..P/2
+    int *gmax;             // optional (fx): maximum over the lines of emax + bits (q64.cuh), zero on entry
     double *copy;          // optional: the input is also copied here (same strides)
 };
 cudaError_t launch_rfft_pass(const RfftPass &a, cudaStream_t st);
@@ -175,6 +176,26 @@ cudaError_t launch_face_pass(const FacePass &a, int nchunk, cudaStream_t st);
 int face_columns_per_block(int L);   // frequencies c per block of the face pass
 int face_blocks_per_sm(int L);       // resident blocks per SM of the face pass
 
+// Stage 2 in fixed point (face.cu): sums over the pairs of slices p and np - 1 - p.
+struct qc;
+struct FaceQPass {
+    const double2 *D;          // as FacePass
+    int64_t sp, sb, sc;
+    int np, Mb, Pb, nc;
+    int lgn;                   // ceil(log2(Mb))
+    const int2 *kq;            // [2][(np+1)/2][nc][Pb+1]: (k_p + k_p') / 2 and (k_p - k_p') / 2 as fractions of
+                               // 2^ek[c][b]: (bits 62..31, bits 30..0) of the value times 2^(62 - ek)
+    qc *part;                  // [nchunk][2][nc][2Pb]
+    int nchunk;                // chunk i takes the pairs i, i + nchunk, ...
+    const int4 *q;             // FFT factors of length 2Pb
+    const int *sliceflag;      // sliceflag[p] != 0 iff slice p has a non-zero value
+    const int *gmax;           // maximum over the lines of D of emax + bits
+};
+cudaError_t launch_face_q(const FaceQPass &a, cudaStream_t st);
+cudaError_t launch_face_kq(const double *khat, int np, int64_t per, int2 *kq, int *ek, cudaStream_t st);
+cudaError_t face_q_set_attributes();
+int face_q_columns(int L);   // frequencies c per block
+
 // 2-D contraction: part[0/1][m] = sum_p khat[p or np-1-p][m] * T[p][m]
 struct FacePass2D {
     const double2 *T; int64_t sp, sm;
@@ -193,6 +214,9 @@ struct FaceInvB {
     FftTables t;               // length 2Pb
     int dd;
     int Pb;                    // 0: Mb
+    int fx, lgn;               // 1: parts of FaceQPass, its lgn and ek[nc][Pb+1]
+    const int *ek;
+    const int *gmax;
 };
 cudaError_t launch_face_inv_b(const FaceInvB &a, cudaStream_t st);
 

@@ -229,6 +229,10 @@ struct idp_plan_s {
     double *khat[3] = {nullptr, nullptr, nullptr};
     ddr *khatd[3] = {nullptr, nullptr, nullptr};   // double-float copies (precision DF32)
     int64_t khat_n[3] = {0, 0, 0};
+    int2 *kq[3] = {nullptr, nullptr, nullptr};   // fixed-point spectra (FaceQPass) and their exponents
+    int *kq_ek[3] = {nullptr, nullptr, nullptr};
+    int qchunk[3] = {1, 1, 1};        // chunks of pairs of slices of the fixed-point face passes
+    int *gmax[2] = {nullptr, nullptr};   // bounds of the lines along axes 2 and 1 (FaceQPass::gmax)
     int nchunk[3] = {1, 1, 1}, pchunk[3] = {1, 1, 1};
     int dst_lines = 0;                // lines per block of the full-volume sine passes (0 = default)
 
@@ -610,11 +614,11 @@ bool tensor_mode(idp_plan p)
 {
     return p->mixed == IDP_PRECISION_MIXED_BF16X3 || p->mixed == IDP_PRECISION_MIXED_TF32X3;
 }
-// the 3-D boundary convolutions (and so T0) in double-float arithmetic: precision
-// DF32, or a tensor-core mode with IDP_KEY_MIXED_BOUNDARY_DF32
+// the 3-D boundary convolutions (and so T0) in double-float arithmetic: a tensor-core
+// mode with IDP_KEY_MIXED_BOUNDARY_DF32
 int boundary_dd(idp_plan p)
 {
-    return p->d == 3 && (p->mixed == IDP_PRECISION_DF32 || (tensor_mode(p) && p->mixed_bdd)) ? 1 : 0;
+    return p->d == 3 && tensor_mode(p) && p->mixed_bdd ? 1 : 0;
 }
 
 // the boundary in fixed point (else FP64 or double-float).  Not in the tensor-core modes: a
@@ -889,21 +893,59 @@ int transform_rho_from_T0(idp_plan p, cudaStream_t st)
     return transform(p, im, p->A, dense(p, p->A), p->tabc2, none, true, st, true, true, dd);
 }
 
+int ceil_log2(int n)
+{
+    int e = 0;
+    while ((1 << e) < n) ++e;
+    return e;
+}
+
+// about n chunks of the np slices of a face pass, no more than pairs: ceil(np / slices per chunk)
+int face_q_chunks(int np, int n)
+{
+    n = std::max(1, std::min(n, (np + 1) / 2));
+    const int per = (np + n - 1) / n;
+    return (np + per - 1) / per;
+}
+
+// the fixed-point face pass of axis a_ into `part`, and what the inverse transform of
+// its parts needs
+int face_q_pass(idp_plan p, int a_, int nchunk, double2 *part, FaceQPass *q, FaceInvB *ib)
+{
+    const int b = a_ == 0 ? 1 : 0, c = a_ == 2 ? 1 : 2;
+    const int64_t r2 = p->P[2] + 1, r1 = p->P[1] + 1;
+    q->D = a_ == 2 ? p->T1 : p->T0;
+    q->sp = a_ == 0 ? p->ni[1] * r2 : a_ == 1 ? r2 : r1;
+    q->sb = a_ == 0 ? r2 : a_ == 1 ? p->ni[1] * r2 : p->ni[2] * r1;
+    q->sc = 1;
+    q->np = p->ni[a_]; q->Mb = p->M[b]; q->Pb = p->P[b]; q->nc = p->P[c] + 1;
+    q->lgn = ceil_log2(p->M[b]);
+    q->kq = p->kq[a_];
+    q->part = reinterpret_cast<qc *>(part);
+    q->nchunk = nchunk;
+    q->sliceflag = p->sl[a_];
+    q->gmax = p->gmax[a_ == 2 ? 1 : 0];
+    ib->fx = 1; ib->nchunk = nchunk; ib->lgn = q->lgn; ib->ek = p->kq_ek[a_]; ib->gmax = q->gmax;
+    const int4 *half;
+    return get_fft_tables(p, 2 * p->P[b], &q->q, &half);
+}
+
 // boundary values g into the boundary nodes of dst0 (and dst1 if not null).
 // rho_src (optional): the node array that the first row transform reads instead
 // of rho, copying its interior into rho for the later stages (a page-locked host
-// buffer, through its device view: the upload then runs inside that pass)
+// buffer, through its device view: the upload then runs inside that pass).
+// stage: g is the output itself: a tensor-core mode with FP64 boundary then gives the
+// values of an FP64 plan
 int boundary(idp_plan p, const double *rho, double *dst0, double *dst1, cudaStream_t st,
-             bool fork_rho = false, const double *rho_src = nullptr)
+             bool fork_rho = false, const double *rho_src = nullptr, bool stage = false)
 {
     Range rg(p, "idp:boundary values g");
     const View3 r = node_interior(p, rho);
     int rc;
     FftTables t;
-    // double-float arithmetic for the 3-D convolutions in precision DF32 (and, on
-    // request, in the tensor-core modes)
+    // double-float arithmetic for the 3-D convolutions, on request, in the tensor-core modes
     const int dd = boundary_dd(p);
-    const int fx = boundary_fx(p);
+    const int fx = stage ? !dd : boundary_fx(p);
     // support flags of rho: set by the first row transform
     IDP_CK(cudaMemsetAsync(p->flags, 0, sizeof(int) * p->nflags, st));
     // stage 1a: along axis 2 -> T0[i0][i1][m2]; stage 1b: along axis 1 -> T1[i0][i2][m1]
@@ -918,6 +960,8 @@ int boundary(idp_plan p, const double *rho, double *dst0, double *dst1, cudaStre
     if ((rc = get_fft(p, p->P[2], &t))) return rc;
     a2.t = t;
     a2.fx = a1.fx = fx;
+    a2.gmax = p->gmax[0];
+    a1.gmax = p->gmax[1];
     if ((rc = get_fft_tables(p, p->P[2], &a2.q, &a2.qhalf))) return rc;
     a2.dd = dd;
     // the pass along axis 2 reads every value of rho once: it also marks which
@@ -1007,12 +1051,18 @@ int boundary(idp_plan p, const double *rho, double *dst0, double *dst1, cudaStre
         f.dd = dd;
         f.khatd = p->khatd[a_];
         f.sliceflag = p->sl[a_];
-        {
-            Mark mk(p, IDP_KERNEL_FACE, sa);
-            IDP_CK(launch_face_pass(f, p->nchunk[a_], sa));
-        }
         FaceInvB ib{};
         ib.part = part; ib.nchunk = p->nchunk[a_];
+        {
+            Mark mk(p, IDP_KERNEL_FACE, sa);
+            if (fx) {
+                FaceQPass q{};
+                if ((rc = face_q_pass(p, a_, p->qchunk[a_], part, &q, &ib))) return rc;
+                IDP_CK(launch_face_q(q, sa));
+            } else {
+                IDP_CK(launch_face_pass(f, p->nchunk[a_], sa));
+            }
+        }
         ib.Mb = p->M[b]; ib.Pb = p->P[b]; ib.nc = f.nc; ib.out = F; ib.t = t;
         ib.dd = dd;
         {
@@ -1137,7 +1187,7 @@ int enqueue_grid(idp_plan p, const double *rho, double *phi, int stop, cudaStrea
     const size_t node_bytes = sizeof(double) * p->nodes;
     if (stop == IDP_STAGE_BOUNDARY) {
         IDP_CK(cudaMemsetAsync(phi, 0, node_bytes, st));
-        return boundary(p, rho, phi, nullptr, st);
+        return boundary(p, rho, phi, nullptr, st, false, nullptr, true);
     }
     if (stop == IDP_STAGE_PHISTAR) {
         IDP_CK(cudaMemsetAsync(phi, 0, node_bytes, st));
@@ -1299,7 +1349,7 @@ int plan_setup(idp_plan p)
         if ((has_fft_dst(p->M[s]) && ((rc = get_fft(p, p->M[s] / 2, &t)) || (rc = get_dst_tables(p, p->M[s], &qt)) || (rc = get_sin2d(p, p->M[s], &sd)))) ||
             (!has_fft_dst(p->M[s]) && (rc = get_sinm(p, p->M[s], &sm_, 0))) ||
             (rc = get_fft(p, p->P[s], &t)) || (rc = get_fft(p, 2 * p->P[s], &t)) ||
-            (rc = get_fft_tables(p, p->P[s], &qt, &qh)))
+            (rc = get_fft_tables(p, p->P[s], &qt, &qh)) || (rc = get_fft_tables(p, 2 * p->P[s], &qt, &qh)))
             return rc;
     }
     if (p->padded) {
@@ -1325,13 +1375,15 @@ int plan_setup(idp_plan p)
     }
     {
         const int64_t n0 = p->ni[0], n1 = p->ni[1], n2 = p->ni[2];
-        p->nflags = n0 * n1 + n0 * n2 + n0 + n1 + n2;
+        p->nflags = n0 * n1 + n0 * n2 + n0 + n1 + n2 + 2;
         if ((rc = p->alloc(&p->flags, p->nflags))) return rc;
         p->row2 = p->flags;
         p->row1 = p->row2 + n0 * n1;
         p->sl[0] = p->row1 + n0 * n2;
         p->sl[1] = p->sl[0] + n0;
         p->sl[2] = p->sl[1] + n1;
+        p->gmax[0] = p->sl[2] + n2;
+        p->gmax[1] = p->gmax[0] + 1;
     }
     if ((rc = plan_streams(p))) return rc;
     {
@@ -1437,6 +1489,11 @@ int plan_setup(idp_plan p)
             p->nchunk[a_] = nch;
             p->pchunk[a_] = pch;
             pmax = std::max<int64_t>(pmax, (int64_t)nch * 2 * L * (Mc + 1));
+            const int npair = (np + 1) / 2;
+            // one wave of two blocks per SM, and at most 64 pairs per block
+            const int qtiles = 2 * ((Mc + face_q_columns(L)) / face_q_columns(L));
+            p->qchunk[a_] = face_q_chunks(np, std::max(2 * nsm / qtiles, npair / 64));
+            pmax = std::max<int64_t>(pmax, (int64_t)p->qchunk[a_] * 2 * L * (Mc + 1));
             fmax = std::max<int64_t>(fmax, (int64_t)2 * (Mb + 1) * (Mc + 1));
             const int64_t per = (int64_t)(Mb + 1) * (Mc + 1);
             if ((rc = p->alloc(&p->khat[a_], (int64_t)np * per))) return rc;
@@ -1472,6 +1529,9 @@ int plan_setup(idp_plan p)
                 IDP_CK(launch_gemm_batched(Mc + 1, Mb + 1, Mb + 1, yb, Mb + 1, per, tbb, Mb + 1, 0,
                                            p->khat[a_] + (int64_t)p0 * per, Mb + 1, per, cnt, 0));
             }
+            // fixed-point spectra
+            if ((rc = p->alloc(&p->kq[a_], 2 * (int64_t)npair * per)) || (rc = p->alloc(&p->kq_ek[a_], per))) return rc;
+            IDP_CK(launch_face_kq(p->khat[a_], np, per, p->kq[a_], p->kq_ek[a_], 0));
         }
         if ((rc = p->alloc(&p->part, 3 * pmax)) || (rc = p->alloc(&p->F, 3 * fmax))) return rc;
         p->part_cap = pmax;
@@ -1509,7 +1569,45 @@ int autotune(idp_plan p)
         }
         return best;
     };
-    if (p->d == 3) {
+    if (boundary_fx(p) && p->d == 3) {
+        // chunk counts of the fixed-point face passes: around the set-up's choice and the
+        // counts that fill whole waves of resident blocks; timed with every slice, and with the
+        // sum of the parts that follows
+        IDP_CK(cudaMemsetAsync(p->flags, 1, sizeof(int) * p->nflags, st));
+        for (int a_ = 0; a_ < 3 && !rc; ++a_) {
+            const int b = a_ == 0 ? 1 : 0, c = a_ == 2 ? 1 : 2;
+            const int L = 2 * p->P[b], nc = p->P[c] + 1, n0 = p->qchunk[a_];
+            int nsm = 152;
+            cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, p->dev);
+            const int tiles = 2 * ((nc + face_q_columns(L) - 1) / face_q_columns(L));
+            std::vector<int> cands = {n0, face_q_chunks(p->ni[a_], n0 / 2), face_q_chunks(p->ni[a_], 2 * n0)};
+            for (int w = 1; w <= 6; ++w) cands.push_back(face_q_chunks(p->ni[a_], w * 2 * nsm / tiles));
+            float best_t = 1e30f;
+            for (size_t i = 0; i < cands.size() && !rc; ++i) {
+                if (std::find(cands.begin(), cands.begin() + i, cands[i]) != cands.begin() + i) continue;
+                const int64_t need = (int64_t)cands[i] * 2 * L * nc;
+                if (need > p->part_cap) {
+                    double2 *np_part;
+                    if ((rc = p->alloc(&np_part, 3 * need))) break;
+                    p->part = np_part;
+                    p->part_cap = need;
+                }
+                FaceQPass f{};
+                FaceInvB ib{};
+                if ((rc = face_q_pass(p, a_, cands[i], p->part, &f, &ib))) break;
+                FftTables t;
+                if ((rc = get_fft(p, L, &t))) break;
+                ib.part = p->part; ib.Mb = p->M[b]; ib.Pb = p->P[b]; ib.nc = nc; ib.out = p->F; ib.t = t;
+                const float ms = timed([&]() -> int {
+                    cudaError_t e = launch_face_q(f, st);
+                    if (e == cudaSuccess) e = launch_face_inv_b(ib, st);
+                    return e == cudaSuccess ? IDP_OK : cuda_fail(e, "face pass (autotune)");
+                });
+                if (ms < best_t) { best_t = ms; p->qchunk[a_] = cands[i]; }
+            }
+        }
+    }
+    if (!boundary_fx(p) && p->d == 3) {
         for (int a_ = 0; a_ < 3 && !rc; ++a_) {
             const int b = a_ == 0 ? 1 : 0, c = a_ == 2 ? 1 : 2;
             const int np = p->ni[a_], L = 2 * p->P[b], nc = p->P[c] + 1;
@@ -1890,14 +1988,6 @@ int idp_plan_set(idp_plan p, int key, int64_t value)
                     return rc;
             }
         }
-        if (value == IDP_PRECISION_DF32 && p->d == 3 && !p->khatd[0]) {
-            int rc;
-            for (int a_ = 0; a_ < 3; ++a_) {
-                if ((rc = p->alloc(&p->khatd[a_], p->khat_n[a_]))) return rc;
-                IDP_CK(launch_to_dd(p->khat[a_], p->khatd[a_], p->khat_n[a_], 0));
-            }
-            IDP_CK(cudaDeviceSynchronize());
-        }
         if (p->mixed != (int)value) {
             p->mixed = (int)value;
             p->mixed_path = 0;
@@ -2182,8 +2272,9 @@ int idp_plan_tuning(idp_plan p, int64_t out[9])
     out[0] = p->tuned;
     out[1] = p->mixed_path;
     for (int a = 0; a < 3; ++a) {
-        out[2 + a] = p->nchunk[a];
-        out[5 + a] = p->pchunk[a];
+        const bool fx = boundary_fx(p) && p->d == 3;
+        out[2 + a] = fx ? p->qchunk[a] : p->nchunk[a];
+        out[5 + a] = fx ? (p->ni[a] + p->qchunk[a] - 1) / p->qchunk[a] : p->pchunk[a];
     }
     out[8] = p->dst_lines;
     return IDP_OK;

@@ -211,6 +211,7 @@ __device__ __forceinline__ long long q_from(double x, int shift)   // shift = em
     return (v ^ s) - s;
 }
 constexpr int Q_NAN = 1 << 30;   // scale of a line with a NaN or an infinity
+constexpr int Q_GNAN = 1 << 20;  // emax + bits of such a line in a maximum over lines
 // v 2^-s as FP64; fast: 2^-s and every |v| keep the result normal
 __device__ __forceinline__ bool q_fast(int s) { return s <= 1022 && s >= -960; }
 __device__ __forceinline__ double q_to(long long v, int s, bool fast)
