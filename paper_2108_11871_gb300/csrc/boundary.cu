@@ -638,6 +638,39 @@ __global__ void face2d_kernel(const FacePass2D a)
     a.acc[a.nm + m] = hi;
 }
 
+// The same with the slices split over the FG groups of a block (32 frequencies each) and the
+// groups' sums added in order: one thread per frequency leaves a serial chain of np steps
+// on a few warps (513 x 385: 143 and 109 us per face, 22 and 19 us split, launch included).
+constexpr int FG = 16;
+__global__ void __launch_bounds__(32 * FG) face2d_split_kernel(const FacePass2D a)
+{
+    __shared__ double2 s_lo[FG][32], s_hi[FG][32];
+    const int t = threadIdx.x & 31, g = threadIdx.x >> 5;
+    const int m = blockIdx.x * 32 + t;
+    double2 lo = make_double2(0.0, 0.0), hi = make_double2(0.0, 0.0);
+    if (m < a.nm) {
+#pragma unroll 4
+        for (int p = g; p < a.np; p += FG) {
+            const double2 x = a.T[(int64_t)p * a.sp + (int64_t)m * a.sm];
+            const double kl = a.khat[(int64_t)p * a.nm + m];
+            const double kh = a.khat[(int64_t)(a.np - 1 - p) * a.nm + m];
+            lo.x = fma(kl, x.x, lo.x); lo.y = fma(kl, x.y, lo.y);
+            hi.x = fma(kh, x.x, hi.x); hi.y = fma(kh, x.y, hi.y);
+        }
+    }
+    s_lo[g][t] = lo;
+    s_hi[g][t] = hi;
+    __syncthreads();
+    // warps 0 and 1: the sums of lo and hi
+    if (g < 2 && m < a.nm) {
+        const double2(*s)[32] = g ? s_hi : s_lo;
+        double2 v = s[0][t];
+#pragma unroll
+        for (int i = 1; i < FG; ++i) v = make_double2(v.x + s[i][t].x, v.y + s[i][t].y);
+        a.acc[(int64_t)g * a.nm + m] = v;
+    }
+}
+
 // ---------------------------------------------------------------- stage 3a
 // columns per block of face_invb: its cost is the FP64 sum of the slice-chunk
 // partials, one value per thread (one column of 256 values at M = 128)
@@ -1032,7 +1065,8 @@ cudaError_t launch_face_pass(const FacePass &a, int nchunk, cudaStream_t st)
 
 cudaError_t launch_face_pass_2d(const FacePass2D &a, cudaStream_t st)
 {
-    face2d_kernel<<<(a.nm + 127) / 128, 128, 0, st>>>(a);
+    if (a.split) face2d_split_kernel<<<(a.nm + 31) / 32, 32 * FG, 0, st>>>(a);
+    else face2d_kernel<<<(a.nm + 127) / 128, 128, 0, st>>>(a);
     return cudaGetLastError();
 }
 

@@ -335,12 +335,8 @@ cudaError_t launch_dst_pass(const DstPass &a, cudaStream_t st)
     IDP_DST_SWITCH(a.M, launch_k<K>(a, st), launch_dst_dd(a, st))
 }
 
-bool q_supported(int L)
-{
-    int m = L % 3 ? L : L / 3;
-    return m >= 8 && (m & (m - 1)) == 0;
-}
 int q_table_radix(int L, int Ns, int RM) { return q_radix(L, Ns, RM); }
+int q_table_count(int L, int RM) { return q_tw_count(L, RM); }
 int dst_table_radix(int K) { return dst_radix(K); }
 
 }  // namespace idp

@@ -97,8 +97,8 @@ cudaError_t launch_dst_pass(const DstPass &a, cudaStream_t st);
 cudaError_t dst_set_attributes();
 cudaError_t launch_dst_dd(const DstPass &a, cudaStream_t st);
 cudaError_t dst_dd_set_attributes();
-bool q_supported(int L);                    // lengths with a fixed-point FFT (q64.cuh)
-int q_table_radix(int L, int Ns, int RM);   // the radix of its pass after span Ns
+int q_table_radix(int L, int Ns, int RM);   // fixed-point FFT of length L (q64.cuh): radix of the pass after Ns,
+int q_table_count(int L, int RM);           // entries of its factor table
 int dst_table_radix(int K);                 // RM of the sine passes' FFT of length K
 cudaError_t boundary_set_attributes();
 
@@ -202,6 +202,7 @@ struct FacePass2D {
     int np, nm;
     const double *khat;        // [np][nm]
     double2 *acc;              // [2][nm]
+    int split;                 // 1: the sum over p split within a block
 };
 cudaError_t launch_face_pass_2d(const FacePass2D &a, cudaStream_t st);
 

@@ -148,6 +148,23 @@ int4 fixed_unit(int64_t m, int64_t L)      // e^{-i pi m / L}
     return make_int4(x.x, x.y, y.x, y.y);
 }
 
+// Host copies of the tables, which depend on the kind and the length alone: made once per
+// process (the long-double sines cost milliseconds on Arm), at most one per supported length
+std::mutex g_table_mu;
+std::map<std::pair<int, int>, std::vector<char>> g_tables;
+template <class Fill>
+const std::vector<char> &host_table(int kind, int key, Fill fill)
+{
+    std::lock_guard<std::mutex> lk(g_table_mu);
+    auto it = g_tables.find({kind, key});
+    if (it == g_tables.end()) {
+        std::vector<char> v;
+        fill(v);
+        it = g_tables.emplace(std::make_pair(kind, key), std::move(v)).first;
+    }
+    return it->second;   // entries are never changed or removed
+}
+
 std::mutex g_attr_mu;
 std::atomic<uint64_t> g_serial{1};
 std::vector<int> g_attr_done;
@@ -203,8 +220,7 @@ struct idp_plan_s {
 
     std::map<int, DevFft> fft;        // by complex length
     std::map<int, ddr *> sin2d;       // by M: 2 sin(pi j / M), j = 0..M/2, double-float pairs
-    std::map<int, int4 *> qdst;       // by M: fixed-point tables of the sine passes
-    std::map<int, int4 *> qfft;       // by length: fixed-point tables of the complex and real FFTs
+    std::map<std::pair<int, int>, int4 *> qtab;   // fixed-point tables by kind (FFTs, sine passes) and length
     std::map<int, double *> sinm;     // by M (lengths without an FFT): sine matrices for direct sums
     std::map<int, ddr *> sinmd;       // double-float form
     int exact = 0;                    // created by idp_create_plan_exact
@@ -382,41 +398,45 @@ int get_fft(idp_plan p, int L, FftTables *out)
         *out = it->second.view(L);
         return IDP_OK;
     }
-    DevFft t;
-    std::vector<Tw> fw(L / 2), iv(L / 2);
-    for (int j = 0; j < L / 2; ++j) {
-        const double c = cospi_frac(2 * j, L), s = sinpi_frac(2 * j, L);
-        fw[j] = make_tw(c, -s);
-        iv[j] = make_tw(c, s);
-    }
-    std::vector<double2> hf(L + 1);
-    std::vector<Tw> hr(L + 1);
-    for (int k = 0; k <= L; ++k) {
-        hf[k] = make_double2(cospi_frac(k, L), -sinpi_frac(k, L));
-        hr[k] = make_tw(hf[k].x, hf[k].y);
-    }
-    std::vector<TwD> fwd2(L / 2), ivd2(L / 2);
-    std::vector<ddc> hfd(L + 1);
-    for (int j = 0; j < L / 2; ++j) {
-        fwd2[j] = make_twd(fw[j]);
-        ivd2[j] = make_twd(iv[j]);
-    }
-    for (int k = 0; k <= L; ++k) {
-        hfd[k].re = host_dd(hf[k].x);
-        hfd[k].im = host_dd(hf[k].y);
-    }
+    // one upload of all tables, made once per process
+    const size_t h = L / 2, f = L + 1;
+    const size_t size[7] = {h * sizeof(Tw), h * sizeof(Tw), f * sizeof(double2), f * sizeof(Tw),
+                            h * sizeof(TwD), h * sizeof(TwD), f * sizeof(ddc)};
+    size_t off[8] = {0};
+    for (int i = 0; i < 7; ++i) off[i + 1] = (off[i] + size[i] + 31) / 32 * 32;
+    const std::vector<char> &blob = host_table(0, L, [&](std::vector<char> &v) {
+        v.resize(off[7]);
+        Tw *fw = reinterpret_cast<Tw *>(v.data() + off[0]), *iv = reinterpret_cast<Tw *>(v.data() + off[1]);
+        double2 *hf = reinterpret_cast<double2 *>(v.data() + off[2]);
+        Tw *hr = reinterpret_cast<Tw *>(v.data() + off[3]);
+        TwD *fwd2 = reinterpret_cast<TwD *>(v.data() + off[4]), *ivd2 = reinterpret_cast<TwD *>(v.data() + off[5]);
+        ddc *hfd = reinterpret_cast<ddc *>(v.data() + off[6]);
+        for (int j = 0; j < L / 2; ++j) {
+            const double c = cospi_frac(2 * j, L), s = sinpi_frac(2 * j, L);
+            fw[j] = make_tw(c, -s);
+            iv[j] = make_tw(c, s);
+            fwd2[j] = make_twd(fw[j]);
+            ivd2[j] = make_twd(iv[j]);
+        }
+        for (int k = 0; k <= L; ++k) {
+            hf[k] = make_double2(cospi_frac(k, L), -sinpi_frac(k, L));
+            hr[k] = make_tw(hf[k].x, hf[k].y);
+            hfd[k].re = host_dd(hf[k].x);
+            hfd[k].im = host_dd(hf[k].y);
+        }
+    });
+    char *d = nullptr;
     int rc;
-    if ((rc = p->alloc(&t.fwd, L / 2)) || (rc = p->alloc(&t.inv, L / 2)) || (rc = p->alloc(&t.half, L + 1)) ||
-        (rc = p->alloc(&t.halfr, L + 1)) ||
-        (rc = p->alloc(&t.fwdd, L / 2)) || (rc = p->alloc(&t.invd, L / 2)) || (rc = p->alloc(&t.halfd, L + 1)))
-        return rc;
-    IDP_CK(cudaMemcpy(t.fwd, fw.data(), sizeof(Tw) * (L / 2), cudaMemcpyHostToDevice));
-    IDP_CK(cudaMemcpy(t.inv, iv.data(), sizeof(Tw) * (L / 2), cudaMemcpyHostToDevice));
-    IDP_CK(cudaMemcpy(t.half, hf.data(), sizeof(double2) * (L + 1), cudaMemcpyHostToDevice));
-    IDP_CK(cudaMemcpy(t.halfr, hr.data(), sizeof(Tw) * (L + 1), cudaMemcpyHostToDevice));
-    IDP_CK(cudaMemcpy(t.fwdd, fwd2.data(), sizeof(TwD) * (L / 2), cudaMemcpyHostToDevice));
-    IDP_CK(cudaMemcpy(t.invd, ivd2.data(), sizeof(TwD) * (L / 2), cudaMemcpyHostToDevice));
-    IDP_CK(cudaMemcpy(t.halfd, hfd.data(), sizeof(ddc) * (L + 1), cudaMemcpyHostToDevice));
+    if ((rc = p->alloc(&d, (int64_t)blob.size()))) return rc;
+    IDP_CK(cudaMemcpy(d, blob.data(), blob.size(), cudaMemcpyHostToDevice));
+    DevFft t;
+    t.fwd = reinterpret_cast<Tw *>(d + off[0]);
+    t.inv = reinterpret_cast<Tw *>(d + off[1]);
+    t.half = reinterpret_cast<double2 *>(d + off[2]);
+    t.halfr = reinterpret_cast<Tw *>(d + off[3]);
+    t.fwdd = reinterpret_cast<TwD *>(d + off[4]);
+    t.invd = reinterpret_cast<TwD *>(d + off[5]);
+    t.halfd = reinterpret_cast<ddc *>(d + off[6]);
     p->fft[L] = t;
     *out = t.view(L);
     return IDP_OK;
@@ -453,19 +473,23 @@ std::vector<int4> q_factors(int L, int RM)
     return q;
 }
 
-// uploads entries made by `fill` once per key
+// uploads a table once per plan
 template <class Fill>
-int cached_table(idp_plan p, std::map<int, int4 *> &cache, int key, Fill fill, const int4 **out)
+int cached_table(idp_plan p, int kind, int key, Fill fill, const int4 **out)
 {
-    auto it = cache.find(key);
-    if (it == cache.end()) {
-        std::vector<int4> q;
-        fill(q);
-        int4 *d = nullptr;
+    auto it = p->qtab.find({kind, key});
+    if (it == p->qtab.end()) {
+        const std::vector<char> &t = host_table(kind, key, [&](std::vector<char> &v) {
+            std::vector<int4> q;
+            fill(q);
+            v.resize(sizeof(int4) * q.size());
+            std::memcpy(v.data(), q.data(), v.size());
+        });
+        char *d = nullptr;
         int rc;
-        if ((rc = p->alloc(&d, (int64_t)q.size()))) return rc;
-        IDP_CK(cudaMemcpy(d, q.data(), sizeof(int4) * q.size(), cudaMemcpyHostToDevice));
-        it = cache.emplace(key, d).first;
+        if ((rc = p->alloc(&d, (int64_t)t.size()))) return rc;
+        IDP_CK(cudaMemcpy(d, t.data(), t.size(), cudaMemcpyHostToDevice));
+        it = p->qtab.emplace(std::make_pair(kind, key), reinterpret_cast<int4 *>(d)).first;
     }
     *out = it->second;
     return IDP_OK;
@@ -475,21 +499,18 @@ int cached_table(idp_plan p, std::map<int, int4 *> &cache, int key, Fill fill, c
 // transforms, e^{-i pi m/L}, m = 0..L/2
 int get_fft_tables(idp_plan p, int L, const int4 **q, const int4 **qhalf)
 {
-    const int n = (int)q_factors(L, 8).size();
-    const int4 *d;
-    const int rc = cached_table(p, p->qfft, L, [&](std::vector<int4> &v) {
+    const int rc = cached_table(p, 1, L, [&](std::vector<int4> &v) {
         v = q_factors(L, 8);
         for (int m = 0; m <= L / 2; ++m) v.push_back(fixed_unit(m, L));
-    }, &d);
-    *q = d;
-    *qhalf = d + n;
+    }, q);
+    *qhalf = *q + q_table_count(L, 8);
     return rc;
 }
 
 // the tables of the sine passes of M panels: see DstPass
 int get_dst_tables(idp_plan p, int M, const int4 **out)
 {
-    return cached_table(p, p->qdst, M, [&](std::vector<int4> &q) {
+    return cached_table(p, 2, M, [&](std::vector<int4> &q) {
         const int K = M / 2;
         q = q_factors(K, dst_table_radix(K));
         for (int k = 0; k <= K / 2; ++k) q.push_back(fixed_unit(k, K));
@@ -992,10 +1013,12 @@ int boundary(idp_plan p, const double *rho, double *dst0, double *dst1, cudaStre
     }
     // the faces of axes 0 and 1 read only T0: with fork_rho they start on their
     // own streams while the rest runs on st
-    const bool conc = fork_rho && p->d == 3;
+    // (2-D: the faces of axis 1)
+    const bool conc = fork_rho;
+    const int nbr = p->d == 3 ? 2 : 1;   // branches
     if (conc) {
         IDP_CK(cudaEventRecord(p->fev[0], st));
-        for (int i = 0; i < 2; ++i) IDP_CK(cudaStreamWaitEvent(p->fst[i], p->fev[0], 0));
+        for (int i = 0; i < nbr; ++i) IDP_CK(cudaStreamWaitEvent(p->fst[i], p->fev[0], 0));
     }
     {
         Mark mk(p, IDP_KERNEL_RFFT, st);
@@ -1006,26 +1029,33 @@ int boundary(idp_plan p, const double *rho, double *dst0, double *dst1, cudaStre
         for (int face = 1; face <= 2; ++face) {
             FacePass2D a{};
             const int other = face == 1 ? 2 : 1;
+            cudaStream_t sa = conc && face == 1 ? p->fst[0] : st;
+            double2 *F = p->F + (face - 1) * p->f_cap;
             if (face == 1) { a.T = p->T0; a.sp = p->P[2] + 1; a.sm = 1; }
             else { a.T = p->T1; a.sp = p->P[1] + 1; a.sm = 1; }
             a.np = p->ni[face];
             a.nm = p->P[other] + 1;
             a.khat = p->khat[face];
-            a.acc = p->F;
+            a.acc = F;
+            a.split = fx;   // (the tensor-core modes keep the order of the sum)
             {
-                Mark mk(p, IDP_KERNEL_FACE, st);
-                IDP_CK(launch_face_pass_2d(a, st));
+                Mark mk(p, IDP_KERNEL_FACE, sa);
+                IDP_CK(launch_face_pass_2d(a, sa));
             }
             FaceC2R c{};
-            c.in = p->F; c.nrows = 1; c.Mc = p->M[other]; c.Pc = p->P[other];
+            c.in = F; c.nrows = 1; c.Mc = p->M[other]; c.Pc = p->P[other];
             c.dst0 = dst0; c.dst1 = dst1;
             c.base[0] = 0; c.base[1] = (int64_t)p->M[face] * p->ns[face];
             c.row_stride = 0; c.col_stride = p->ns[other];
             c.skip_row_edges = 0; c.skip_col_edges = (face == 2);
             if ((rc = get_fft(p, p->P[other], &t))) return rc;
             c.t = t;
-            Mark mk(p, IDP_KERNEL_FACE_C2R, st);
-            IDP_CK(launch_face_c2r(c, st));
+            Mark mk(p, IDP_KERNEL_FACE_C2R, sa);
+            IDP_CK(launch_face_c2r(c, sa));
+        }
+        if (conc) {
+            IDP_CK(cudaEventRecord(p->fev[1], p->fst[0]));
+            IDP_CK(cudaStreamWaitEvent(st, p->fev[1], 0));
         }
         return IDP_OK;
     }
@@ -1468,7 +1498,8 @@ int plan_setup(idp_plan p)
                                        1, 0));
             fmax = std::max<int64_t>(fmax, 2 * (Mb + 1));
         }
-        if ((rc = p->alloc(&p->F, fmax))) return rc;
+        if ((rc = p->alloc(&p->F, 2 * fmax))) return rc;
+        p->f_cap = fmax;
     } else {
         int64_t pmax = 0, fmax = 0;
         for (int a_ = 0; a_ < 3; ++a_) {
