@@ -35,8 +35,11 @@ import workloads as w  # noqa: E402
 METRIC = "grid points/s at 6th order, FP64 vs mixed-precision at stated max error"
 UNIT = "grid points/s"
 L2_FLUSH_BYTES = 512 << 20          # > 129 MB of L2
-FP64_PEAK_TFLOPS = 152 * 4 * 2.07e9 / 1e12   # 152 SMs x 4 FP64 flop/clk x 2.07 GHz
-FP64_PROBE_TFLOPS = 1.198           # FMA-chain probe on this GPU model, 1995 MHz
+# The sine passes run in 64-bit fixed point on the two integer pipes: 152 SMs x 2 x 64 lanes
+# per clock x 2.07 GHz.  An addition takes 2 lane operations, a product 6 (three multiply-adds
+# and the splitting of an operand); an FFT has about three additions to a product.
+INT_PEAK_TOPS = 152 * 128 * 2.07e9 / 1e12
+INT_OPS_PER_FLOP = 3.0
 KERNEL_NAMES = {1: "dst_pass", 2: "rfft", 3: "face", 4: "face_invb", 5: "face_c2r", 6: "gtilde_layers",
                 7: "rhs6_w", 8: "rhs6_core", 9: "rhs6_extrap", 10: "gtilde_expand", 11: "dst_pass_layers",
                 12: "mixed_pass", 13: "support_flags", 14: "rhs6_expand", 15: "line1d", 16: "pad",
@@ -408,12 +411,12 @@ def run_headline(g, args, prob):
     out["kernel_ms_per_step"] = {k: sum(v) / reps for k, v in ks.items()}
     out["dominant_kernel"] = max(ks, key=lambda k: sum(ks[k]))
     dst_ms = statistics.mean(ks["dst_pass"])
-    achieved = dst_flops_per_launch(prob) / (dst_ms / 1e3) / 1e12
-    out["roofline"] = {"bound": "alu", "kernel": "dst_pass (FP64 sine-transform pass)",
-                       "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                       "frac": achieved / FP64_PEAK_TFLOPS,
-                       "peak_note": "FP64 derived: 152 SMs x 4 flop/clk x 2.07 GHz; "
-                                    "FMA-chain probe measured %.3f" % FP64_PROBE_TFLOPS,
+    achieved = INT_OPS_PER_FLOP * dst_flops_per_launch(prob) / (dst_ms / 1e3) / 1e12
+    out["roofline"] = {"bound": "alu", "kernel": "dst_pass (sine-transform pass, 64-bit fixed point)",
+                       "achieved": achieved, "peak": INT_PEAK_TOPS, "unit": "T integer lane operations/s",
+                       "frac": achieved / INT_PEAK_TOPS,
+                       "peak_note": "derived: 152 SMs x 128 integer lanes/clk x 2.07 GHz; 3 lane operations "
+                                    "per flop of the transform (2 an addition, 6 a product)",
                        "traffic": DST_TRAFFIC.get(tuple(prob.n)), "avg_launch_ms": dst_ms,
                        "flops_per_launch": dst_flops_per_launch(prob)}
     out["tuning"] = idp.plan_tuning(plan)

@@ -261,22 +261,23 @@ struct QLineCfg {
     static constexpr int G = THIN ? G1 : G0, C = L / G, W = G < 32 ? G : 32;
     static constexpr int LBw = (THIN || L % 3 == 0 ? 128 : 256) / G;
     static constexpr int LB = LBw < 32 ? LBw : 32, T = LB * G;
-    static constexpr int LS = L + 1, BUF = LB * LS, RM = 8, TW = q_tw_count(L, RM);
-    static constexpr size_t SMEM = sizeof(qc) * (2 * BUF + TW);
+    static constexpr int LS = q_line(L), BUF = LB * LS, RM = 8, TW = q_tw_count(L, RM);
+    static constexpr size_t SMEM = sizeof(qc) * (BUF + TW);
+    static constexpr int BPS = (C <= 8 ? 1024 : 640) / T;   // blocks per SM that the registers allow
     static_assert((G & (G - 1)) == 0 && T % 32 == 0, "power-of-two groups, whole warps");
-    static_assert(sizeof(int) * (L + LB) <= sizeof(qc) * BUF, "the non-zero marks fit the scratch buffer");
+    static_assert(sizeof(int) * (L + LB) <= sizeof(qc) * BUF, "the non-zero marks fit the buffer");
 };
 
 template <int L, bool THIN>
-__global__ void __launch_bounds__(QLineCfg<L, THIN>::T) rfft_q_kernel(const RfftPass a)
+__global__ void __launch_bounds__(QLineCfg<L, THIN>::T, QLineCfg<L, THIN>::BPS) rfft_q_kernel(const RfftPass a)
 {
     using Cfg = QLineCfg<L, THIN>;
     constexpr int LB = Cfg::LB, NT = Cfg::T, G = Cfg::G, C = Cfg::C, LS = Cfg::LS;
     const int M = a.M, N = M - 1;
     extern __shared__ qc smem_q[];
-    qc *bufA = smem_q, *bufB = smem_q + Cfg::BUF;
-    int4 *tws = reinterpret_cast<int4 *>(bufB + Cfg::BUF);
-    __shared__ int s_emax[LB], s_scale[LB], s_any, s_gmax;
+    qc *buf = smem_q;
+    int4 *tws = reinterpret_cast<int4 *>(buf + Cfg::BUF);
+    __shared__ int s_high[LB], s_scale[LB], s_any, s_gmax;
     __shared__ unsigned s_sum[LB];
     int nv;
     int64_t isu, isv, ise, osu, osv, ose;
@@ -312,11 +313,11 @@ __global__ void __launch_bounds__(QLineCfg<L, THIN>::T) rfft_q_kernel(const Rfft
         }
     }
     // stage 1a: non-zero marks of the block's lines and of their element
-    // positions, in the FFT scratch (free until the FFT)
+    // positions, in the FFT buffer (free until the values go in)
     const bool mk = a.fl_row2 != nullptr;
-    int *colnz = reinterpret_cast<int *>(bufB), *rownz = colnz + L;
+    int *colnz = reinterpret_cast<int *>(buf), *rownz = colnz + L;
     if (threadIdx.x < LB) {
-        s_emax[threadIdx.x] = 1;
+        s_high[threadIdx.x] = 0;
         s_sum[threadIdx.x] = 0;
     }
     if (threadIdx.x == 0) s_gmax = 0;
@@ -327,26 +328,22 @@ __global__ void __launch_bounds__(QLineCfg<L, THIN>::T) rfft_q_kernel(const Rfft
     // 1. load: thread (l, g) takes the elements e = g + i G of line l
     const int l = contig ? threadIdx.x / G : threadIdx.x % LB;
     const int g = contig ? threadIdx.x % G : threadIdx.x / LB;
-    const int64_t inb = (int64_t)u * isu + (int64_t)(v0 + l) * isv;
+    const double *in = a.in + (int64_t)u * isu + (int64_t)(v0 + l) * isv + (int64_t)g * ise;
     double x[C];
 #pragma unroll
-    for (int i = 0; i < C; ++i) {
-        const int e = g + i * G;
-        x[i] = (l < nl && e < N) ? a.in[inb + (int64_t)e * ise] : 0.0;
-    }
+    for (int i = 0; i < C; ++i) x[i] = (l < nl && g + i * G < N) ? in[(int64_t)(i * G) * ise] : 0.0;
     if (a.copy) {
+        double *cp = a.copy + (in - a.in);
 #pragma unroll
-        for (int i = 0; i < C; ++i) {
-            const int e = g + i * G;
-            if (l < nl && e < N) a.copy[inb + (int64_t)e * ise] = x[i];
-        }
+        for (int i = 0; i < C; ++i)
+            if (l < nl && g + i * G < N) cp[(int64_t)(i * G) * ise] = x[i];
     }
     __syncthreads();   // the scales and marks are reset
-    int emax = 1;
+    int high = 0;
     bool nz = false;
 #pragma unroll
     for (int i = 0; i < C; ++i) {
-        emax = max(emax, q_expo(x[i]));
+        high = max(high, q_high(x[i]));
         // zero test on the bits (+0 and -0 are zero)
         if ((__double_as_longlong(x[i]) << 1) != 0) {
             nz = true;
@@ -356,9 +353,9 @@ __global__ void __launch_bounds__(QLineCfg<L, THIN>::T) rfft_q_kernel(const Rfft
     if (mk && nz) rownz[l] = 1;
     // 2. the line's scale (lanes of one line: consecutive ones, or those LB apart)
     const int d0 = contig ? 1 : LB, d1 = contig ? Cfg::W : 32;
-    for (int d = d0; d < d1; d <<= 1) emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, d));
+    for (int d = d0; d < d1; d <<= 1) high = max(high, __shfl_xor_sync(0xffffffffu, high, d));
     const bool lead = contig ? (threadIdx.x & (Cfg::W - 1)) == 0 : (threadIdx.x & 31) < LB;
-    if (lead) atomicMax(&s_emax[l], emax);
+    if (lead) atomicMax(&s_high[l], high);
     const int any = __syncthreads_or(nz);
     if (mk) {
         if (threadIdx.x < nl) {
@@ -382,58 +379,56 @@ __global__ void __launch_bounds__(QLineCfg<L, THIN>::T) rfft_q_kernel(const Rfft
         write_zero();
         return;
     }
-    emax = s_emax[l];
-    unsigned sum = 0;
+    const int emax = q_emax(s_high[l]);
+    unsigned sum = C;
 #pragma unroll
     for (int i = 0; i < C; ++i) sum += q_weight(x[i], emax);
     for (int d = d0; d < d1; d <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
     if (lead) atomicAdd(&s_sum[l], sum);
     __syncthreads();
-    const int bits = q_bits(s_sum[l]);
-    if (threadIdx.x < LB) {
-        const int e = s_emax[threadIdx.x];
-        const int eb = e + q_bits(s_sum[threadIdx.x]);
-        s_scale[threadIdx.x] = e == 0x7ff ? Q_NAN : 1102 - eb;
-        atomicMax(&s_gmax, e == 0x7ff ? Q_GNAN : eb);
+    const int eb = emax + q_bits(s_sum[l]), scale = 1102 - eb;   // absolute sum below 2^59 units
+    if (g == 0) {
+        s_scale[l] = emax == 0x7ff ? Q_NAN : scale;
+        if (a.gmax) atomicMax(&s_gmax, emax == 0x7ff ? Q_GNAN : eb);
     }
-    // 3. into bufA viewed as reals: x_e at position e + 1 of the padded sequence (component
+    // 3. into buf viewed as reals: x_e at position e + 1 of the padded sequence (component
     //    1 of element e / 2 for even e), zeros elsewhere; the elements from L / 2 on are
     //    zero and are not read by the first pass
     {
-        long long *zl = reinterpret_cast<long long *>(bufA + l * LS);
-        const int shift = emax + bits - 20;
+        long long *zl = reinterpret_cast<long long *>(buf + l * LS);
+        const QFrom from(scale, emax);
 #pragma unroll
         for (int i = 0; i < C; ++i) {
             const int q = g + i * G + 1;   // <= L
-            if (q < L) zl[2 * q_slot(q >> 1) + (q & 1)] = q_from(x[i], shift);
+            if (i < C - 1 || q < L) zl[2 * q_slot(q >> 1) + (q & 1)] = from(x[i]);
         }
         if (g == 0) zl[0] = 0;
     }
     __syncthreads();
     if (a.gmax && threadIdx.x == 0 && *a.gmax < s_gmax) atomicMax(a.gmax, s_gmax);
     // 4. complex FFT of length L
-    q_fft<L, Cfg::RM, LB, NT, LS, 1, true>(bufA, bufB, tws);
-    const qc *Z = q_passes(L, Cfg::RM) % 2 == 0 ? bufA : bufB;
-    // 5. X'_m = 2 X_m, m = 0..L
-    for (int f = threadIdx.x; f < LB * (L / 2); f += NT) {
-        const int ll = f / (L / 2);
-        const int m = f - ll * (L / 2) + 1;   // 1..L/2
-        if (ll >= nl) continue;
-        const qc *zl = Z + ll * LS;
+    q_fft<L, Cfg::RM, LB, NT, LS, 1, true>(buf, tws);
+    // 5. X'_m = 2 X_m, m = 0..L: G consecutive threads per line
+    const int ll = threadIdx.x / G, gg = threadIdx.x % G;
+    if (ll >= nl) return;
+    const qc *zl = buf + ll * LS;
+    double2 *ol = outb + (int64_t)ll * osv;
+    const QTo to(s_scale[ll]);
+#pragma unroll
+    for (int i = 0; i < (L / 2 + G - 1) / G; ++i) {
+        const int m = 1 + gg + i * G;   // 1..L/2
+        if ((L / 2) % G != 0 && m > L / 2) break;
         const qc zm = zl[q_slot(m)], zc = zl[q_slot(L - m)];
         const long long Er = zm.re + zc.re, Ei = zm.im - zc.im;
         const qc P = q_cmul(qc{zm.re - zc.re, zm.im + zc.im}, __ldg(a.qhalf + m));   // W O = P; X' = E - i P
-        const int s = s_scale[ll];
-        const bool fast = q_fast(s);
-        double2 *ol = outb + (int64_t)ll * osv;
-        ol[(int64_t)m * ose] = make_double2(q_to(Er + P.im, s, fast), q_to(Ei - P.re, s, fast));
-        ol[(int64_t)(L - m) * ose] = make_double2(q_to(Er - P.im, s, fast), q_to(-Ei - P.re, s, fast));
-        if (m == 1) {
-            const qc z0 = zl[0];
-            ol[0] = make_double2(q_to((z0.re + z0.im) << 1, s, fast), s == Q_NAN ? q_to(0, s, fast) : 0.0);
-            ol[(int64_t)L * ose] =
-                make_double2(q_to((z0.re - z0.im) << 1, s, fast), s == Q_NAN ? q_to(0, s, fast) : 0.0);
-        }
+        ol[(int64_t)m * ose] = make_double2(to(Er + P.im), to(Ei - P.re));
+        ol[(int64_t)(L - m) * ose] = make_double2(to(Er - P.im), to(-Ei - P.re));
+    }
+    if (gg == 0) {
+        const qc z0 = zl[0];
+        const double im = to(0);
+        ol[0] = make_double2(to((z0.re + z0.im) << 1), im);
+        ol[(int64_t)L * ose] = make_double2(to((z0.re - z0.im) << 1), im);
     }
 }
 
@@ -718,9 +713,8 @@ __global__ void __launch_bounds__(NT) face_invb_kernel(const FaceInvB a)
                 }
             const qc v = face ? q_sub(sum, dif) : q_add(sum, dif);
             const int ek = t < ncl ? a.ek[(int64_t)(c0 + t) * (L / 2 + 1) + (m <= L / 2 ? m : L - m)] : 0;
-            const int s = g >= Q_GNAN ? Q_NAN : base - ek;
-            const bool fast = q_fast(s);
-            bufA[t * L + m] = make_double2(q_to(v.re, s, fast), q_to(v.im, s, fast));
+            const QTo to(g >= Q_GNAN ? Q_NAN : base - ek);
+            bufA[t * L + m] = make_double2(to(v.re), to(v.im));
         }
     } else {
     const Cx *part = reinterpret_cast<const Cx *>(a.part);

@@ -39,26 +39,30 @@ struct DstCfg {
     static constexpr int M = 2 * K, N = M - 1;
     static constexpr int G = GO, C = K / G, RM = dst_radix(K);
     static constexpr int LB = LBO, T = LB * G;
-    static constexpr int LS = K + 1;                      // line stride of the FFT buffers (16-byte elements)
-    static constexpr int OS = (2 * K + G + 1) | 1;        // line stride of the outputs (8-byte words, odd: lanes
-                                                          // on consecutive lines hit different banks)
-    static constexpr int BUF = (LB * (OS > 2 * LS ? OS : 2 * LS) + 1) / 2;   // 16-byte elements of one buffer
+    static constexpr int LS = q_line(K);                  // line stride of the FFT buffers (16-byte elements)
+    // outputs of a line (8-byte words): U_{2k} at q_slot(k - 1), the odd slots (Re T_k, then
+    // U_{2k+1}) at OD + q_slot(k); line stride OS, odd (lanes on consecutive lines hit
+    // different banks)
+    static constexpr int OD = q_slot(K), OS = 2 * OD - 1;
+    static constexpr int BUF = LB * LS;                   // 16-byte elements of one buffer
+    static_assert(OS <= 2 * LS, "the outputs fit a buffer");
     // tables: FFT factors, e^{-i pi k/K} (k = 0..K/2), sin(pi j/M) (j = 0..K-1, 8 bytes each)
     static constexpr int TW = q_tw_count(K, RM), HALF = TW, SIN = TW + K / 2 + 1, TAB = SIN + K / 2;
-    static constexpr size_t SMEM = sizeof(qc) * (2 * BUF + TAB);
+    static constexpr size_t SMEM = sizeof(qc) * (BUF + TAB);
+    static constexpr int BPS = (C <= 8 ? 1024 : 640) / T;   // blocks per SM that the registers allow
     static_assert(K % G == 0 && (G & (G - 1)) == 0 && G <= 32 && T % 32 == 0 && T <= 256,
                   "whole warps; a group fits a warp");
 };
 
 template <class Cfg, int K>
-__global__ void __launch_bounds__(Cfg::T) dst_pass_kernel(const DstPass a)
+__global__ void __launch_bounds__(Cfg::T, Cfg::BPS) dst_pass_kernel(const DstPass a)
 {
     constexpr int M = Cfg::M, N = Cfg::N, LB = Cfg::LB, NT = Cfg::T, G = Cfg::G, C = Cfg::C, RM = Cfg::RM;
     constexpr int LS = Cfg::LS, OS = Cfg::OS;
     extern __shared__ qc smem_q[];
-    qc *bufA = smem_q, *bufB = smem_q + Cfg::BUF;
-    int4 *tabs = reinterpret_cast<int4 *>(bufB + Cfg::BUF);
-    __shared__ int s_emax[LB], s_scale[LB];
+    qc *buf = smem_q;
+    int4 *tabs = reinterpret_cast<int4 *>(buf + Cfg::BUF);
+    __shared__ int s_high[LB], s_scale[LB];
     __shared__ unsigned s_sum[LB];
     // the tables, made with the plan, come in while the previous launch drains (they are
     // visible after the first barrier)
@@ -67,7 +71,7 @@ __global__ void __launch_bounds__(Cfg::T) dst_pass_kernel(const DstPass a)
         for (int i = threadIdx.x; i < Cfg::TAB; i += NT) tabs[i] = __ldg(a.qtab + i);
     }
     if (threadIdx.x < LB) {
-        s_emax[threadIdx.x] = 1;
+        s_high[threadIdx.x] = 0;
         s_sum[threadIdx.x] = 0;
     }
     pdl_wait();
@@ -88,15 +92,14 @@ __global__ void __launch_bounds__(Cfg::T) dst_pass_kernel(const DstPass a)
         int64_t isu, isv, ise;
         view_strides(a.in, a.axis, isu, isv, ise);
         const double *in = a.in.p + (int64_t)u * isu + (int64_t)(v0 + l) * isv;   // x_i at element i - 1
+        const double *pa = in + (int64_t)(g - 1) * ise, *pb = in + (int64_t)(M - 1 - g) * ise;
+        const int64_t step = G * ise;
+        const bool on = l < nl;
 #pragma unroll
-        for (int i = 0; i < C; ++i) {
-            const int j = g + i * G;
-            xa[i] = 0.0;
-            xb[i] = 0.0;
-            if (l < nl) {
-                xa[i] = in[(int64_t)((j ? j : K) - 1) * ise];
-                if (j) xb[i] = in[(int64_t)(M - j - 1) * ise];
-            }
+        for (int i = 0; i < C; ++i, pa += step, pb -= step) {
+            const bool mid = i == 0 && g == 0;
+            xa[i] = on ? *(mid ? in + (int64_t)(K - 1) * ise : pa) : 0.0;
+            xb[i] = on && !mid ? *pb : 0.0;
         }
         if (a.in_dd) {
 #pragma unroll
@@ -107,81 +110,87 @@ __global__ void __launch_bounds__(Cfg::T) dst_pass_kernel(const DstPass a)
         }
     }
 
-    // 2. the line's scale, from its largest exponent and its absolute sum
-    int emax = 1;
+    // 2. the line's scale, from its largest exponent and its absolute sum (q64.cuh)
+    int high = 0;
 #pragma unroll
-    for (int i = 0; i < C; ++i) emax = max(emax, max(q_expo(xa[i]), q_expo(xb[i])));
+    for (int i = 0; i < C; ++i) high = max(high, max(q_high(xa[i]), q_high(xb[i])));
     // lanes of one line: G consecutive ones, or those LB apart
     const int d0 = contig ? 1 : LB, d1 = contig ? G : 32;
-    for (int d = d0; d < d1; d <<= 1) emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, d));
+    for (int d = d0; d < d1; d <<= 1) high = max(high, __shfl_xor_sync(0xffffffffu, high, d));
     __syncthreads();
     const bool lead = contig ? g == 0 : (threadIdx.x & 31) < LB;
-    if (lead) atomicMax(&s_emax[l], emax);
+    if (lead) atomicMax(&s_high[l], high);
     __syncthreads();
-    emax = s_emax[l];
-    unsigned sum = 0;
+    const int emax = q_emax(s_high[l]);
+    unsigned sum = 2 * C;
 #pragma unroll
     for (int i = 0; i < C; ++i) sum += q_weight(xa[i], emax) + q_weight(xb[i], emax);
     for (int d = d0; d < d1; d <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
     if (lead) atomicAdd(&s_sum[l], sum);
     __syncthreads();
-    const int bits = q_bits(s_sum[l]);
-    if (threadIdx.x < LB) {
-        const int e = s_emax[threadIdx.x];
-        s_scale[threadIdx.x] = e == 0x7ff ? Q_NAN : 1101 - e - q_bits(s_sum[threadIdx.x]);
-    }
+    const int scale = 1101 - emax - q_bits(s_sum[l]);   // absolute sum below 2^58 units
+    if (g == 0) s_scale[l] = emax == 0x7ff ? Q_NAN : scale;
 
-    // 3. pre-processing into bufA viewed as y'[LB][M] (y'_j in component j mod 2 of
+    // 3. pre-processing into buf viewed as y'[LB][M] (y'_j in component j mod 2 of
     //    element j / 2): y'_j = sin(pi j/M) (2 x_j + 2 x_{M-j}) + (x_j - x_{M-j})
     {
-        long long *zl = reinterpret_cast<long long *>(bufA + l * LS);
-        const int shift = emax + bits - 19;
+        long long *zl = reinterpret_cast<long long *>(buf + l * LS);
+        const int2 *sn = reinterpret_cast<const int2 *>(tabs + Cfg::SIN) + g;
+        const QFrom from(scale, emax);
 #pragma unroll
         for (int i = 0; i < C; ++i) {
             const int j = g + i * G;
-            const long long va = q_from(xa[i], shift), vb = q_from(xb[i], shift);
-            const int2 sn = reinterpret_cast<const int2 *>(tabs + Cfg::SIN)[j];
-            const long long p = q_rmul((va + vb) << 1, sn.x, sn.y), m = va - vb;
-            const int j1 = j ? M - j : K;
-            zl[2 * q_slot(j >> 1) + (j & 1)] = j ? p + m : 0;
-            zl[2 * q_slot(j1 >> 1) + (j1 & 1)] = j ? p - m : va << 2;
+            const bool mid = i == 0 && g == 0;
+            const long long va = from(xa[i]), vb = from(xb[i]);
+            const int2 w = sn[i * G];
+            const long long p = q_rmul((va + vb) << 1, w.x, w.y), m = va - vb;
+            const int j1 = mid ? K : M - j;
+            zl[2 * q_slot(j >> 1) + (j & 1)] = mid ? 0 : p + m;
+            zl[2 * q_slot(j1 >> 1) + (j1 & 1)] = mid ? va << 2 : p - m;
         }
     }
     __syncthreads();
 
     // 4. complex FFT of length K
-    q_fft<K, RM, LB, NT, LS>(bufA, bufB, tabs);
-    constexpr bool INA = q_passes(K, RM) % 2 == 0;
-    const qc *Z = INA ? bufA : bufB;
-    long long *o = reinterpret_cast<long long *>(INA ? bufB : bufA);
-    // outputs of a line: U_{2k} at word k - 1; the odd slots (Re T_k, then U_{2k+1}) at
-    // word K + k + k / C (one word of padding per thread of the prefix sum)
+    q_fft<K, RM, LB, NT, LS>(buf, tabs);
 
-    // 5. post-processing: even outputs final, odd slots get Re T_k
-    for (int f = threadIdx.x; f < LB * (K / 2); f += NT) {
-        const int ll = f / (K / 2);
-        const int k = f - ll * (K / 2) + 1;      // 1..K/2
-        const qc *zl = Z + ll * LS;
-        long long *ol = o + ll * OS;
-        const qc zk = zl[q_slot(k)], zc = zl[q_slot(K - k)];
-        const long long Er = zk.re + zc.re, Ei = zk.im - zc.im;
-        const qc P = q_cmul(qc{zk.re - zc.re, zk.im + zc.im}, tabs[Cfg::HALF + k]);
-        ol[k - 1] = P.re - Ei;
-        ol[K - k - 1] = P.re + Ei;
-        ol[K + k + k / C] = Er + P.im;
-        ol[K + (K - k) + (K - k) / C] = Er - P.im;
-        if (k == 1) ol[K] = zl[0].re + zl[0].im;
+    // 5. post-processing, in place like the passes: even outputs final, odd slots get
+    //    Re T_k.  From here to the prefix sum: G consecutive threads per line
+    const int ll = threadIdx.x / G, gg = threadIdx.x % G;
+    long long *o = reinterpret_cast<long long *>(buf), *ol = o + ll * OS;
+    {
+        constexpr int H = (K / 2 + G - 1) / G;
+        const qc *zl = buf + ll * LS;
+        const int4 *half = tabs + Cfg::HALF;
+        qc zk[H], zc[H], z0;
+#pragma unroll
+        for (int i = 0; i < H; ++i) {
+            const int k = min(1 + gg + i * G, K / 2);   // 1..K/2
+            zk[i] = zl[q_slot(k)];
+            zc[i] = zl[q_slot(K - k)];
+        }
+        if (gg == 0) z0 = zl[0];
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < H; ++i) {
+            const int k = min(1 + gg + i * G, K / 2);
+            const long long Er = zk[i].re + zc[i].re, Ei = zk[i].im - zc[i].im;
+            const qc P = q_cmul(qc{zk[i].re - zc[i].re, zk[i].im + zc[i].im}, half[k]);
+            ol[q_slot(k - 1)] = P.re - Ei;
+            ol[q_slot(K - k - 1)] = P.re + Ei;
+            ol[Cfg::OD + q_slot(k)] = Er + P.im;
+            ol[Cfg::OD + q_slot(K - k)] = Er - P.im;
+        }
+        if (gg == 0) ol[Cfg::OD] = z0.re + z0.im;
     }
     __syncthreads();
 
-    // 6. prefix sum over the odd slots: G lanes per line, C consecutive slots each
+    // 6. prefix sum over the odd slots: C consecutive ones per lane
     {
-        const int ll = threadIdx.x / G, gg = threadIdx.x % G;
-        long long *ol = o + ll * OS + K + gg * (C + 1);
         long long val[C], run = 0;
 #pragma unroll
         for (int c = 0; c < C; ++c) {
-            run += ol[c];
+            run += ol[Cfg::OD + q_slot(gg * C + c)];
             val[c] = run;
         }
         long long incl = run;
@@ -192,55 +201,56 @@ __global__ void __launch_bounds__(Cfg::T) dst_pass_kernel(const DstPass a)
         }
         const long long below = incl - run;
 #pragma unroll
-        for (int c = 0; c < C; ++c) ol[c] = val[c] + below;
+        for (int c = 0; c < C; ++c) ol[Cfg::OD + q_slot(gg * C + c)] = val[c] + below;
     }
     __syncthreads();
 
-    // 7. epilogue and store
-    int64_t osu, osv, ose, asu, asv, ase, tsu, tsv, tse;
+    // 7. epilogue and store: thread (l, g) of the load takes the outputs e = g + i G of line l
+    //    (U_{e+1}); consecutive threads again on consecutive e or on consecutive lines
+    if (l >= nl) return;
+    int64_t osu, osv, ose;
     view_strides(a.out, a.axis, osu, osv, ose);
-    view_strides(a.add, a.axis, asu, asv, ase);
-    {
-        // the tables are dense interior arrays n0 x n1 x n2
-        const View3 tv{nullptr, (int64_t)a.n1 * a.n2, a.n2, 1};
-        view_strides(tv, a.axis, tsu, tsv, tse);
+    double *out = a.out.p + (int64_t)u * osu + (int64_t)(v0 + l) * osv + (int64_t)g * ose;
+    const int64_t step = G * ose;
+    const QTo to(s_scale[l]);
+    const long long *w0 = o + l * OS;
+    auto word = [&](int i) -> long long {
+        const int e = g + i * G, h = e >> 1;
+        return w0[((e & 1) ? 0 : Cfg::OD) + q_slot(h)];
+    };
+    if (!a.tab && !a.add.p) {
+#pragma unroll
+        for (int i = 0; i < 2 * C; ++i, out += step)
+            if (i < 2 * C - 1 || g + i * G < N) *out = to(word(i));
+        return;
     }
-    double *out = a.out.p + (int64_t)u * osu + (int64_t)v0 * osv;
-    const double *tab = a.tab + ((int64_t)u * tsu + (int64_t)v0 * tsv);
-    const double *add = a.add.p + ((int64_t)u * asu + (int64_t)v0 * asv);
+    int64_t asu, asv, ase, tsu, tsv, tse;
+    view_strides(a.add, a.axis, asu, asv, ase);
+    // the tables are dense interior arrays n0 x n1 x n2
+    view_strides(View3{nullptr, (int64_t)a.n1 * a.n2, a.n2, 1}, a.axis, tsu, tsv, tse);
+    const double *tab = a.tab + ((int64_t)u * tsu + (int64_t)(v0 + l) * tsv + (int64_t)g * tse);
+    const double *add = a.add.p + ((int64_t)u * asu + (int64_t)(v0 + l) * asv + (int64_t)g * ase);
     // groups of EG outputs: the table and addend loads of a group go out before
     // its stores (which, as far as the compiler knows, could alias them)
-    constexpr int EG = 4;
-    for (int f0 = threadIdx.x; f0 < LB * N; f0 += EG * NT) {
-        double tv[EG], av[EG];
-        if (a.tab || a.add.p) {
+    constexpr int EG = (2 * C) % 4 == 0 ? 4 : 2;
 #pragma unroll
-            for (int q = 0; q < EG; ++q) {
-                const int f = f0 + q * NT;
-                int ll, e;
-                if (contig) { ll = f / N; e = f - ll * N; }
-                else { e = f / LB; ll = f - e * LB; }
-                tv[q] = 1.0;
-                av[q] = 0.0;
-                if (f >= LB * N || ll >= nl) continue;
-                if (a.tab) tv[q] = tab[(int64_t)ll * tsv + (int64_t)e * tse];
-                if (a.add.p) av[q] = add[(int64_t)ll * asv + (int64_t)e * ase];
-            }
-        }
+    for (int i0 = 0; i0 < 2 * C; i0 += EG) {
+        double tv[EG], av[EG];
 #pragma unroll
         for (int q = 0; q < EG; ++q) {
-            const int f = f0 + q * NT;
-            if (f >= LB * N) break;
-            int ll, e;
-            if (contig) { ll = f / N; e = f - ll * N; }
-            else { e = f / LB; ll = f - e * LB; }
-            if (ll >= nl) continue;
-            const int h = e >> 1, s = s_scale[ll];
-            const long long w = o[ll * OS + ((e & 1) ? h : K + h + h / C)];
-            double y = q_to(w, s, q_fast(s));
+            const int i = i0 + q;
+            const bool on = i < 2 * C - 1 || g + i * G < N;
+            tv[q] = on && a.tab ? tab[(int64_t)(i * G) * tse] : 1.0;
+            av[q] = on && a.add.p ? add[(int64_t)(i * G) * ase] : 0.0;
+        }
+#pragma unroll
+        for (int q = 0; q < EG; ++q, out += step) {
+            const int i = i0 + q;
+            if (i == 2 * C - 1 && g + i * G >= N) break;
+            double y = to(word(i));
             if (a.tab) y = a.add.p ? fma(tv[q], y, av[q]) : tv[q] * y;
-            else if (a.add.p) y += av[q];
-            out[(int64_t)ll * osv + (int64_t)e * ose] = y;
+            else y += av[q];
+            *out = y;
         }
     }
 }

@@ -27,22 +27,10 @@ template <int L_>
 struct FaceQCfg {
     static constexpr int L = L_, RM = 8, U = L / 8;
     static constexpr int TC = (L % 3 == 0 ? 1536 : 2048) / L < 32 ? (L % 3 == 0 ? 1536 : 2048) / L : 32;
-    static constexpr int NT = TC * U, LS = L + 1, Ph = L / 2, KS = Ph + 1;
+    static constexpr int NT = TC * U, LS = q_line(L), Ph = L / 2, KS = Ph + 1;
     static constexpr int R0 = q_radix(L, 1, RM), TW = q_tw_count(L, RM);
-    static constexpr size_t SMEM = sizeof(qc) * (2 * TC * LS + TW) + sizeof(int2) * TC * KS;
+    static constexpr size_t SMEM = sizeof(qc) * (TC * LS + TW) + sizeof(int2) * TC * KS;
 };
-
-// the passes from span Ns to span L / 8; the result is in X or Y (q_passes)
-template <class Cfg, int Ns>
-__device__ __forceinline__ void face_passes(qc *X, qc *Y, const int4 *tw)
-{
-    if constexpr (Ns * 8 < Cfg::L) {
-        constexpr int R = q_radix(Cfg::L, Ns, Cfg::RM);
-        q_pass<Cfg::L, Ns, Cfg::RM, Cfg::TC, Cfg::NT, Cfg::LS>(X, Y, tw);
-        __syncthreads();
-        face_passes<Cfg, Ns * R>(Y, X, tw + (R - 1) * Ns);
-    }
-}
 
 __device__ __forceinline__ void cp_async8(void *dst, const void *src)
 {
@@ -56,13 +44,14 @@ __global__ void __launch_bounds__(FaceQCfg<L>::NT, 2) face_q_kernel(const FaceQP
     using Cfg = FaceQCfg<L>;
     constexpr int TC = Cfg::TC, NT = Cfg::NT, LS = Cfg::LS, KS = Cfg::KS, U = Cfg::U, Ph = Cfg::Ph, R0 = Cfg::R0;
     extern __shared__ qc smem_q[];
-    qc *bufA = smem_q, *bufB = bufA + TC * LS;
-    int4 *tws = reinterpret_cast<int4 *>(bufB + TC * LS);
+    qc *buf = smem_q;
+    int4 *tws = reinterpret_cast<int4 *>(buf + TC * LS);
     int2 *ks = reinterpret_cast<int2 *>(tws + Cfg::TW);
     const int c0 = blockIdx.x * TC, ncl = min(TC, a.nc - c0);
     const int chunk = blockIdx.y, diff = blockIdx.z;
     const int npair = (a.np + 1) / 2;
-    const int shift = *a.gmax + a.lgn - 20;
+    const int g = *a.gmax;
+    const QFrom from(1102 - min(g, 2100) - a.lgn, g - 31);   // every column's absolute sum below 2^61 units
     for (int f = threadIdx.x; f < Cfg::TW; f += NT) tws[f] = __ldg(a.q + f);
     const int2 *kq = a.kq + ((int64_t)diff * npair * a.nc + c0) * KS;
 
@@ -107,23 +96,22 @@ __global__ void __launch_bounds__(FaceQCfg<L>::NT, 2) face_q_kernel(const FaceQP
                     if (q < NZ) {
                         const double sr = diff ? y1[q].x - y2[q].x : y1[q].x + y2[q].x;
                         const double si = diff ? y1[q].y - y2[q].y : y1[q].y + y2[q].y;
-                        v[q] = qc{q_from(sr, shift), q_from(si, shift)};
+                        v[q] = qc{from(sr), from(si)};
                     }
                 }
                 q_dft<R0>(v);
-                qc *y = bufA + t * LS;
+                qc *y = buf + t * LS;
 #pragma unroll
                 for (int q = 0; q < R0; ++q) y[q_slot(jj * R0 + q)] = v[q];
             }
         }
         __syncthreads();
-        face_passes<Cfg, R0>(bufA, bufB, tws);
+        q_fft<L, Cfg::RM, TC, NT, LS, R0, false, U>(buf, tws);
         // the last pass, its outputs times the spectra
-        constexpr bool INA = (q_passes(L, Cfg::RM) - 2) % 2 == 0;
         asm volatile("cp.async.wait_all;\n" ::: "memory");
         __syncthreads();
         {
-            const qc *x = (INA ? bufA : bufB) + ct * LS;
+            const qc *x = buf + ct * LS;
             const int4 *tw = tws + (Cfg::TW - 7 * U);
             qc v[8];
 #pragma unroll
@@ -140,7 +128,7 @@ __global__ void __launch_bounds__(FaceQCfg<L>::NT, 2) face_q_kernel(const FaceQP
                 acc[q].im += q_rmul(v[q].im, w.x, w.y);
             }
         }
-        __syncthreads();   // the buffers are free
+        __syncthreads();   // the buffer is free
     }
     if (ct < ncl) {
         qc *part = a.part + (((int64_t)chunk * 2 + diff) * a.nc + c0 + ct) * L;

@@ -112,10 +112,13 @@ __device__ __forceinline__ void q_dft(qc *v)
     else q_dft8(v);
 }
 
-// shared-memory place of element e of a line (16-byte elements): the three low bits are
-// XORed with the next three, so that the eight lanes of a quarter-warp hit eight
-// bank groups both in a pass's reads (consecutive e) and in its writes (stride R)
-__device__ __forceinline__ int q_slot(int e) { return e ^ ((e >> 3) & 7); }
+// Shared-memory place of element e of a line (16-byte elements): one element of padding
+// after every eight, so that the eight lanes of a quarter-warp hit eight bank groups in a
+// pass's reads (consecutive e) and in its writes (stride R), at offsets that are constants
+// of the pass (an XOR of the low bits does the same, but costs integer instructions on
+// every access).  q_line: padded length of a line, odd.
+__host__ __device__ constexpr int q_slot(int e) { return e + (e >> 3); }
+__host__ __device__ constexpr int q_line(int L) { return q_slot(L) | 1; }
 
 // The radices of the passes of length L after a span of Ns: one radix-3 pass first for
 // 3 * 2^m, then radix-4 (or radix-2) until a power of RM (4 or 8) is left, then RM.
@@ -130,10 +133,6 @@ __host__ __device__ constexpr int q_radix(int L, int Ns, int RM)
     if (head == 2) return RM == 8 && rest >= 16 ? 4 : 2;   // 16 = 4 * 4, 128 = 4 * 4 * 8
     return RM;
 }
-__host__ __device__ constexpr int q_passes(int L, int RM, int Ns = 1)
-{
-    return Ns == L ? 0 : 1 + q_passes(L, RM, Ns * q_radix(L, Ns, RM));
-}
 // entries of the factor table of length L, from span Ns on
 __host__ __device__ constexpr int q_tw_count(int L, int RM, int Ns = 1)
 {
@@ -141,84 +140,125 @@ __host__ __device__ constexpr int q_tw_count(int L, int RM, int Ns = 1)
 }
 
 // One Stockham pass of radix R at span Ns over LB lines (line stride LS elements) by
-// NT threads; tw: the pass's factors w_{R Ns}^{k q}, [q - 1][k].  HZ: the elements from
-// L / 2 on are zero and not read.
+// NT threads, in place: every thread takes its units into registers, and after a block
+// barrier writes their results.  tw: the pass's factors w_{R Ns}^{k q}, [q - 1][k].  HZ: the
+// elements from L / 2 on are zero and not read.  Ends with a block barrier.
+// (One buffer and a second barrier per pass against two buffers: at M = 256 the sine
+// pass then keeps four blocks per SM where two buffers with their padding allowed two.)
 template <int L, int Ns, int RM, int LB, int NT, int LS, bool HZ = false>
-__device__ __forceinline__ void q_pass(const qc *__restrict__ X, qc *__restrict__ Y, const int4 *__restrict__ tw)
+__device__ __forceinline__ void q_pass(qc *X, const int4 *__restrict__ tw)
 {
-    constexpr int R = q_radix(L, Ns, RM), U = L / R;
-#pragma unroll 1
-    for (int b = threadIdx.x; b < LB * U; b += NT) {
-        const int line = b / U, j = b - line * U, k = j % Ns;
-        const qc *x = X + line * LS;
-        qc v[R];
+    constexpr int R = q_radix(L, Ns, RM), U = L / R, UNITS = LB * U, IT = (UNITS + NT - 1) / NT;
+    // j + q U and (j - k) R + k + q Ns: place of the first plus a constant where nothing
+    // carries into the padding count
+    constexpr bool RLIN = U % 8 == 0, WLIN = Ns % 8 == 0 || (R != 3 && (Ns & (Ns - 1)) == 0);
+    qc v[IT][R];
+#pragma unroll
+    for (int it = 0; it < IT; ++it) {
+        const int b = threadIdx.x + it * NT, line = b / U, j = b - line * U;
+        if (UNITS % NT != 0 && b >= UNITS) break;
+        const qc *x = X + line * LS + (RLIN ? q_slot(j) : 0);
 #pragma unroll
         for (int q = 0; q < R; ++q) {
-            if (HZ && q * U >= L / 2) v[q] = qc{0, 0};
-            else if (HZ && (q + 1) * U > L / 2) v[q] = j + q * U < L / 2 ? x[q_slot(j + q * U)] : qc{0, 0};
-            else v[q] = x[q_slot(j + q * U)];
+            const int at = RLIN ? q_slot(q * U) : q_slot(j + q * U);
+            if (HZ && q * U >= L / 2) v[it][q] = qc{0, 0};
+            else if (HZ && (q + 1) * U > L / 2) v[it][q] = j + q * U < L / 2 ? x[at] : qc{0, 0};
+            else v[it][q] = x[at];
         }
-        if constexpr (Ns > 1) {
-#pragma unroll
-            for (int q = 1; q < R; ++q) v[q] = q_cmul(v[q], tw[(q - 1) * Ns + k]);
-        }
-        q_dft<R>(v);
-        qc *y = Y + line * LS;
-        const int base = (j - k) * R + k;
-#pragma unroll
-        for (int q = 0; q < R; ++q) y[q_slot(base + q * Ns)] = v[q];
     }
+    __syncthreads();
+#pragma unroll
+    for (int it = 0; it < IT; ++it) {
+        const int b = threadIdx.x + it * NT, line = b / U, j = b - line * U, k = j % Ns;
+        if (UNITS % NT != 0 && b >= UNITS) break;
+        if constexpr (Ns > 1) {
+            const int4 *w = tw + k;
+#pragma unroll
+            for (int q = 1; q < R; ++q) v[it][q] = q_cmul(v[it][q], w[(q - 1) * Ns]);
+        }
+        q_dft<R>(v[it]);
+        const int base = (j - k) * R + k;
+        qc *y = X + line * LS + (WLIN ? q_slot(base) : 0);
+#pragma unroll
+        for (int q = 0; q < R; ++q) y[WLIN ? q_slot(q * Ns) : q_slot(base + q * Ns)] = v[it][q];
+    }
+    __syncthreads();
 }
 
-// Forward FFT of LB lines of length L (a multiple of 8) in X, from span Ns on; Y is
-// scratch.  The result is in X if the number of passes is even, else in Y; ends
-// with a block barrier.  tw: the factors of the passes after span Ns, one after the
-// other (none for the first pass at Ns = 1).  HZ (first pass): see q_pass.
-template <int L, int RM, int LB, int NT, int LS, int Ns = 1, bool HZ = false>
-__device__ __forceinline__ void q_fft(qc *X, qc *Y, const int4 *__restrict__ tw)
+// Forward FFT of LB lines of length L (a multiple of 8) in place, from span Ns on up to
+// span NE.  tw: the factors of the passes after span Ns, one after the other (none for
+// the first pass at Ns = 1).  HZ (first pass): see q_pass.
+template <int L, int RM, int LB, int NT, int LS, int Ns = 1, bool HZ = false, int NE = L>
+__device__ __forceinline__ void q_fft(qc *X, const int4 *__restrict__ tw)
 {
-    if constexpr (Ns < L) {
+    if constexpr (Ns < NE) {
         constexpr int R = q_radix(L, Ns, RM);
-        q_pass<L, Ns, RM, LB, NT, LS, HZ>(X, Y, tw);
-        __syncthreads();
-        q_fft<L, RM, LB, NT, LS, Ns * R>(Y, X, tw + (Ns > 1 ? (R - 1) * Ns : 0));
+        q_pass<L, Ns, RM, LB, NT, LS, HZ>(X, tw);
+        q_fft<L, RM, LB, NT, LS, Ns * R, false, NE>(X, tw + (Ns > 1 ? (R - 1) * Ns : 0));
     }
 }
 
 // ---- scales --------------------------------------------------------------------
-// A line's scale from two reductions over its FP64 values: the largest exponent field
-// emax, and the sum S of q_weight (the magnitudes in units of 2^(emax - 1043), each
-// rounded up).  With bits = bit length of S, the absolute sum is below 2^(emax - 1043 + bits).
-// (a subnormal value has the exponent field 1 and no leading bit; zeros weigh 1 unit)
-__device__ __forceinline__ int q_expo(double x) { return max((__double2hiint(x) >> 20) & 0x7ff, 1); }
-__device__ __forceinline__ unsigned q_lead(int h) { return (h & 0x7ff00000) ? 0x100000u : 0u; }
+// A line's scale from two reductions over its FP64 values: the largest high word (sign off),
+// whose exponent field is emax, and the sum S of the magnitudes in units of
+// 2^(emax - 1043), each rounded up.  With bits = bit length of S, the absolute sum is below
+// 2^(emax - 1043 + bits).  (A subnormal value counts as the smallest normal one here.)
+__device__ __forceinline__ int q_high(double x) { return __double2hiint(x) & 0x7fffffff; }
+__device__ __forceinline__ int q_emax(int high) { return max(high >> 20, 1); }
+__device__ __forceinline__ unsigned q_shr(unsigned x, int n)   // 0 for n >= 32
+{
+    unsigned r;
+    asm("shr.u32 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(n));
+    return r;
+}
+// one unit less than the value's part of S
 __device__ __forceinline__ unsigned q_weight(double x, int emax)
 {
-    const int h = __double2hiint(x);
-    const unsigned m = ((unsigned)h & 0xfffffu) | q_lead(h);
-    return (m >> min(emax - q_expo(x), 31)) + 1u;
+    const int h = q_high(x);
+    return q_shr(((unsigned)h & 0xfffffu) | 0x100000u, max(emax - (h >> 20), 0));
 }
 __device__ __forceinline__ int q_bits(unsigned S) { return max(32 - __clz((int)S), 21); }
 
-// x 2^(1101 - emax - bits) rounded to nearest: below 2^58 in sum over the line
-__device__ __forceinline__ long long q_from(double x, int shift)   // shift = emax + bits - 19
-{
-    const int h = __double2hiint(x);
-    const unsigned m = ((unsigned)h & 0xfffffu) | q_lead(h);
-    const unsigned long long f = (((unsigned long long)m << 32) | (unsigned)__double2loint(x)) << 7;
-    const int r = min(shift - q_expo(x), 63);
-    const long long v = (long long)(((f >> (r - 1)) + 1) >> 1), s = h >> 31;
-    return (v ^ s) - s;
-}
+// x 2^s rounded to nearest, |x| 2^s < 2^60
+struct QFrom {
+    int add, low, s;
+    __device__ __forceinline__ QFrom(int s_, int emax) : add(s_ << 20), s(s_)
+    {
+        // values whose exponent field plus s is below 1 give 0 (their half unit is far
+        // above them); next to the smallest numbers the general form below runs instead
+        low = emax < 128 ? -1 : max(1 - s_, 1) << 20;
+    }
+    __device__ __forceinline__ long long operator()(double x) const
+    {
+        const int h = __double2hiint(x);
+        if (low >= 0) {
+            // the power of two goes into the exponent field, the conversion runs on the
+            // otherwise idle FP64 pipe (18 integer instructions if done by shifts)
+            const int g = (h & 0x7fffffff) < low ? 0 : h + add;
+            return __double2ll_rn(__hiloint2double(g, __double2loint(x)));
+        }
+        const unsigned lead = (h & 0x7ff00000) ? 0x100000u : 0u;
+        const unsigned long long f =
+            (((unsigned long long)(((unsigned)h & 0xfffffu) | lead) << 32) | (unsigned)__double2loint(x)) << 7;
+        const int r = max(min(1082 - s - q_emax(h & 0x7fffffff), 63), 1);
+        const long long v = (long long)(((f >> (r - 1)) + 1) >> 1), t = h >> 31;
+        return (v ^ t) - t;
+    }
+};
 constexpr int Q_NAN = 1 << 30;   // scale of a line with a NaN or an infinity
 constexpr int Q_GNAN = 1 << 20;  // emax + bits of such a line in a maximum over lines
-// v 2^-s as FP64; fast: 2^-s and every |v| keep the result normal
-__device__ __forceinline__ bool q_fast(int s) { return s <= 1022 && s >= -960; }
-__device__ __forceinline__ double q_to(long long v, int s, bool fast)
-{
-    const double d = __ll2double_rn(v);
-    if (fast) return __hiloint2double(v ? __double2hiint(d) - (s << 20) : 0, __double2loint(d));
-    return s == Q_NAN ? __longlong_as_double(0x7ff8000000000000LL) : scalbn(d, -s);
-}
+// v 2^-s as FP64
+struct QTo {
+    int sub, s;
+    bool fast;   // 2^-s and every |v| keep the result normal
+    __device__ __forceinline__ explicit QTo(int s_) : sub(s_ << 20), s(s_), fast(s_ <= 1022 && s_ >= -960) {}
+    __device__ __forceinline__ double operator()(long long v) const
+    {
+        const double d = __ll2double_rn(v);
+        const int h = __double2hiint(d);
+        if (fast) return __hiloint2double(h ? h - sub : 0, __double2loint(d));
+        return s == Q_NAN ? __longlong_as_double(0x7ff8000000000000LL) : scalbn(d, -s);
+    }
+};
 
 }  // namespace idp
