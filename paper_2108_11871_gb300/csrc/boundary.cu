@@ -251,19 +251,19 @@ __global__ void __launch_bounds__(RfftThreads<R, L>::value) rfft_kernel(const Rf
 // ---------------------------------------------------------------- stage 1, fixed point
 // The FP64 form of stage 1 in block fixed point (q64.cuh): every line on its own
 // scale, FP64 in and out.  G threads per line, C of its elements each; LB lines per block.
-// Two shapes: up to 256 threads with 8 or 12 elements each, and, for launches below four of
+// Two shapes: up to 256 threads with 8 or 6 elements each, and, for launches below four of
 // its blocks per SM, whose time is the latency of one block, fewer lines on up to four
 // times the threads per line (65^2: 28 us per solve with the first, 22 with the second).
 template <int L_, bool THIN>
 struct QLineCfg {
     static constexpr int L = L_;
-    static constexpr int G0 = L % 3 == 0 ? L / 12 : L / 8, G1 = 4 * G0 > 64 ? 64 : 4 * G0;
+    static constexpr int G0 = L % 3 == 0 ? L / 6 : L / 8, G4 = (L % 3 == 0 ? 2 : 4) * G0, G1 = G4 > 64 ? 64 : G4;
     static constexpr int G = THIN ? G1 : G0, C = L / G, W = G < 32 ? G : 32;
-    static constexpr int LBw = (THIN || L % 3 == 0 ? 128 : 256) / G;
+    static constexpr int LBw = (THIN ? 128 : 256) / G;
     static constexpr int LB = LBw < 32 ? LBw : 32, T = LB * G;
     static constexpr int LS = q_line(L), BUF = LB * LS, RM = 8, TW = q_tw_count(L, RM);
     static constexpr size_t SMEM = sizeof(qc) * (BUF + TW);
-    static constexpr int BPS = (C <= 8 ? 1024 : 640) / T;   // blocks per SM that the registers allow
+    static constexpr int BPS = 1024 / T;   // blocks per SM that the registers allow
     static_assert((G & (G - 1)) == 0 && T % 32 == 0, "power-of-two groups, whole warps");
     static_assert(sizeof(int) * (L + LB) <= sizeof(qc) * BUF, "the non-zero marks fit the buffer");
 };

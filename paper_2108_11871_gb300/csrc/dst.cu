@@ -49,7 +49,7 @@ struct DstCfg {
     // tables: FFT factors, e^{-i pi k/K} (k = 0..K/2), sin(pi j/M) (j = 0..K-1, 8 bytes each)
     static constexpr int TW = q_tw_count(K, RM), HALF = TW, SIN = TW + K / 2 + 1, TAB = SIN + K / 2;
     static constexpr size_t SMEM = sizeof(qc) * (BUF + TAB);
-    static constexpr int BPS = (C <= 8 ? 1024 : 640) / T;   // blocks per SM that the registers allow
+    static constexpr int BPS = 1024 / T;   // blocks per SM that the registers allow
     static_assert(K % G == 0 && (G & (G - 1)) == 0 && G <= 32 && T % 32 == 0 && T <= 256,
                   "whole warps; a group fits a warp");
 };
@@ -261,14 +261,14 @@ cudaError_t launch_cfg(const DstPass &a, int nu, int nv, cudaStream_t st)
     return launch_pdl(dst_pass_kernel<Cfg, K>, dim3((nv + Cfg::LB - 1) / Cfg::LB, nu), dim3(Cfg::T), Cfg::SMEM, st, a);
 }
 
-// The shapes of a pass: Big (up to 256 threads, C = 8 or 12 pairs a thread), Mid with half
+// The shapes of a pass: Big (up to 256 threads, C = 8 or 6 pairs a thread), Mid with half
 // its lines, and Thin with up to four times the threads per line, for launches that leave most of the chip idle and so are as long as one block.
 template <int K>
 struct DstShapes {
-    static constexpr int G = K % 3 == 0 ? K / 12 : K / 8;
+    static constexpr int G = K % 3 == 0 ? K / 6 : K / 8;
     static constexpr int BIG = 256 / G < 32 ? 256 / G : 32;
     static constexpr int MID = BIG / 2 * G >= 32 ? BIG / 2 : BIG;
-    static constexpr int GT = 4 * G < 32 ? 4 * G : 32;
+    static constexpr int GT = (K % 3 == 0 ? 2 : 4) * G < 32 ? (K % 3 == 0 ? 2 : 4) * G : 32;
     static constexpr int THIN = GT >= 32 ? 2 : GT >= 16 ? 4 : 8;
     using Big = DstCfg<K, BIG, G>;
     using Mid = DstCfg<K, MID, G>;

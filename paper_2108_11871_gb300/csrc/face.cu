@@ -21,13 +21,24 @@ namespace idp {
 
 namespace {
 
-// TC columns (consecutive frequencies c) per block, a thread for each radix-8 unit of the
-// last pass, which keeps the unit's 8 sums in registers
+// TC columns (consecutive frequencies c) per block and E = 8 elements (3 * 2^m: 6) of a
+// column per thread: one or two units of the last pass, whose sums it keeps in registers.
+// The line stride makes the first pass's writes conflict-free (8 / TC units of TC columns
+// at a time).
 template <int L_>
 struct FaceQCfg {
-    static constexpr int L = L_, RM = 8, U = L / 8;
-    static constexpr int TC = (L % 3 == 0 ? 1536 : 2048) / L < 32 ? (L % 3 == 0 ? 1536 : 2048) / L : 32;
-    static constexpr int NT = TC * U, LS = q_line(L), Ph = L / 2, KS = Ph + 1;
+    static constexpr int L = L_, RM = 8, E = L % 3 == 0 ? 6 : 8;
+    static constexpr int last(int Ns)
+    {
+        return Ns * q_radix(L_, Ns, 8) == L_ ? q_radix(L_, Ns, 8) : last(Ns * q_radix(L_, Ns, 8));
+    }
+    static constexpr int RL = last(1), UL = L / RL, IL = E / RL;   // the last pass: radix, units, units per thread
+    static constexpr int TC = 256 * E / L < 32 ? 256 * E / L : 32, NT = TC * L / E;
+    // the registers allow 768 threads of 80 (with two blocks of 256 of them at 124 registers
+    // the passes ran 15 % slower at 257^3)
+    static constexpr int BPS = 768 / NT;
+    static constexpr int LSM = TC <= 4 ? 2 : 1, LS = q_slot(L) + (LSM + 8 - q_slot(L) % 8) % 8;
+    static constexpr int Ph = L / 2, KS = Ph + 1;
     static constexpr int R0 = q_radix(L, 1, RM), TW = q_tw_count(L, RM);
     static constexpr size_t SMEM = sizeof(qc) * (TC * LS + TW) + sizeof(int2) * TC * KS;
 };
@@ -39,10 +50,11 @@ __device__ __forceinline__ void cp_async8(void *dst, const void *src)
 }
 
 template <int L>
-__global__ void __launch_bounds__(FaceQCfg<L>::NT, 2) face_q_kernel(const FaceQPass a)
+__global__ void __launch_bounds__(FaceQCfg<L>::NT, FaceQCfg<L>::BPS) face_q_kernel(const FaceQPass a)
 {
     using Cfg = FaceQCfg<L>;
-    constexpr int TC = Cfg::TC, NT = Cfg::NT, LS = Cfg::LS, KS = Cfg::KS, U = Cfg::U, Ph = Cfg::Ph, R0 = Cfg::R0;
+    constexpr int TC = Cfg::TC, NT = Cfg::NT, LS = Cfg::LS, KS = Cfg::KS, Ph = Cfg::Ph, R0 = Cfg::R0;
+    constexpr int RL = Cfg::RL, UL = Cfg::UL, IL = Cfg::IL;
     extern __shared__ qc smem_q[];
     qc *buf = smem_q;
     int4 *tws = reinterpret_cast<int4 *>(buf + TC * LS);
@@ -55,11 +67,14 @@ __global__ void __launch_bounds__(FaceQCfg<L>::NT, 2) face_q_kernel(const FaceQP
     for (int f = threadIdx.x; f < Cfg::TW; f += NT) tws[f] = __ldg(a.q + f);
     const int2 *kq = a.kq + ((int64_t)diff * npair * a.nc + c0) * KS;
 
-    // the unit of the last pass: column ct, frequencies j + q U
-    const int ct = threadIdx.x / U, j = threadIdx.x - ct * U;
-    qc acc[8];
+    // a unit of the last pass: column, frequencies j + q UL
+    auto column = [](int it) { return (int)(threadIdx.x + it * NT) / UL; };
+    auto freq = [](int it) { return (int)(threadIdx.x + it * NT) % UL; };
+    qc acc[IL][RL];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) acc[q] = qc{0, 0};
+    for (int it = 0; it < IL; ++it)
+#pragma unroll
+        for (int q = 0; q < RL; ++q) acc[it][q] = qc{0, 0};
 
     for (int pr = chunk; pr < npair; pr += a.nchunk) {
         const int p2 = a.np - 1 - pr;
@@ -74,7 +89,7 @@ __global__ void __launch_bounds__(FaceQCfg<L>::NT, 2) face_q_kernel(const FaceQP
         // the first pass (radix R0, no factors) on the load: data at positions 1..Mb-1 of
         // a column, zeros elsewhere, in particular from L / 2 on
         {
-            constexpr int U0 = L / R0, NZ = R0 == 3 ? 2 : R0 / 2;   // units, inputs that can be non-zero
+            constexpr int U0 = L / R0, NZ = R0 / 2;   // units, inputs that can be non-zero
             const double2 *x1 = a.D + (int64_t)pr * a.sp + (int64_t)c0 * a.sc;
             const double2 *x2 = a.D + (int64_t)p2 * a.sp + (int64_t)c0 * a.sc;
 #pragma unroll 2
@@ -106,34 +121,39 @@ __global__ void __launch_bounds__(FaceQCfg<L>::NT, 2) face_q_kernel(const FaceQP
             }
         }
         __syncthreads();
-        q_fft<L, Cfg::RM, TC, NT, LS, R0, false, U>(buf, tws);
+        q_fft<L, Cfg::RM, TC, NT, LS, R0, false, UL>(buf, tws);
         // the last pass, its outputs times the spectra
         asm volatile("cp.async.wait_all;\n" ::: "memory");
         __syncthreads();
-        {
-            const qc *x = buf + ct * LS;
-            const int4 *tw = tws + (Cfg::TW - 7 * U);
-            qc v[8];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) v[q] = x[q_slot(j + q * U)];
+        for (int it = 0; it < IL; ++it) {
+            const int ct = column(it), j = freq(it);
+            const qc *x = buf + ct * LS + q_slot(j);
+            const int4 *tw = tws + (Cfg::TW - (RL - 1) * UL) + j;
+            qc v[RL];
 #pragma unroll
-            for (int q = 1; q < 8; ++q) v[q] = q_cmul(v[q], tw[(q - 1) * U + j]);
-            q_dft8(v);
+            for (int q = 0; q < RL; ++q) v[q] = x[UL % 8 == 0 ? q_slot(q * UL) : q_slot(j + q * UL) - q_slot(j)];
+#pragma unroll
+            for (int q = 1; q < RL; ++q) v[q] = q_cmul(v[q], tw[(q - 1) * UL]);
+            q_dft<RL>(v);
             const int2 *k = ks + ct * KS;
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const int m = j + q * U;
+            for (int q = 0; q < RL; ++q) {
+                const int m = j + q * UL;
                 const int2 w = k[m <= Ph ? m : L - m];
-                acc[q].re += q_rmul(v[q].re, w.x, w.y);
-                acc[q].im += q_rmul(v[q].im, w.x, w.y);
+                acc[it][q].re += q_rmul(v[q].re, w.x, w.y);
+                acc[it][q].im += q_rmul(v[q].im, w.x, w.y);
             }
         }
         __syncthreads();   // the buffer is free
     }
-    if (ct < ncl) {
-        qc *part = a.part + (((int64_t)chunk * 2 + diff) * a.nc + c0 + ct) * L;
 #pragma unroll
-        for (int q = 0; q < 8; ++q) part[j + q * U] = acc[q];
+    for (int it = 0; it < IL; ++it) {
+        const int ct = column(it);
+        if (ct >= ncl) continue;
+        qc *part = a.part + (((int64_t)chunk * 2 + diff) * a.nc + c0 + ct) * L + freq(it);
+#pragma unroll
+        for (int q = 0; q < RL; ++q) part[q * UL] = acc[it][q];
     }
 }
 
@@ -208,6 +228,11 @@ cudaError_t launch_face_kq(const double *khat, int np, int64_t per, int2 *kq, in
 int face_q_columns(int L)
 {
     IDP_FACE_SWITCH(L, return FaceQCfg<L>::TC;)
+}
+
+int face_q_blocks_per_sm(int L)
+{
+    IDP_FACE_SWITCH(L, return FaceQCfg<L>::BPS;)
 }
 
 }  // namespace idp

@@ -194,7 +194,8 @@ struct FaceQPass {
 cudaError_t launch_face_q(const FaceQPass &a, cudaStream_t st);
 cudaError_t launch_face_kq(const double *khat, int np, int64_t per, int2 *kq, int *ek, cudaStream_t st);
 cudaError_t face_q_set_attributes();
-int face_q_columns(int L);   // frequencies c per block
+int face_q_columns(int L);        // frequencies c per block
+int face_q_blocks_per_sm(int L);  // resident blocks per SM
 
 // 2-D contraction: part[0/1][m] = sum_p khat[p or np-1-p][m] * T[p][m]
 struct FacePass2D {

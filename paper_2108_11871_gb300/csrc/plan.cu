@@ -1521,9 +1521,10 @@ int plan_setup(idp_plan p)
             p->pchunk[a_] = pch;
             pmax = std::max<int64_t>(pmax, (int64_t)nch * 2 * L * (Mc + 1));
             const int npair = (np + 1) / 2;
-            // one wave of two blocks per SM, and at most 64 pairs per block
+            // three waves of resident blocks, at least 8 pairs a block
             const int qtiles = 2 * ((Mc + face_q_columns(L)) / face_q_columns(L));
-            p->qchunk[a_] = face_q_chunks(np, std::max(2 * nsm / qtiles, npair / 64));
+            const int qslots = face_q_blocks_per_sm(L) * nsm;
+            p->qchunk[a_] = face_q_chunks(np, std::max(std::min(3 * qslots / qtiles, npair / 8), qslots / qtiles));
             pmax = std::max<int64_t>(pmax, (int64_t)p->qchunk[a_] * 2 * L * (Mc + 1));
             fmax = std::max<int64_t>(fmax, (int64_t)2 * (Mb + 1) * (Mc + 1));
             const int64_t per = (int64_t)(Mb + 1) * (Mc + 1);
@@ -1612,7 +1613,8 @@ int autotune(idp_plan p)
             cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, p->dev);
             const int tiles = 2 * ((nc + face_q_columns(L) - 1) / face_q_columns(L));
             std::vector<int> cands = {n0, face_q_chunks(p->ni[a_], n0 / 2), face_q_chunks(p->ni[a_], 2 * n0)};
-            for (int w = 1; w <= 6; ++w) cands.push_back(face_q_chunks(p->ni[a_], w * 2 * nsm / tiles));
+            for (int w = 1; w <= 4; ++w)
+                cands.push_back(face_q_chunks(p->ni[a_], w * face_q_blocks_per_sm(L) * nsm / tiles));
             float best_t = 1e30f;
             for (size_t i = 0; i < cands.size() && !rc; ++i) {
                 if (std::find(cands.begin(), cands.begin() + i, cands[i]) != cands.begin() + i) continue;

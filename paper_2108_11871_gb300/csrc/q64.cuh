@@ -67,15 +67,25 @@ __device__ __forceinline__ void q_dft2(qc *v)
     v[0] = q_add(a, v[1]);
     v[1] = q_sub(a, v[1]);
 }
-__device__ __forceinline__ void q_dft3(qc *v)
+__device__ __forceinline__ void q_dft3(qc &a0, qc &a1, qc &a2)
 {
-    const qc t = q_add(v[1], v[2]), d = q_sub(v[1], v[2]);
+    const qc t = q_add(a1, a2), d = q_sub(a1, a2);
     // t / 2, an odd t rounded up or down by the last bit of another value (no bias)
-    const qc m = qc{v[0].re - ((t.re + (v[0].re & 1)) >> 1), v[0].im - ((t.im + (v[0].im & 1)) >> 1)};
+    const qc m = qc{a0.re - ((t.re + (a0.re & 1)) >> 1), a0.im - ((t.im + (a0.im & 1)) >> 1)};
     const long long pr = q_rmul(d.im, Q_S3H, Q_S3L), pi = q_rmul(d.re, Q_S3H, Q_S3L);
-    v[0] = q_add(v[0], t);
-    v[1] = qc{m.re + pr, m.im - pi};
-    v[2] = qc{m.re - pr, m.im + pi};
+    a0 = q_add(a0, t);
+    a1 = qc{m.re + pr, m.im - pi};
+    a2 = qc{m.re - pr, m.im + pi};
+}
+// 6 = 2 * 3 by the residues (x_{3a+2b} -> X_{3c+4d}): two 3-point transforms, no factors
+__device__ __forceinline__ void q_dft6(qc *v)
+{
+    qc s0 = q_add(v[0], v[3]), s1 = q_add(v[2], v[5]), s2 = q_add(v[4], v[1]);
+    qc d0 = q_sub(v[0], v[3]), d1 = q_sub(v[2], v[5]), d2 = q_sub(v[4], v[1]);
+    q_dft3(s0, s1, s2);
+    q_dft3(d0, d1, d2);
+    v[0] = s0; v[4] = s1; v[2] = s2;
+    v[3] = d0; v[1] = d1; v[5] = d2;
 }
 __device__ __forceinline__ void q_dft4(qc &a0, qc &a1, qc &a2, qc &a3)
 {
@@ -107,7 +117,8 @@ template <int R>
 __device__ __forceinline__ void q_dft(qc *v)
 {
     if constexpr (R == 2) q_dft2(v);
-    else if constexpr (R == 3) q_dft3(v);
+    else if constexpr (R == 3) q_dft3(v[0], v[1], v[2]);
+    else if constexpr (R == 6) q_dft6(v);
     else if constexpr (R == 4) q_dft4(v[0], v[1], v[2], v[3]);
     else q_dft8(v);
 }
@@ -120,18 +131,28 @@ __device__ __forceinline__ void q_dft(qc *v)
 __host__ __device__ constexpr int q_slot(int e) { return e + (e >> 3); }
 __host__ __device__ constexpr int q_line(int L) { return q_slot(L) | 1; }
 
-// The radices of the passes of length L after a span of Ns: one radix-3 pass first for
-// 3 * 2^m, then radix-4 (or radix-2) until a power of RM (4 or 8) is left, then RM.
+// The radix of the pass of length L after a span of Ns, RM = 4 or 8.
+//   2^m:     a radix-4 pass (RM = 4: radix-2) first where 2^m is no power of RM, then radix
+//            RM, and for 2^m = 2 * 8^i a last radix-4 pass (two radix-4 passes in a row
+//            would write two elements to one bank group)
+//   3 * 2^m: the same with a last pass of radix 3, or 6 for 2^m = 2 * RM^i (radix 3 first
+//            has no factors, but costs a radix-8 pass that has none and leaves spans that are
+//            no powers of two: 193^3 with radix 3 first, face passes 640 us per solve, sine passes 442;
+//            with it last 503 and 354)
 __host__ __device__ constexpr int q_radix(int L, int Ns, int RM)
 {
-    const int rest = L / Ns;
-    if (rest % 3 == 0) return 3;
+    const int rest = L / Ns, three = L % 3 == 0 ? 3 : 1, two = rest / three;   // 2^m left
     int p = 1;
-    while (p * RM <= rest) p *= RM;
-    const int head = rest / p;
-    if (head == 4) return 4;
-    if (head == 2) return RM == 8 && rest >= 16 ? 4 : 2;   // 16 = 4 * 4, 128 = 4 * 4 * 8
-    return RM;
+    while (p * RM <= two) p *= RM;
+    const int head = two / p;   // 1, 2 or 4
+    if (three == 3) {
+        if (two <= 2) return three * two;
+        return head == 4 && Ns == 1 ? 4 : RM;
+    }
+    if (rest <= RM) return rest;
+    if (Ns > 1 && RM == 8) return 8;
+    if (head == 1) return RM;
+    return RM == 8 ? 4 : 2;
 }
 // entries of the factor table of length L, from span Ns on
 __host__ __device__ constexpr int q_tw_count(int L, int RM, int Ns = 1)
