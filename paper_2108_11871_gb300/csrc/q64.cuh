@@ -22,8 +22,18 @@ struct __align__(16) qc {
     long long re, im;
 };
 
-__device__ __forceinline__ long long q_mulw(int a, int b) { return (long long)a * b; }
-__device__ __forceinline__ long long q_madw(int a, int b, long long c) { return (long long)a * b + c; }
+__device__ __forceinline__ long long q_mulw(int a, int b)
+{
+    long long d;
+    asm("mul.wide.s32 %0, %1, %2;" : "=l"(d) : "r"(a), "r"(b));
+    return d;
+}
+__device__ __forceinline__ long long q_madw(int a, int b, long long c)
+{
+    long long d;
+    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+    return d;
+}
 
 __device__ __forceinline__ qc q_add(qc a, qc b) { return qc{a.re + b.re, a.im + b.im}; }
 __device__ __forceinline__ qc q_sub(qc a, qc b) { return qc{a.re - b.re, a.im - b.im}; }
