@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(Cfg::T, Cfg::BPS) dst_pass_kernel(const DstPas
     extern __shared__ qc smem_q[];
     qc *buf = smem_q;
     int4 *tabs = reinterpret_cast<int4 *>(buf + Cfg::BUF);
-    __shared__ int s_high[LB], s_scale[LB];
+    __shared__ int s_high[LB], s_scale[LB], s_gmax;
     __shared__ unsigned s_sum[LB];
     // the tables, made with the plan, come in while the previous launch drains (they are
     // visible after the first barrier)
@@ -70,6 +70,7 @@ __global__ void __launch_bounds__(Cfg::T, Cfg::BPS) dst_pass_kernel(const DstPas
     {
         for (int i = threadIdx.x; i < Cfg::TAB; i += NT) tabs[i] = __ldg(a.qtab + i);
     }
+    if (threadIdx.x == 0) s_gmax = 0;
     if (threadIdx.x < LB) {
         s_high[threadIdx.x] = 0;
         s_sum[threadIdx.x] = 0;
@@ -128,8 +129,11 @@ __global__ void __launch_bounds__(Cfg::T, Cfg::BPS) dst_pass_kernel(const DstPas
     for (int d = d0; d < d1; d <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
     if (lead) atomicAdd(&s_sum[l], sum);
     __syncthreads();
-    const int scale = 1101 - emax - q_bits(s_sum[l]);   // absolute sum below 2^58 units
-    if (g == 0) s_scale[l] = emax == 0x7ff ? Q_NAN : scale;
+    const int eb = emax + q_bits(s_sum[l]), scale = 1101 - eb;   // absolute sum below 2^58 units
+    if (g == 0) {
+        s_scale[l] = emax == 0x7ff ? Q_NAN : scale;
+        if (a.gmax && l < nl) atomicMax(&s_gmax, emax == 0x7ff ? Q_GNAN : eb);
+    }
 
     // 3. pre-processing into buf viewed as y'[LB][M] (y'_j in component j mod 2 of
     //    element j / 2): y'_j = sin(pi j/M) (2 x_j + 2 x_{M-j}) + (x_j - x_{M-j})
@@ -150,6 +154,8 @@ __global__ void __launch_bounds__(Cfg::T, Cfg::BPS) dst_pass_kernel(const DstPas
         }
     }
     __syncthreads();
+
+    if (a.gmax && threadIdx.x == 0 && *a.gmax < s_gmax) atomicMax(a.gmax, s_gmax);
 
     // 4. complex FFT of length K
     q_fft<K, RM, LB, NT, LS>(buf, tabs);

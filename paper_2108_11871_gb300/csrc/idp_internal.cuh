@@ -53,6 +53,8 @@ struct DstPass {
     // length K = M/2 pass by pass, e^{-i pi k/K} (k = 0..K/2), sin(pi j/M) (j = 0..K-1)
     const int4 *qtab;
     int in_dd;             // the input holds double-float pairs
+    int *gmax;             // optional (fixed-point passes): maximum over the lines of emax + bits (q64.cuh), which
+                           // bounds every output by 2^(gmax - 1041); zero on entry
     int lines;   // lines per block: 0 = by size, 8 = fewest, 16, 32 = most
     // double-float variant (dd = 1): arithmetic on the FP32 pipe; in/out/add
     // may hold FP64 values or double-float pairs (in_dd / out_dd / add_dd)
@@ -285,10 +287,20 @@ cudaError_t launch_gtilde_expand(const Grid3 &g, const double *Q0, const double 
                                  const double *sin4, const double *tab, const double *add, double *out,
                                  cudaStream_t st, const double *tab2 = nullptr, const double *add2 = nullptr,
                                  double *out2 = nullptr, int fold = 0, const double *ascale = nullptr);
+// The same (add2 null: out only) and rhs6_e_expand from layers in fixed point
+// (launch_layers_combine with gmax): gmax as there, sq / sq2: sin(pi (k+1)/M_s) and
+// sin(2 pi (k+1)/M_s) per active axis as fixed-point factors (q64.cuh)
+cudaError_t launch_gtilde_expand_q(const Grid3 &g, const double *Q0, const double *Q1, const double *Q2,
+                                   const int2 *sq, const int *gmax, const double *tab, const double *add, double *out,
+                                   const double *tab2, const double *add2, double *out2, cudaStream_t st);
+cudaError_t launch_rhs6_e_expand_q(const Grid3 &g, const double *E0, const double *E1, const double *E2,
+                                   const int2 *sq, const int2 *sq2, const int *gmax, const double *tab, double *out,
+                                   cudaStream_t st);
 // (a, b) -> (a + b, a - b) for the pairs of transformed layers at the two faces of
-// an axis: part i holds [2][nl][pl_i] (pl_i = 0: absent)
+// an axis: part i holds [2][nl][pl_i] (pl_i = 0: absent); with gmax (DstPass::gmax of the
+// passes that made them) the results are 64-bit integers in units of 2^(gmax - 1100)
 cudaError_t launch_layers_combine(double *P0, int64_t pl0, double *P1, int64_t pl1, double *P2, int64_t pl2,
-                                  int nl, cudaStream_t st);
+                                  int nl, cudaStream_t st, const int *gmax = nullptr);
 cudaError_t launch_gtilde_scatter(const Grid3 &g, const double *Q0, const double *Q1, const double *Q2,
                                   double *out, cudaStream_t st);
 // W_s = sum_{r != s} a_sr (u(+e_r) + u(-e_r) - 2u) on nodes; W is 3 node arrays (2 for d = 2).

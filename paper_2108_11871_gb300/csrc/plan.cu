@@ -248,7 +248,9 @@ struct idp_plan_s {
     int2 *kq[3] = {nullptr, nullptr, nullptr};   // fixed-point spectra (FaceQPass) and their exponents
     int *kq_ek[3] = {nullptr, nullptr, nullptr};
     int qchunk[3] = {1, 1, 1};        // chunks of pairs of slices of the fixed-point face passes
-    int *gmax[2] = {nullptr, nullptr};   // bounds of the lines along axes 2 and 1 (FaceQPass::gmax)
+    int *gmax[4] = {};                // bounds of the lines along axes 2 and 1 (FaceQPass::gmax), of the layers
+                                      // of gtilde and of E; zeroed with the flags
+    int2 *sinq = nullptr, *sinq2 = nullptr;   // fixed-point forms of sin4 / 4 and sin4b / 4
     int nchunk[3] = {1, 1, 1}, pchunk[3] = {1, 1, 1};
     int dst_lines = 0;                // lines per block of the full-volume sine passes (0 = default)
 
@@ -817,9 +819,18 @@ int transform(idp_plan p, View3 in, double *work, View3 out, const double *tab, 
     return IDP_OK;
 }
 
+// The transformed layers as fixed-point numbers and their expansions in integers: where every
+// sine pass of the layers is a fixed-point one (its bound sets the scale)
+bool layers_fx(idp_plan p)
+{
+    bool fx = !tensor_mode(p);
+    for (int s = 0; s < 3; ++s) fx = fx && (!p->act[s] || has_fft_dst(p->M[s]));
+    return fx;
+}
+
 // in-place sine passes over a dense box b0 x b1 x b2 along axis 2, then axis 1
 // (if M1 > 0), with panel counts M2 / M1
-int dst_box(idp_plan p, double *x, int b0, int b1, int b2, int M2, int M1, cudaStream_t st)
+int dst_box(idp_plan p, double *x, int b0, int b1, int b2, int M2, int M1, cudaStream_t st, int *gmax)
 {
     const int axes[2] = {2, 1};
     const int Ms[2] = {M2, M1};
@@ -831,6 +842,7 @@ int dst_box(idp_plan p, double *x, int b0, int b1, int b2, int M2, int M1, cudaS
         a.n0 = b0; a.n1 = b1; a.n2 = b2;
         a.axis = axes[q];
         a.M = Ms[q];
+        a.gmax = q == 1 || Ms[1] <= 0 ? gmax : nullptr;   // the last pass
         FftTables t{};
         int rc;
         const bool ddm = p->mixed == IDP_PRECISION_DF32 || tensor_mode(p);
@@ -861,21 +873,22 @@ int gtilde_parts(idp_plan p, bool transform_parts, cudaStream_t st)
     }
     if (!transform_parts) return IDP_OK;
     int rc;
+    int *gm = layers_fx(p) ? p->gmax[2] : nullptr;
     const int n0 = p->ni[0], n1 = p->ni[1], n2 = p->ni[2];
     if (p->d == 3 && n0 == n1 && n1 == n2) {
         // equal shapes: the three parts form one box of 6 layers
-        if ((rc = dst_box(p, p->Q0, 6, n1, n2, p->M[2], p->M[1], st))) return rc;
+        if ((rc = dst_box(p, p->Q0, 6, n1, n2, p->M[2], p->M[1], st, gm))) return rc;
     } else if (p->d == 3) {
-        if ((rc = dst_box(p, p->Q0, 2, n1, n2, p->M[2], p->M[1], st))) return rc;
-        if ((rc = dst_box(p, p->Q1, 2, n0, n2, p->M[2], p->M[0], st))) return rc;
-        if ((rc = dst_box(p, p->Q2, 2, n0, n1, p->M[1], p->M[0], st))) return rc;
+        if ((rc = dst_box(p, p->Q0, 2, n1, n2, p->M[2], p->M[1], st, gm))) return rc;
+        if ((rc = dst_box(p, p->Q1, 2, n0, n2, p->M[2], p->M[0], st, gm))) return rc;
+        if ((rc = dst_box(p, p->Q2, 2, n0, n1, p->M[1], p->M[0], st, gm))) return rc;
     } else {
-        if ((rc = dst_box(p, p->Q1, 2, 1, n2, p->M[2], 0, st))) return rc;
-        if ((rc = dst_box(p, p->Q2, 2, 1, n1, p->M[1], 0, st))) return rc;
+        if ((rc = dst_box(p, p->Q1, 2, 1, n2, p->M[2], 0, st, gm))) return rc;
+        if ((rc = dst_box(p, p->Q2, 2, 1, n1, p->M[1], 0, st, gm))) return rc;
     }
     Mark mk(p, IDP_KERNEL_GTILDE, st);
     IDP_CK(launch_layers_combine(p->Q0, p->d == 3 ? (int64_t)n1 * n2 : 0, p->Q1, (int64_t)n0 * n2, p->Q2,
-                                 (int64_t)n0 * n1, 1, st));
+                                 (int64_t)n0 * n1, 1, st, gm));
     return IDP_OK;
 }
 
@@ -883,20 +896,21 @@ int gtilde_parts(idp_plan p, bool transform_parts, cudaStream_t st)
 int e_layers(idp_plan p, cudaStream_t st)
 {
     int rc;
+    int *gm = layers_fx(p) ? p->gmax[3] : nullptr;
     const int n0 = p->ni[0], n1 = p->ni[1], n2 = p->ni[2];
     if (p->d == 3 && n0 == n1 && n1 == n2) {
-        if ((rc = dst_box(p, p->E0, 12, n1, n2, p->M[2], p->M[1], st))) return rc;
+        if ((rc = dst_box(p, p->E0, 12, n1, n2, p->M[2], p->M[1], st, gm))) return rc;
     } else if (p->d == 3) {
-        if ((rc = dst_box(p, p->E0, 4, n1, n2, p->M[2], p->M[1], st))) return rc;
-        if ((rc = dst_box(p, p->E1, 4, n0, n2, p->M[2], p->M[0], st))) return rc;
-        if ((rc = dst_box(p, p->E2, 4, n0, n1, p->M[1], p->M[0], st))) return rc;
+        if ((rc = dst_box(p, p->E0, 4, n1, n2, p->M[2], p->M[1], st, gm))) return rc;
+        if ((rc = dst_box(p, p->E1, 4, n0, n2, p->M[2], p->M[0], st, gm))) return rc;
+        if ((rc = dst_box(p, p->E2, 4, n0, n1, p->M[1], p->M[0], st, gm))) return rc;
     } else {
-        if ((rc = dst_box(p, p->E1, 4, 1, n2, p->M[2], 0, st))) return rc;
-        if ((rc = dst_box(p, p->E2, 4, 1, n1, p->M[1], 0, st))) return rc;
+        if ((rc = dst_box(p, p->E1, 4, 1, n2, p->M[2], 0, st, gm))) return rc;
+        if ((rc = dst_box(p, p->E2, 4, 1, n1, p->M[1], 0, st, gm))) return rc;
     }
     Mark mk(p, IDP_KERNEL_RHS6_EXPAND, st);
     IDP_CK(launch_layers_combine(p->E0, p->d == 3 ? (int64_t)n1 * n2 : 0, p->E1, (int64_t)n0 * n2, p->E2,
-                                 (int64_t)n0 * n1, 2, st));
+                                 (int64_t)n0 * n1, 2, st, gm));
     return IDP_OK;
 }
 
@@ -1274,8 +1288,10 @@ int enqueue_grid(idp_plan p, const double *rho, double *phi, int stop, cudaStrea
         // A += tab4 * S gtilde; phi = S A inside
         {
             Mark mk(p, IDP_KERNEL_GTILDE_EXPAND, st);
-            IDP_CK(launch_gtilde_expand(p->grid, p->Q0, p->Q1, p->Q2, p->sin4, p->tab4, p->A, p->A, st, nullptr,
-                                        nullptr, nullptr, 0, ascale));
+            IDP_CK(layers_fx(p) ? launch_gtilde_expand_q(p->grid, p->Q0, p->Q1, p->Q2, p->sinq, p->gmax[2], p->tab4,
+                                                         p->A, p->A, nullptr, nullptr, nullptr, st)
+                                : launch_gtilde_expand(p->grid, p->Q0, p->Q1, p->Q2, p->sin4, p->tab4, p->A, p->A,
+                                                       st, nullptr, nullptr, nullptr, 0, ascale));
         }
         return transform(p, dense(p, p->A), p->A, node_interior(p, phi), nullptr, none, false, st);
     }
@@ -1285,8 +1301,11 @@ int enqueue_grid(idp_plan p, const double *rho, double *phi, int stop, cudaStrea
     // the final transform takes u1 in C (S C + S B = S (C + B)), in every mode
     {
         Mark mk(p, IDP_KERNEL_GTILDE_EXPAND, st);
-        IDP_CK(launch_gtilde_expand(p->grid, p->Q0, p->Q1, p->Q2, p->sin4, p->tab4, nullptr, p->B, st,
-                                    p->tabR, p->A, stop == 0 ? p->C : nullptr, 1, ascale));
+        double *C = stop == 0 ? p->C : nullptr;
+        IDP_CK(layers_fx(p) ? launch_gtilde_expand_q(p->grid, p->Q0, p->Q1, p->Q2, p->sinq, p->gmax[2], p->tab4,
+                                                     nullptr, p->B, p->tabR, p->A, C, st)
+                            : launch_gtilde_expand(p->grid, p->Q0, p->Q1, p->Q2, p->sin4, p->tab4, nullptr, p->B,
+                                                   st, p->tabR, p->A, C, 1, ascale));
     }
     // u1 feeds the sixth differences of R, which amplify its rounding by ~1e4-1e7:
     // this inverse transform stays FP64 in the FP64 and DF32 modes, and is a
@@ -1317,7 +1336,10 @@ int enqueue_grid(idp_plan p, const double *rho, double *phi, int stop, cudaStrea
         // dense interior array
         {
             Mark mk(p, IDP_KERNEL_GTILDE_EXPAND, st);
-            IDP_CK(launch_gtilde_expand(p->grid, p->Q0, p->Q1, p->Q2, p->sin4, p->tab4, nullptr, p->C, st));
+            IDP_CK(layers_fx(p) ? launch_gtilde_expand_q(p->grid, p->Q0, p->Q1, p->Q2, p->sinq, p->gmax[2], p->tab4,
+                                                         nullptr, p->C, nullptr, nullptr, nullptr, st)
+                                : launch_gtilde_expand(p->grid, p->Q0, p->Q1, p->Q2, p->sin4, p->tab4, nullptr,
+                                                       p->C, st));
         }
         IDP_CK(launch_rhs6_symbol(p->grid, p->ld, p->ldoff[1], p->ldoff[2], p->C, st));
         if ((rc = transform(p, dense(p, p->C), p->C, dense(p, phi), nullptr, none, false, st, false))) return rc;
@@ -1328,7 +1350,10 @@ int enqueue_grid(idp_plan p, const double *rho, double *phi, int stop, cudaStrea
     if ((rc = e_layers(p, st))) return rc;
     {
         Mark mk(p, IDP_KERNEL_RHS6_EXPAND, st);
-        IDP_CK(launch_rhs6_e_expand(p->grid, p->E0, p->E1, p->E2, p->sin4, p->sin4b, p->tab4, p->C, st));
+        IDP_CK(layers_fx(p) ? launch_rhs6_e_expand_q(p->grid, p->E0, p->E1, p->E2, p->sinq, p->sinq2, p->gmax[3],
+                                                     p->tab4, p->C, st)
+                            : launch_rhs6_e_expand(p->grid, p->E0, p->E1, p->E2, p->sin4, p->sin4b, p->tab4, p->C,
+                                                   st));
     }
     return transform(p, dense(p, p->C), p->C, node_interior(p, phi), nullptr, none, false, st);
 }
@@ -1405,7 +1430,7 @@ int plan_setup(idp_plan p)
     }
     {
         const int64_t n0 = p->ni[0], n1 = p->ni[1], n2 = p->ni[2];
-        p->nflags = n0 * n1 + n0 * n2 + n0 + n1 + n2 + 2;
+        p->nflags = n0 * n1 + n0 * n2 + n0 + n1 + n2 + 4;
         if ((rc = p->alloc(&p->flags, p->nflags))) return rc;
         p->row2 = p->flags;
         p->row1 = p->row2 + n0 * n1;
@@ -1413,7 +1438,7 @@ int plan_setup(idp_plan p)
         p->sl[1] = p->sl[0] + n0;
         p->sl[2] = p->sl[1] + n1;
         p->gmax[0] = p->sl[2] + n2;
-        p->gmax[1] = p->gmax[0] + 1;
+        for (int i = 1; i < 4; ++i) p->gmax[i] = p->gmax[0] + i;
     }
     if ((rc = plan_streams(p))) return rc;
     {
@@ -1431,6 +1456,19 @@ int plan_setup(idp_plan p)
         }
         if ((rc = p->alloc(&p->sin4b, (int64_t)s4b.size()))) return rc;
         IDP_CK(cudaMemcpy(p->sin4b, s4b.data(), sizeof(double) * s4b.size(), cudaMemcpyHostToDevice));
+        std::vector<int2> sq;
+        for (int m = 1; m <= 2; ++m)
+            for (int s = 0; s < 3; ++s) {
+                if (!p->act[s]) continue;
+                for (int k = 0; k < p->ni[s]; ++k) {
+                    long double c, sn;
+                    cossinpi((int64_t)m * (k + 1), p->M[s], c, sn);
+                    sq.push_back(fixed_factor(sn));
+                }
+            }
+        if ((rc = p->alloc(&p->sinq, (int64_t)sq.size()))) return rc;
+        IDP_CK(cudaMemcpy(p->sinq, sq.data(), sizeof(int2) * sq.size(), cudaMemcpyHostToDevice));
+        p->sinq2 = p->sinq + s4.size();
     }
     {
         // layers of E (two per face): E0 [2][2][n1][n2] (3-D), E1 [2][2][n0][n2], E2 [2][2][n0][n1]

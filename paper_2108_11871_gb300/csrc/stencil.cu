@@ -5,6 +5,7 @@
 // axes 1, 2.  Interior arrays are dense over the interior nodes.
 #include "dd.cuh"
 #include "idp_internal.cuh"
+#include "q64.cuh"
 
 namespace idp {
 
@@ -575,8 +576,11 @@ __global__ void rhs6_e_kernel(const Grid3 gg, const StencilCoef c, const double 
 // b at (nl + l)*pl of each part): (a, b) -> (a + b, a - b), the two sign patterns
 // of sin(pi m j / M) and sin(pi m (M - j) / M) = (-1)^(m+1) sin(pi m j / M).
 __global__ void layers_combine_kernel(double *__restrict__ P0, int pl0, double *__restrict__ P1, int pl1,
-                                      double *__restrict__ P2, int pl2, int nl)
+                                      double *__restrict__ P2, int pl2, int nl, const int *__restrict__ gmax)
 {
+    // gmax: fixed-point results, |a +- b| < 2^(gmax - 1040), so below 2^60 units
+    const int gm = gmax ? min(*gmax, 2100) : 0;
+    const QFrom from(1100 - gm, gm - 31);
     // 32-bit index arithmetic: at most 2 * 3 * 511^2 entries
     const int tot = nl * (pl0 + pl1 + pl2);
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < tot; t += gridDim.x * blockDim.x) {
@@ -588,8 +592,14 @@ __global__ void layers_combine_kernel(double *__restrict__ P0, int pl0, double *
         const int l = q / pl;
         const int x = q - l * pl;
         const double av = P[l * pl + x], bv = P[(nl + l) * pl + x];
-        P[l * pl + x] = av + bv;
-        P[(nl + l) * pl + x] = av - bv;
+        if (gmax) {
+            long long *Pq = reinterpret_cast<long long *>(P);
+            Pq[l * pl + x] = from(av + bv);
+            Pq[(nl + l) * pl + x] = from(av - bv);
+        } else {
+            P[l * pl + x] = av + bv;
+            P[(nl + l) * pl + x] = av - bv;
+        }
     }
 }
 
@@ -627,6 +637,96 @@ __global__ void rhs6_e_expand_kernel(const Grid3 gg, const double *__restrict__ 
     }
     const int64_t t = k0 * g.is[0] + (int64_t)k1 * g.is[1] + k2;
     out[t] = fma(tab[t], v, out[t]);
+}
+
+// The two expansions from layers in fixed point (layers_combine with gmax): the sums over the
+// axes run in integers, so that the FP64 pipe, which bounded the kernels above (5 and 7
+// instructions a point: 1.71 and 1.59 ms at 513^3), has the conversion of the sum and the
+// products with the tables left (3 and 2): 0.95 and 0.80 ms.  A thread takes one (k1, k2) and
+// ck (even) consecutive k0: its two (four) values of the layers of axis 0 and the factors of
+// axes 1 and 2 stay in registers.  Eight k0 from 2^20 points on; below that two, which
+// leaves more threads (65^3: 3 us per solve).
+int expand_chunk(const Grid3 &g)
+{
+    return (int64_t)(g.d == 3 ? g.n0 : 1) * g.n1 * g.n2 >= (1 << 20) ? 8 : 2;
+}
+
+__device__ __forceinline__ QTo expand_to(const int *gmax)
+{
+    const int gm = *gmax;   // units of 2^(gmax - 1100), and a factor 4 = 4 sin / sin
+    return QTo(gm >= Q_GNAN ? Q_NAN : 1098 - gm);
+}
+
+__global__ void gtilde_expand_q_kernel(const Grid3 gg, const long long *__restrict__ Q0, const long long *__restrict__ Q1,
+                                       const long long *__restrict__ Q2, const int2 *__restrict__ sq,
+                                       const int *__restrict__ gmax, const double *__restrict__ tab, const double *add,
+                                       double *out, const double *__restrict__ tab2, const double *__restrict__ add2,
+                                       double *__restrict__ out2, int ck)
+{
+    const Geo g = make_geo(gg);
+    const int n0 = g.ni[0], n1 = g.ni[1], n2 = g.ni[2];
+    const int k2 = blockIdx.x * blockDim.x + threadIdx.x, k1 = blockIdx.y * blockDim.y + threadIdx.y;
+    if (k2 >= n2 || k1 >= n1) return;
+    const int k0 = blockIdx.z * ck, e0 = min(k0 + ck, n0);
+    const int a0 = g.act[0] ? n0 : 0;
+    const int2 s1 = sq[a0 + k1], s2 = sq[a0 + n1 + k2];
+    const QTo to = expand_to(gmax);
+    long long q0[2] = {0, 0};
+    if (g.act[0]) {
+        q0[0] = Q0[(int64_t)k1 * n2 + k2];
+        q0[1] = Q0[(int64_t)(n1 + k1) * n2 + k2];
+    }
+    const long long *q1 = Q1 + (int64_t)((k1 & 1) ? n0 + k0 : k0) * n2 + k2;
+    const long long *q2 = Q2 + (int64_t)((k2 & 1) ? n0 + k0 : k0) * n1 + k1;
+    int64_t t = k0 * g.is[0] + (int64_t)k1 * g.is[1] + k2;
+#pragma unroll 4
+    for (int k = k0; k < e0; ++k, q1 += n2, q2 += n1, t += g.is[0]) {
+        long long v = q_rmul(*q1, s1.x, s1.y) + q_rmul(*q2, s2.x, s2.y);
+        if (g.act[0]) {
+            const int2 s0 = sq[k];
+            v += q_rmul(q0[(k - k0) & 1], s0.x, s0.y);   // k0 is even
+        }
+        const double x = to(v), tb = tab[t];
+        out[t] = add ? fma(tb, x, add[t]) : tb * x;
+        if (out2) out2[t] = fma(tab2[t], x, add2[t]);
+    }
+}
+
+__global__ void rhs6_e_expand_q_kernel(const Grid3 gg, const long long *__restrict__ E0, const long long *__restrict__ E1,
+                                       const long long *__restrict__ E2, const int2 *__restrict__ sq,
+                                       const int2 *__restrict__ sq2, const int *__restrict__ gmax,
+                                       const double *__restrict__ tab, double *__restrict__ out, int ck)
+{
+    const Geo g = make_geo(gg);
+    const int n0 = g.ni[0], n1 = g.ni[1], n2 = g.ni[2];
+    const int k2 = blockIdx.x * blockDim.x + threadIdx.x, k1 = blockIdx.y * blockDim.y + threadIdx.y;
+    if (k2 >= n2 || k1 >= n1) return;
+    const int k0 = blockIdx.z * ck, e0 = min(k0 + ck, n0);
+    const int a0 = g.act[0] ? n0 : 0;
+    const int2 s1 = sq[a0 + k1], d1 = sq2[a0 + k1], s2 = sq[a0 + n1 + k2], d2 = sq2[a0 + n1 + k2];
+    const QTo to = expand_to(gmax);
+    long long q0[2] = {0, 0}, r0[2] = {0, 0};
+    if (g.act[0]) {
+        const int64_t pl = (int64_t)n1 * n2, o = (int64_t)k1 * n2 + k2;
+        q0[0] = E0[o];
+        r0[0] = E0[pl + o];
+        q0[1] = E0[2 * pl + o];
+        r0[1] = E0[3 * pl + o];
+    }
+    const int64_t p1 = (int64_t)n0 * n2, p2 = (int64_t)n0 * n1;
+    const long long *q1 = E1 + (int64_t)k0 * n2 + k2 + ((k1 & 1) ? 2 * p1 : 0);
+    const long long *q2 = E2 + (int64_t)k0 * n1 + k1 + ((k2 & 1) ? 2 * p2 : 0);
+    int64_t t = k0 * g.is[0] + (int64_t)k1 * g.is[1] + k2;
+#pragma unroll 4
+    for (int k = k0; k < e0; ++k, q1 += n2, q2 += n1, t += g.is[0]) {
+        long long v = q_rmul(q1[0], s1.x, s1.y) + q_rmul(q1[p1], d1.x, d1.y);
+        v += q_rmul(q2[0], s2.x, s2.y) + q_rmul(q2[p2], d2.x, d2.y);
+        if (g.act[0]) {
+            const int2 s0 = sq[k], d0 = sq2[k];
+            v += q_rmul(q0[(k - k0) & 1], s0.x, s0.y) + q_rmul(r0[(k - k0) & 1], d0.x, d0.y);
+        }
+        out[t] = fma(tab[t], to(v), out[t]);
+    }
 }
 
 // x(k) *= Lambda_R(k) (stage output only); ld: per-axis eigenvalues of D2_s,
@@ -819,10 +919,10 @@ cudaError_t launch_rhs6_spectral(const Grid3 &g, const StencilCoef &c, const dou
 }
 
 cudaError_t launch_layers_combine(double *P0, int64_t pl0, double *P1, int64_t pl1, double *P2, int64_t pl2,
-                                  int nl, cudaStream_t st)
+                                  int nl, cudaStream_t st, const int *gmax)
 {
     layers_combine_kernel<<<grid_for((int64_t)nl * (pl0 + pl1 + pl2)), 256, 0, st>>>(P0, (int)pl0, P1, (int)pl1, P2,
-                                                                                   (int)pl2, nl);
+                                                                                   (int)pl2, nl, gmax);
     return cudaGetLastError();
 }
 
@@ -832,6 +932,28 @@ cudaError_t launch_rhs6_e_expand(const Grid3 &g, const double *E0, const double 
 {
     rhs6_e_expand_kernel<<<grid3(g.n2 - 2, g.n1 - 2, g.d == 3 ? g.n0 - 2 : 1), dim3(32, 8), 0, st>>>(
         g, E0, E1, E2, sin4, sin4b, tab, out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_gtilde_expand_q(const Grid3 &g, const double *Q0, const double *Q1, const double *Q2,
+                                   const int2 *sq, const int *gmax, const double *tab, const double *add, double *out,
+                                   const double *tab2, const double *add2, double *out2, cudaStream_t st)
+{
+    const int n0 = g.d == 3 ? g.n0 - 2 : 1, ck = expand_chunk(g);
+    gtilde_expand_q_kernel<<<grid3(g.n2 - 2, g.n1 - 2, (n0 + ck - 1) / ck), dim3(32, 8), 0, st>>>(
+        g, reinterpret_cast<const long long *>(Q0), reinterpret_cast<const long long *>(Q1),
+        reinterpret_cast<const long long *>(Q2), sq, gmax, tab, add, out, tab2, add2, out2, ck);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_rhs6_e_expand_q(const Grid3 &g, const double *E0, const double *E1, const double *E2,
+                                   const int2 *sq, const int2 *sq2, const int *gmax, const double *tab, double *out,
+                                   cudaStream_t st)
+{
+    const int n0 = g.d == 3 ? g.n0 - 2 : 1, ck = expand_chunk(g);
+    rhs6_e_expand_q_kernel<<<grid3(g.n2 - 2, g.n1 - 2, (n0 + ck - 1) / ck), dim3(32, 8), 0, st>>>(
+        g, reinterpret_cast<const long long *>(E0), reinterpret_cast<const long long *>(E1),
+        reinterpret_cast<const long long *>(E2), sq, sq2, gmax, tab, out, ck);
     return cudaGetLastError();
 }
 
