@@ -864,28 +864,51 @@ int dst_box(idp_plan p, double *x, int b0, int b1, int b2, int M2, int M1, cudaS
     return IDP_OK;
 }
 
+// (d-1)-dimensional sine transforms of `nl` layers per axis.  Equal shapes form one box; else
+// each axis has its own box, and with conc they run beside each other on the plan's face
+// streams (each is one or two launches of a few microseconds that fill a part of the chip:
+// 33 x 65 x 97 has twelve of them per solve)
+int layer_transforms(idp_plan p, double *P0, double *P1, double *P2, int nl, cudaStream_t st, int *gm, bool conc)
+{
+    const int n0 = p->ni[0], n1 = p->ni[1], n2 = p->ni[2];
+    if (p->d == 3 && n0 == n1 && n1 == n2) return dst_box(p, P0, 3 * nl, n1, n2, p->M[2], p->M[1], st, gm);
+    const int nside = p->d == 3 ? 2 : 1;   // boxes on other streams
+    cudaStream_t s1 = st, s2 = st;
+    if (conc) {
+        s1 = p->fst[0];
+        if (nside == 2) s2 = p->fst[1];
+        IDP_CK(cudaEventRecord(p->fev[0], st));
+        for (int i = 0; i < nside; ++i) IDP_CK(cudaStreamWaitEvent(p->fst[i], p->fev[0], 0));
+    }
+    int rc;
+    if (p->d == 3) {
+        if ((rc = dst_box(p, P0, nl, n1, n2, p->M[2], p->M[1], st, gm))) return rc;
+        if ((rc = dst_box(p, P1, nl, n0, n2, p->M[2], p->M[0], s1, gm))) return rc;
+        if ((rc = dst_box(p, P2, nl, n0, n1, p->M[1], p->M[0], s2, gm))) return rc;
+    } else {
+        if ((rc = dst_box(p, P1, nl, 1, n2, p->M[2], 0, st, gm))) return rc;
+        if ((rc = dst_box(p, P2, nl, 1, n1, p->M[1], 0, s1, gm))) return rc;
+    }
+    if (conc)
+        for (int i = 0; i < nside; ++i) {
+            IDP_CK(cudaEventRecord(p->fev[1 + i], p->fst[i]));
+            IDP_CK(cudaStreamWaitEvent(st, p->fev[1 + i], 0));
+        }
+    return IDP_OK;
+}
+
 // gtilde parts Q0, Q1, Q2 and their (d-1)-dimensional sine transforms
-int gtilde_parts(idp_plan p, bool transform_parts, cudaStream_t st)
+int gtilde_parts(idp_plan p, bool transform_parts, cudaStream_t st, bool conc)
 {
     {
         Mark mk(p, IDP_KERNEL_GTILDE, st);
         IDP_CK(launch_gtilde_planes(p->grid, p->coef, p->U, p->Q0, p->Q1, p->Q2, st));
     }
     if (!transform_parts) return IDP_OK;
-    int rc;
     int *gm = layers_fx(p) ? p->gmax[2] : nullptr;
     const int n0 = p->ni[0], n1 = p->ni[1], n2 = p->ni[2];
-    if (p->d == 3 && n0 == n1 && n1 == n2) {
-        // equal shapes: the three parts form one box of 6 layers
-        if ((rc = dst_box(p, p->Q0, 6, n1, n2, p->M[2], p->M[1], st, gm))) return rc;
-    } else if (p->d == 3) {
-        if ((rc = dst_box(p, p->Q0, 2, n1, n2, p->M[2], p->M[1], st, gm))) return rc;
-        if ((rc = dst_box(p, p->Q1, 2, n0, n2, p->M[2], p->M[0], st, gm))) return rc;
-        if ((rc = dst_box(p, p->Q2, 2, n0, n1, p->M[1], p->M[0], st, gm))) return rc;
-    } else {
-        if ((rc = dst_box(p, p->Q1, 2, 1, n2, p->M[2], 0, st, gm))) return rc;
-        if ((rc = dst_box(p, p->Q2, 2, 1, n1, p->M[1], 0, st, gm))) return rc;
-    }
+    const int rc = layer_transforms(p, p->Q0, p->Q1, p->Q2, 2, st, gm, conc);
+    if (rc) return rc;
     Mark mk(p, IDP_KERNEL_GTILDE, st);
     IDP_CK(launch_layers_combine(p->Q0, p->d == 3 ? (int64_t)n1 * n2 : 0, p->Q1, (int64_t)n0 * n2, p->Q2,
                                  (int64_t)n0 * n1, 1, st, gm));
@@ -893,21 +916,12 @@ int gtilde_parts(idp_plan p, bool transform_parts, cudaStream_t st)
 }
 
 // (d-1)-dimensional sine transforms of the layers of E (two per face)
-int e_layers(idp_plan p, cudaStream_t st)
+int e_layers(idp_plan p, cudaStream_t st, bool conc)
 {
-    int rc;
     int *gm = layers_fx(p) ? p->gmax[3] : nullptr;
     const int n0 = p->ni[0], n1 = p->ni[1], n2 = p->ni[2];
-    if (p->d == 3 && n0 == n1 && n1 == n2) {
-        if ((rc = dst_box(p, p->E0, 12, n1, n2, p->M[2], p->M[1], st, gm))) return rc;
-    } else if (p->d == 3) {
-        if ((rc = dst_box(p, p->E0, 4, n1, n2, p->M[2], p->M[1], st, gm))) return rc;
-        if ((rc = dst_box(p, p->E1, 4, n0, n2, p->M[2], p->M[0], st, gm))) return rc;
-        if ((rc = dst_box(p, p->E2, 4, n0, n1, p->M[1], p->M[0], st, gm))) return rc;
-    } else {
-        if ((rc = dst_box(p, p->E1, 4, 1, n2, p->M[2], 0, st, gm))) return rc;
-        if ((rc = dst_box(p, p->E2, 4, 1, n1, p->M[1], 0, st, gm))) return rc;
-    }
+    const int rc = layer_transforms(p, p->E0, p->E1, p->E2, 4, st, gm, conc);
+    if (rc) return rc;
     Mark mk(p, IDP_KERNEL_RHS6_EXPAND, st);
     IDP_CK(launch_layers_combine(p->E0, p->d == 3 ? (int64_t)n1 * n2 : 0, p->E1, (int64_t)n0 * n2, p->E2,
                                  (int64_t)n0 * n1, 2, st, gm));
@@ -1269,7 +1283,7 @@ int enqueue_grid(idp_plan p, const double *rho, double *phi, int stop, cudaStrea
                        overlap_rho && rho_from_T0, rho_src)))
         return rc;
     // 2. gtilde on the boundary-adjacent layers, and the transforms of its parts
-    if ((rc = gtilde_parts(p, stop != IDP_STAGE_GTILDE, st))) return rc;
+    if ((rc = gtilde_parts(p, stop != IDP_STAGE_GTILDE, st, overlap_rho))) return rc;
     if (stop == IDP_STAGE_GTILDE) {
         IDP_CK(launch_gtilde_scatter(p->grid, p->Q0, p->Q1, p->Q2, phi, st));
         return IDP_OK;
@@ -1347,7 +1361,7 @@ int enqueue_grid(idp_plan p, const double *rho, double *phi, int stop, cudaStrea
         return IDP_OK;
     }
     // 6. the layer transforms of E; C += tab4 * S E;  phi = S C + u1 inside
-    if ((rc = e_layers(p, st))) return rc;
+    if ((rc = e_layers(p, st, overlap_rho))) return rc;
     {
         Mark mk(p, IDP_KERNEL_RHS6_EXPAND, st);
         IDP_CK(layers_fx(p) ? launch_rhs6_e_expand_q(p->grid, p->E0, p->E1, p->E2, p->sinq, p->sinq2, p->gmax[3],
