@@ -706,6 +706,7 @@ __global__ void __launch_bounds__(NT) face_invb_kernel(const FaceInvB a)
             const int t = f / L, m = f - t * L;
             qc sum{0, 0}, dif{0, 0};
             if (t < ncl)
+#pragma unroll 8
                 for (int ch = 0; ch < a.nchunk; ++ch) {
                     const qc *x = part + ((int64_t)ch * 2 * a.nc + c0 + t) * L + m;
                     sum = q_add(sum, x[0]);

@@ -1573,10 +1573,11 @@ int plan_setup(idp_plan p)
             p->pchunk[a_] = pch;
             pmax = std::max<int64_t>(pmax, (int64_t)nch * 2 * L * (Mc + 1));
             const int npair = (np + 1) / 2;
-            // three waves of resident blocks, at least 8 pairs a block
+            // three waves of resident blocks with at least 8 pairs a block; one wave with at least
+            // 2 on small grids
             const int qtiles = 2 * ((Mc + face_q_columns(L)) / face_q_columns(L));
             const int qslots = face_q_blocks_per_sm(L) * nsm;
-            p->qchunk[a_] = face_q_chunks(np, std::max(std::min(3 * qslots / qtiles, npair / 8), qslots / qtiles));
+            p->qchunk[a_] = face_q_chunks(np, std::max(std::min(3 * qslots / qtiles, npair / 8), std::min(qslots / qtiles, npair / 2)));
             pmax = std::max<int64_t>(pmax, (int64_t)p->qchunk[a_] * 2 * L * (Mc + 1));
             fmax = std::max<int64_t>(fmax, (int64_t)2 * (Mb + 1) * (Mc + 1));
             const int64_t per = (int64_t)(Mb + 1) * (Mc + 1);
