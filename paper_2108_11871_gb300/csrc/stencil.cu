@@ -50,10 +50,29 @@ __device__ __forceinline__ int face_dist(const Geo &g, int s, int js)
 // (eq. harmonic4thOrderNH2D).  L4 weights (host-computed in c): face +-e_s:
 // 1/h_s^2 - 2 sum_r c_sr/(h_s^2 h_r^2); edge +-e_s +-e_r: c_sr/(h_s^2 h_r^2),
 // c_sr = (h_s^2 + h_r^2)/12.
+// AHEAD: the loads first (their latencies overlap), then the sum, in the same order
+template <bool AHEAD>
 __device__ __forceinline__ double gtilde_at(const Geo &g, const StencilCoef &c, const double *__restrict__ U,
                                             const int i[3])
 {
-    // the loads first (their latencies overlap), then the sum in the order of the offsets
+    if constexpr (!AHEAD) {
+        double acc = 0.0;
+        for (int d0 = -1; d0 <= 1; ++d0) {
+            if (d0 != 0 && !g.act[0]) continue;
+            for (int d1 = -1; d1 <= 1; ++d1)
+                for (int d2 = -1; d2 <= 1; ++d2) {
+                    const int nz = (d0 != 0) + (d1 != 0) + (d2 != 0);
+                    if (nz == 0 || nz == 3) continue;
+                    const int j[3] = {i[0] + d0, i[1] + d1, i[2] + d2};
+                    if (!on_boundary(g, j)) continue;
+                    double wgt;
+                    if (nz == 1) wgt = c.wf[d0 != 0 ? 0 : (d1 != 0 ? 1 : 2)];
+                    else wgt = c.we[d0 != 0 ? 0 : 1][d2 != 0 ? 2 : 1];
+                    acc = fma(wgt, U[j[0] * g.ns[0] + j[1] * g.ns[1] + j[2]], acc);
+                }
+        }
+        return -acc;
+    }
     double u[27];
 #pragma unroll
     for (int q = 0; q < 27; ++q) {
@@ -86,6 +105,7 @@ __device__ __forceinline__ double gtilde_at(const Geo &g, const StencilCoef &c, 
 //   Q2[side][i0][i1]                  i2 = side ? n2-1 : 0, i0, i1 not on their layers
 // (2-D: axis 0 is inactive, Q1[side][i2] and Q2[side][i1]).  Entries outside a
 // part are zero.  Interior indices i_s = node index - 1.
+template <bool AHEAD>
 __global__ void gtilde_planes_kernel(const Grid3 gg, const StencilCoef c, const double *__restrict__ U,
                                      double *__restrict__ Q0, double *__restrict__ Q1, double *__restrict__ Q2)
 {
@@ -115,7 +135,7 @@ __global__ void gtilde_planes_kernel(const Grid3 gg, const StencilCoef c, const 
         double v = 0.0;
         if (keep) {
             const int i[3] = {g.act[0] ? k[0] + 1 : 0, k[1] + 1, k[2] + 1};
-            v = gtilde_at(g, c, U, i);
+            v = gtilde_at<AHEAD>(g, c, U, i);
         }
         *dst = v;
     }
@@ -501,6 +521,7 @@ __device__ __forceinline__ double extrap_w(int q) { return q == 0 ? 4.0 : q == 1
 //   Es[side][l][a][b], l = distance - 1, (a, b) the interior indices of the other
 //   two axes in increasing order; entries that belong to a lower part are zero.
 // E0 (3-D only) is followed by E1 and E2 in memory.
+template <bool AHEAD>
 __global__ void rhs6_e_kernel(const Grid3 gg, const StencilCoef c, const double *__restrict__ U,
                               const double *__restrict__ W, const double *__restrict__ Rt, double *__restrict__ E0,
                               double *__restrict__ E1, double *__restrict__ E2)
@@ -555,25 +576,36 @@ __global__ void rhs6_e_kernel(const Grid3 gg, const StencilCoef c, const double 
                     const int64_t step = nt0 == 4 ? st0 * g.is[0] : nt1 == 4 ? st1 * g.is[1] : st2;
                     acc = fma(4.0, Rt[base] + Rt[base + 2 * step], fma(-6.0, Rt[base + step], -Rt[base + 3 * step]));
                 } else {
-                    // edges and corners: 16 or 64 taps, a plane of up to 16 loaded at a time
-                    // (one load after the other made these few nodes the time of the kernel:
-                    // 33 x 65 x 97 16.5 -> 11.6 us)
+                    // edges and corners: 16 or 64 taps.  AHEAD: a plane of up to 16 loaded at a
+                    // time (one load after the other made these few nodes the time of the
+                    // kernel on small grids: 33 x 65 x 97 16.5 -> 11.6 us, 129^3 21.8 -> 15.6)
                     acc = 0.0;
                     for (int q0 = 0; q0 < nt0; ++q0) {
                         const double w0 = nt0 == 4 ? extrap_w(q0) : 1.0;
                         const double *rt = Rt + (int64_t)(f0 + q0 * st0) * g.is[0] + (int64_t)f1 * g.is[1] + f2;
-                        double x[4][4];
+                        if constexpr (AHEAD) {
+                            double x[4][4];
 #pragma unroll
-                        for (int q1 = 0; q1 < 4; ++q1)
+                            for (int q1 = 0; q1 < 4; ++q1)
 #pragma unroll
-                            for (int q2 = 0; q2 < 4; ++q2)
-                                x[q1][q2] = q1 < nt1 && q2 < nt2 ? rt[(int64_t)(q1 * st1) * g.is[1] + q2 * st2] : 0.0;
+                                for (int q2 = 0; q2 < 4; ++q2)
+                                    x[q1][q2] =
+                                        q1 < nt1 && q2 < nt2 ? rt[(int64_t)(q1 * st1) * g.is[1] + q2 * st2] : 0.0;
 #pragma unroll
-                        for (int q1 = 0; q1 < 4; ++q1) {
-                            const double w1 = nt1 == 4 ? w0 * extrap_w(q1) : w0;
+                            for (int q1 = 0; q1 < 4; ++q1) {
+                                const double w1 = nt1 == 4 ? w0 * extrap_w(q1) : w0;
 #pragma unroll
-                            for (int q2 = 0; q2 < 4; ++q2)
-                                if (q1 < nt1 && q2 < nt2) acc = fma(nt2 == 4 ? w1 * extrap_w(q2) : w1, x[q1][q2], acc);
+                                for (int q2 = 0; q2 < 4; ++q2)
+                                    if (q1 < nt1 && q2 < nt2)
+                                        acc = fma(nt2 == 4 ? w1 * extrap_w(q2) : w1, x[q1][q2], acc);
+                            }
+                        } else {
+                            for (int q1 = 0; q1 < nt1; ++q1) {
+                                const double w1 = nt1 == 4 ? w0 * extrap_w(q1) : w0;
+                                const double *r1 = rt + (int64_t)(q1 * st1) * g.is[1];
+                                for (int q2 = 0; q2 < nt2; ++q2)
+                                    acc = fma(nt2 == 4 ? w1 * extrap_w(q2) : w1, r1[q2 * st2], acc);
+                            }
                         }
                     }
                 }
@@ -865,6 +897,14 @@ StencilCoef make_stencil_coef(const Grid3 &g)
     return c;
 }
 
+// layers small enough that a kernel over them is as long as its slowest threads: loads ahead of
+// the sums (129^3: 33 us in the two kernels with them, 40 without; 257^3: 65 against 54)
+static bool few_layers(const Grid3 &g)
+{
+    const int64_t n0 = g.d == 3 ? g.n0 : 1, n1 = g.n1, n2 = g.n2;
+    return (g.d == 3 ? n1 * n2 : 0) + n0 * n2 + n0 * n1 < 100000;
+}
+
 dim3 grid3(int x, int y, int z) { return dim3((x + 31) / 32, (y + 7) / 8, z); }
 
 cudaError_t launch_gtilde_planes(const Grid3 &g, const StencilCoef &c, const double *U, double *Q0, double *Q1,
@@ -872,7 +912,8 @@ cudaError_t launch_gtilde_planes(const Grid3 &g, const StencilCoef &c, const dou
 {
     const int64_t n0 = g.d == 3 ? g.n0 - 2 : 1, n1 = g.n1 - 2, n2 = g.n2 - 2;
     const int64_t total = (g.d == 3 ? 2 * n1 * n2 : 0) + 2 * n0 * n2 + 2 * n0 * n1;
-    gtilde_planes_kernel<<<grid_for(total), 256, 0, st>>>(g, c, U, Q0, Q1, Q2);
+    auto kern = few_layers(g) ? gtilde_planes_kernel<true> : gtilde_planes_kernel<false>;
+    kern<<<grid_for(total), 256, 0, st>>>(g, c, U, Q0, Q1, Q2);
     return cudaGetLastError();
 }
 
@@ -929,7 +970,8 @@ cudaError_t launch_rhs6_spectral(const Grid3 &g, const StencilCoef &c, const dou
     } else {
         const int64_t n0 = g.d == 3 ? g.n0 - 2 : 1, n1 = g.n1 - 2, n2 = g.n2 - 2;
         const int64_t total = 4 * ((g.d == 3 ? n1 * n2 : 0) + n0 * n2 + n0 * n1);
-        rhs6_e_kernel<<<grid_for(total), 256, 0, st>>>(g, c, U, W, Rt, E0, E1, E2);
+        auto kern = few_layers(g) ? rhs6_e_kernel<true> : rhs6_e_kernel<false>;
+        kern<<<grid_for(total), 256, 0, st>>>(g, c, U, W, Rt, E0, E1, E2);
     }
     return cudaGetLastError();
 }
