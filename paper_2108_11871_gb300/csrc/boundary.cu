@@ -400,7 +400,7 @@ __global__ void __launch_bounds__(QLineCfg<L, THIN>::T, QLineCfg<L, THIN>::BPS) 
 #pragma unroll
         for (int i = 0; i < C; ++i) {
             const int q = g + i * G + 1;   // <= L
-            if (i < C - 1 || q < L) zl[2 * q_slot(q >> 1) + (q & 1)] = from(x[i]);
+            if (i < C - 1 || q < L) zl[2 * q_slot(q >> 1) + (q & 1)] = from.by_int(x[i]);
         }
         if (g == 0) zl[0] = 0;
     }

@@ -268,10 +268,22 @@ struct QFrom {
             const int g = (h & 0x7fffffff) < low ? 0 : h + add;
             return __double2ll_rn(__hiloint2double(g, __double2loint(x)));
         }
-        const unsigned lead = (h & 0x7ff00000) ? 0x100000u : 0u;
+        return shifted(x, (h & 0x7ff00000) ? 0x100000u : 0u);
+    }
+    // the same by integer shifts, for a kernel whose outputs keep the FP64 pipe busy (the real
+    // FFTs, two outputs to an input: 257^3 325 -> 303 us per solve; no gain in the sine pass)
+    __device__ __forceinline__ long long by_int(double x) const
+    {
+        return shifted(x, low >= 0 || (__double2hiint(x) & 0x7ff00000) ? 0x100000u : 0u);
+    }
+
+private:
+    __device__ __forceinline__ long long shifted(double x, unsigned lead) const
+    {
+        const int h = __double2hiint(x);
         const unsigned long long f =
-            (((unsigned long long)(((unsigned)h & 0xfffffu) | lead) << 32) | (unsigned)__double2loint(x)) << 7;
-        const int r = max(min(1082 - s - q_emax(h & 0x7fffffff), 63), 1);
+            (((unsigned long long)(((unsigned)h & 0xfffffu) | lead) << 32) | (unsigned)__double2loint(x)) << 10;
+        const int r = max(min(1085 - s - q_emax(h & 0x7fffffff), 64), 1);
         const long long v = (long long)(((f >> (r - 1)) + 1) >> 1), t = h >> 31;
         return (v ^ t) - t;
     }
