@@ -50,6 +50,9 @@ struct DstCfg {
     static constexpr int TW = q_tw_count(K, RM), HALF = TW, SIN = TW + K / 2 + 1, TAB = SIN + K / 2;
     static constexpr size_t SMEM = sizeof(qc) * (BUF + TAB);
     static constexpr int BPS = 1024 / T;   // blocks per SM that the registers allow
+    // contiguous outputs: whole warps on one line at a time (LW lines of a warp)
+    static constexpr bool WIDE = G < 32 && (2 * K) % 32 == 0;
+    static constexpr int LW = 32 / G;
     static_assert(K % G == 0 && (G & (G - 1)) == 0 && G <= 32 && T % 32 == 0 && T <= 256,
                   "whole warps; a group fits a warp");
 };
@@ -58,7 +61,8 @@ template <class Cfg, int K>
 __global__ void __launch_bounds__(Cfg::T, Cfg::BPS) dst_pass_kernel(const DstPass a)
 {
     constexpr int M = Cfg::M, N = Cfg::N, LB = Cfg::LB, NT = Cfg::T, G = Cfg::G, C = Cfg::C, RM = Cfg::RM;
-    constexpr int LS = Cfg::LS, OS = Cfg::OS;
+    constexpr int LS = Cfg::LS, OS = Cfg::OS, LW = Cfg::LW;
+    constexpr bool WIDE = Cfg::WIDE;
     extern __shared__ qc smem_q[];
     qc *buf = smem_q;
     int4 *tabs = reinterpret_cast<int4 *>(buf + Cfg::BUF);
@@ -213,9 +217,28 @@ __global__ void __launch_bounds__(Cfg::T, Cfg::BPS) dst_pass_kernel(const DstPas
 
     // 7. epilogue and store: thread (l, g) of the load takes the outputs e = g + i G of line l
     //    (U_{e+1}); consecutive threads again on consecutive e or on consecutive lines
-    if (l >= nl) return;
     int64_t osu, osv, ose;
     view_strides(a.out, a.axis, osu, osv, ose);
+    if (WIDE && contig && !a.tab && !a.add.p) {
+        // lines along axis 2: a warp writes its lines one after the other, 32 outputs at a time,
+        // in half as many pieces of 128-byte lines as the mapping below has: nothing to gain in
+        // device memory (257^3: 114.5 us a pass either way), but phi in host memory goes out over
+        // the link (host-buffer solve at 129^3: 662 -> 624 us)
+        const int lane = threadIdx.x & 31;
+#pragma unroll
+        for (int b = 0; b < LW; ++b) {
+            const int ln = threadIdx.x / 32 * LW + b;
+            if (ln >= nl) return;
+            double *out = a.out.p + (int64_t)u * osu + (int64_t)(v0 + ln) * osv + lane;
+            const QTo to(s_scale[ln]);
+            const long long *w0 = o + ln * OS + ((lane & 1) ? 0 : Cfg::OD);
+#pragma unroll
+            for (int i = 0; i < 2 * K / 32; ++i)
+                if (i < 2 * K / 32 - 1 || lane < 31) out[i * 32] = to(w0[q_slot(i * 16 + (lane >> 1))]);
+        }
+        return;
+    }
+    if (l >= nl) return;
     double *out = a.out.p + (int64_t)u * osu + (int64_t)(v0 + l) * osv + (int64_t)g * ose;
     const int64_t step = G * ose;
     const QTo to(s_scale[l]);
