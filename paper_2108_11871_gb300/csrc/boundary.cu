@@ -685,9 +685,7 @@ struct C2rCfg {
 template <int L>
 size_t smem_c2r() { return 2 * sizeof(double2) * C2rCfg<L>::LB * L; }
 
-// FX: the parts are the fixed-point sums of face.cu ([chunk][S, D][column][m]): the face is
-// S + D or S - D, added over the chunks in integers
-template <class R, int L, bool FX>
+template <class R, int L>
 __global__ void __launch_bounds__(NT) face_invb_kernel(const FaceInvB a)
 {
     using A = Ar<R>;
@@ -699,25 +697,6 @@ __global__ void __launch_bounds__(NT) face_invb_kernel(const FaceInvB a)
     const int c0 = blockIdx.x * TC;
     const int face = blockIdx.y;
     const int ncl = min(TC, a.nc - c0);
-    if constexpr (FX) {
-        const qc *part = reinterpret_cast<const qc *>(a.part);
-        const int g = *a.gmax, base = 1102 - g - a.lgn;
-        for (int f = threadIdx.x; f < TC * L; f += NT) {
-            const int t = f / L, m = f - t * L;
-            qc sum{0, 0}, dif{0, 0};
-            if (t < ncl)
-#pragma unroll 8
-                for (int ch = 0; ch < a.nchunk; ++ch) {
-                    const qc *x = part + ((int64_t)ch * 2 * a.nc + c0 + t) * L + m;
-                    sum = q_add(sum, x[0]);
-                    dif = q_add(dif, x[(int64_t)a.nc * L]);
-                }
-            const qc v = face ? q_sub(sum, dif) : q_add(sum, dif);
-            const int ek = t < ncl ? a.ek[(int64_t)(c0 + t) * (L / 2 + 1) + (m <= L / 2 ? m : L - m)] : 0;
-            const QTo to(g >= Q_GNAN ? Q_NAN : base - ek);
-            bufA[t * L + m] = make_double2(to(v.re), to(v.im));
-        }
-    } else {
     const Cx *part = reinterpret_cast<const Cx *>(a.part);
     for (int f = threadIdx.x; f < TC * L; f += NT) {
         const int m = f / TC, t = f - m * TC;
@@ -730,7 +709,6 @@ __global__ void __launch_bounds__(NT) face_invb_kernel(const FaceInvB a)
             }
         }
         bufA[t * L + m] = A::cmake(sr, si);
-    }
     }
     __syncthreads();
     const Cx *Z = cta_fft_t<R, L, TC, NT, true>(bufA, bufB, inv_tw<R>(a.t), false);
@@ -787,6 +765,216 @@ __global__ void __launch_bounds__(NT) face_c2r_kernel(const FaceC2R a)
         const int64_t node = fbase + (int64_t)row * a.row_stride + (int64_t)t * a.col_stride;
         st_real<R>(a.dst0, node, v);
         if (a.dst1) st_real<R>(a.dst1, node, v);
+    }
+}
+
+// ---------------------------------------------------------------- stage 3, fixed point
+// The inverse transforms in block fixed point (q64.cuh): every line on its own scale, FP64
+// out.  An inverse FFT is the forward one of the conjugates, conjugated.  (The FP64 forms, which
+// the tensor-core modes keep, are bound by the FP64 pipe and summed the parts once per face;
+// these wait for memory and for their barriers, a few microseconds each.  257^3: 85 -> 56 us per
+// solve in stage 3a and 46 -> 35 in 3b, 513 x 385: stage 3b 26 -> 21; whole solves 0.5 to 2.7 %.)
+__device__ __forceinline__ int line_high(double2 v) { return max(q_high(v.x), q_high(v.y)); }
+// (half of each weight: the sum over 1024 complex values stays below 2^32)
+__device__ __forceinline__ unsigned line_weight(double2 v, int emax)
+{
+    return (q_weight(v.x, emax) >> 1) + (q_weight(v.y, emax) >> 1) + 2;
+}
+
+// Stage 3a, L = 2 Pb: a block has TC columns of both faces, the sum S + D and the difference
+// S - D of the parts (each read once); L / 2 threads per column, two frequencies each.
+template <int L>
+struct InvbQCfg {
+    static constexpr int G = L / 2, R = (L % 3 == 0 ? 192 : 256) / L, TC = R < 1 ? 1 : R, T = TC * G, LB = 2 * TC;
+    static constexpr int LS = q_line(L), TW = q_tw_count(L, 8);
+    static constexpr size_t SMEM = sizeof(qc) * (LB * LS + TW);
+    static_assert(T % 32 == 0, "whole warps");
+};
+
+template <int L>
+__global__ void __launch_bounds__(InvbQCfg<L>::T) face_invb_q_kernel(const FaceInvB a)
+{
+    using Cfg = InvbQCfg<L>;
+    constexpr int TC = Cfg::TC, G = Cfg::G, NT = Cfg::T, LS = Cfg::LS;
+    extern __shared__ qc smem_q[];
+    qc *buf = smem_q;   // line 2 t + face
+    int4 *tws = reinterpret_cast<int4 *>(buf + Cfg::LB * LS);
+    __shared__ int s_high[Cfg::LB];
+    __shared__ unsigned s_sum[Cfg::LB];
+    for (int f = threadIdx.x; f < Cfg::TW; f += NT) tws[f] = __ldg(a.q + f);
+    if (threadIdx.x < Cfg::LB) {
+        s_high[threadIdx.x] = 0;
+        s_sum[threadIdx.x] = 0;
+    }
+    const int Mb = a.Mb, c0 = blockIdx.x * TC, ncl = min(TC, a.nc - c0);
+    const int t = threadIdx.x / G, e = threadIdx.x % G;
+    const int g = *a.gmax, base = 1102 - g - a.lgn;
+    double2 x[2][2];   // [face][frequency e, e + G]
+    {
+        qc sum[2] = {{0, 0}, {0, 0}}, dif[2] = {{0, 0}, {0, 0}};
+        int ek[2] = {0, 0};
+        if (t < ncl) {
+            const int *k = a.ek + (int64_t)(c0 + t) * (L / 2 + 1);
+            ek[0] = k[e];
+            ek[1] = k[L / 2 - e];
+            const qc *x0 = reinterpret_cast<const qc *>(a.part) + (int64_t)(c0 + t) * L + e;
+            const int64_t half = (int64_t)a.nc * L;
+#pragma unroll 4
+            for (int ch = 0; ch < a.nchunk; ++ch, x0 += 2 * half) {
+                sum[0] = q_add(sum[0], x0[0]);
+                sum[1] = q_add(sum[1], x0[G]);
+                dif[0] = q_add(dif[0], x0[half]);
+                dif[1] = q_add(dif[1], x0[half + G]);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const QTo to(g >= Q_GNAN ? Q_NAN : base - ek[i]);
+            x[0][i] = make_double2(to(sum[i].re + dif[i].re), to(sum[i].im + dif[i].im));
+            x[1][i] = make_double2(to(sum[i].re - dif[i].re), to(sum[i].im - dif[i].im));
+        }
+    }
+    __syncthreads();
+    auto scale = [&](int face, int &emax) {
+        emax = q_emax(s_high[2 * t + face]);
+        return emax == 0x7ff ? Q_NAN : 1103 - (emax + q_bits(s_sum[2 * t + face]) + 1);   // absolute sum below 2^60 units
+    };
+#pragma unroll
+    for (int f = 0; f < 2; ++f) {
+        const int high = max(line_high(x[f][0]), line_high(x[f][1]));
+        if constexpr (G % 32 == 0) {
+            const int w = __reduce_max_sync(0xffffffffu, high);
+            if ((threadIdx.x & 31) == 0) atomicMax(&s_high[2 * t + f], w);
+        } else {
+            atomicMax(&s_high[2 * t + f], high);
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int f = 0; f < 2; ++f) {
+        const int emax = q_emax(s_high[2 * t + f]);
+        const unsigned sum = line_weight(x[f][0], emax) + line_weight(x[f][1], emax);
+        if constexpr (G % 32 == 0) {
+            const unsigned w = __reduce_add_sync(0xffffffffu, sum);
+            if ((threadIdx.x & 31) == 0) atomicAdd(&s_sum[2 * t + f], w);
+        } else {
+            atomicAdd(&s_sum[2 * t + f], sum);
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int f = 0; f < 2; ++f) {
+        int emax;
+        const int sc = scale(f, emax);
+        const QFrom from(sc, emax);
+        qc *z = buf + (2 * t + f) * LS;
+        z[q_slot(e)] = qc{from(x[f][0].x), -from(x[f][0].y)};
+        z[q_slot(e + G)] = qc{from(x[f][1].x), -from(x[f][1].y)};
+    }
+    __syncthreads();
+    q_fft<L, 8, Cfg::LB, NT, LS>(buf, tws);
+    // rows 0..Mb (Mb <= L / 2); column fastest, as in the output
+#pragma unroll
+    for (int face = 0; face < 2; ++face) {
+        double2 *out = a.out + (int64_t)face * (Mb + 1) * a.nc + c0;
+        for (int f = threadIdx.x; f < TC * (Mb + 1); f += NT) {
+            const int j = f / TC, tt = f % TC;
+            if (tt >= ncl) continue;
+            const int emax = q_emax(s_high[2 * tt + face]);
+            const QTo to(emax == 0x7ff ? Q_NAN : 1103 - (emax + q_bits(s_sum[2 * tt + face]) + 1));
+            const qc z = buf[(2 * tt + face) * LS + q_slot(j)];
+            out[(int64_t)j * a.nc + tt] = make_double2(to(z.re), to(-z.im));
+        }
+    }
+}
+
+// Stage 3b, L = Pc: G threads per row, C pairs (X_k, X_{L-k}) each.
+template <int L>
+struct C2rQCfg {
+    static constexpr int G1 = L % 3 == 0 ? L / 6 : L / 2, G = G1 > 64 ? 64 : G1, C = L / 2 / G, W = G < 32 ? G : 32;
+    static constexpr int T = 128, LB = T / G, LS = q_line(L), TW = q_tw_count(L, 8);
+    static constexpr size_t SMEM = sizeof(qc) * (LB * LS + TW);
+    static_assert((G & (G - 1)) == 0 && C * G * 2 == L, "power-of-two groups, whole lines");
+};
+
+template <int L>
+__global__ void __launch_bounds__(C2rQCfg<L>::T) face_c2r_q_kernel(const FaceC2R a)
+{
+    using Cfg = C2rQCfg<L>;
+    constexpr int LB = Cfg::LB, G = Cfg::G, C = Cfg::C, NT = Cfg::T, LS = Cfg::LS;
+    extern __shared__ qc smem_q[];
+    qc *buf = smem_q;
+    int4 *tws = reinterpret_cast<int4 *>(buf + LB * LS);
+    __shared__ int s_high[LB];
+    __shared__ unsigned s_sum[LB];
+    for (int f = threadIdx.x; f < Cfg::TW; f += NT) tws[f] = __ldg(a.q + f);
+    if (threadIdx.x < LB) {
+        s_high[threadIdx.x] = 0;
+        s_sum[threadIdx.x] = 0;
+    }
+    const int face = blockIdx.y, r0 = blockIdx.x * LB, nl = min(LB, a.nrows - r0);
+    const int l = threadIdx.x / G, g = threadIdx.x % G;
+    // pairs k = g + i G; the thread with k = 0 has X_{L/2} too
+    double2 xk[C], xc[C], xm = make_double2(0.0, 0.0);
+    const double2 *in = a.in + ((int64_t)face * a.nrows + r0 + l) * (L + 1);
+#pragma unroll
+    for (int i = 0; i < C; ++i) {
+        xk[i] = l < nl ? in[g + i * G] : make_double2(0.0, 0.0);
+        xc[i] = l < nl ? in[L - g - i * G] : make_double2(0.0, 0.0);
+    }
+    if (g == 0 && l < nl) xm = in[L / 2];
+    __syncthreads();
+    int high = line_high(xm);
+#pragma unroll
+    for (int i = 0; i < C; ++i) high = max(high, max(line_high(xk[i]), line_high(xc[i])));
+    for (int d = 1; d < Cfg::W; d <<= 1) high = max(high, __shfl_xor_sync(0xffffffffu, high, d));
+    const bool lead = (threadIdx.x & (Cfg::W - 1)) == 0;
+    if (lead) atomicMax(&s_high[l], high);
+    __syncthreads();
+    const int emax = q_emax(s_high[l]);
+    unsigned sum = line_weight(xm, emax);
+#pragma unroll
+    for (int i = 0; i < C; ++i) sum += line_weight(xk[i], emax) + line_weight(xc[i], emax);
+    for (int d = 1; d < Cfg::W; d <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
+    if (lead) atomicAdd(&s_sum[l], sum);
+    __syncthreads();
+    // absolute sum below 2^58 units; that of the FFT's inputs is up to four times as large
+    const int sc = 1101 - (emax + q_bits(s_sum[l]) + 1);
+    {
+        const QFrom from(sc, emax);
+        qc *z = buf + l * LS;
+        // A = X_k + conj X_{L-k}, B = e^{+i pi k/L} (X_k - conj X_{L-k}): Z'_k = A + i B and
+        // Z'_{L-k} = conj A + i conj B, of which the conjugates go in
+        auto pair = [&](int k, qc p, qc q) {
+            const long long Ar = p.re + q.re, Ai = p.im - q.im;
+            const qc Bc = q_cmul(qc{p.re - q.re, -(p.im + q.im)}, __ldg(a.qhalf + k));   // conj B
+            z[q_slot(k)] = qc{Ar + Bc.im, -Ai - Bc.re};
+            if (k > 0) z[q_slot(L - k)] = qc{Ar - Bc.im, Ai - Bc.re};
+        };
+#pragma unroll
+        for (int i = 0; i < C; ++i)
+            pair(g + i * G, qc{from(xk[i].x), from(xk[i].y)}, qc{from(xc[i].x), from(xc[i].y)});
+        if (g == 0) {
+            const qc m = qc{from(xm.x), from(xm.y)};
+            pair(L / 2, m, m);
+        }
+    }
+    __syncthreads();
+    q_fft<L, 8, LB, NT, LS>(buf, tws);
+    if (l >= nl) return;
+    const int Mc = a.Mc, row = r0 + l;
+    if (a.skip_row_edges && (row == 0 || row == a.nrows - 1)) return;
+    const QTo to(emax == 0x7ff ? Q_NAN : sc);
+    const long long *w = reinterpret_cast<const long long *>(buf + l * LS);
+    const int64_t fbase = (face ? a.base[1] : a.base[0]) + (int64_t)row * a.row_stride;
+    const int lo = a.skip_col_edges ? 1 : 0, hi = a.skip_col_edges ? Mc - 1 : Mc;
+    for (int t = g; t <= hi; t += G) {   // t <= Mc <= L, so t / 2 < L
+        if (t < lo) continue;
+        const long long q = w[2 * q_slot(t >> 1) + (t & 1)];
+        const double v = to((t & 1) ? -q : q);
+        const int64_t node = fbase + (int64_t)t * a.col_stride;
+        a.dst0[node] = v;
+        if (a.dst1) a.dst1[node] = v;
     }
 }
 
@@ -940,15 +1128,18 @@ cudaError_t attrs_len_r()
         if ((e = cudaFuncSetAttribute(rfft_q_kernel<L, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)QLineCfg<L, true>::SMEM)))
             return e;
+        if ((e = cudaFuncSetAttribute(face_c2r_q_kernel<L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)C2rQCfg<L>::SMEM)))
+            return e;
     }
     if ((e = cudaFuncSetAttribute(face_kernel<R, L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)smem_face<L>())))
         return e;
-    if ((e = cudaFuncSetAttribute(face_invb_kernel<R, L, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if ((e = cudaFuncSetAttribute(face_invb_kernel<R, L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)smem_invb<L>())))
         return e;
-    if ((e = cudaFuncSetAttribute(face_invb_kernel<double, L, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)smem_invb<L>())))
+    if ((e = cudaFuncSetAttribute(face_invb_q_kernel<L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)InvbQCfg<L>::SMEM)))
         return e;
     return cudaFuncSetAttribute(face_c2r_kernel<R, L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)smem_c2r<L>());
@@ -1068,10 +1259,14 @@ cudaError_t launch_face_pass_2d(const FacePass2D &a, cudaStream_t st)
 cudaError_t launch_face_inv_b(const FaceInvB &a, cudaStream_t st)
 {
     IDP_LEN_SWITCH(2 * (a.Pb ? a.Pb : a.Mb), {
+        if (a.fx) {
+            using Cfg = InvbQCfg<L>;
+            face_invb_q_kernel<L><<<(a.nc + Cfg::TC - 1) / Cfg::TC, Cfg::T, Cfg::SMEM, st>>>(a);
+            return cudaGetLastError();
+        }
         dim3 grid((a.nc + InvbCfg<L>::TC - 1) / InvbCfg<L>::TC, 2);
-        if (a.fx) face_invb_kernel<double, L, true><<<grid, NT, smem_invb<L>(), st>>>(a);
-        else if (a.dd) face_invb_kernel<ddr, L, false><<<grid, NT, smem_invb<L>(), st>>>(a);
-        else face_invb_kernel<double, L, false><<<grid, NT, smem_invb<L>(), st>>>(a);
+        if (a.dd) face_invb_kernel<ddr, L><<<grid, NT, smem_invb<L>(), st>>>(a);
+        else face_invb_kernel<double, L><<<grid, NT, smem_invb<L>(), st>>>(a);
         return cudaGetLastError();
     })
 }
@@ -1079,6 +1274,12 @@ cudaError_t launch_face_inv_b(const FaceInvB &a, cudaStream_t st)
 cudaError_t launch_face_c2r(const FaceC2R &a, cudaStream_t st)
 {
     IDP_LEN_SWITCH(a.Pc ? a.Pc : a.Mc, {
+        if constexpr (L <= 512)
+            if (a.fx) {
+                using Cfg = C2rQCfg<L>;
+                face_c2r_q_kernel<L><<<dim3((a.nrows + Cfg::LB - 1) / Cfg::LB, 2), Cfg::T, Cfg::SMEM, st>>>(a);
+                return cudaGetLastError();
+            }
         dim3 grid((a.nrows + C2rCfg<L>::LB - 1) / C2rCfg<L>::LB, 2);
         if (a.dd) face_c2r_kernel<ddr, L><<<grid, NT, smem_c2r<L>(), st>>>(a);
         else face_c2r_kernel<double, L><<<grid, NT, smem_c2r<L>(), st>>>(a);

@@ -221,6 +221,7 @@ struct FaceInvB {
     int fx, lgn;               // 1: parts of FaceQPass, its lgn and ek[nc][Pb+1]
     const int *ek;
     const int *gmax;
+    const int4 *q;             // fx: factors of length 2Pb (q64.cuh)
 };
 cudaError_t launch_face_inv_b(const FaceInvB &a, cudaStream_t st);
 
@@ -240,6 +241,8 @@ struct FaceC2R {
     FftTables t;               // length Pc
     int dd;
     int Pc;                    // 0: Mc
+    int fx;                    // 1: block fixed point
+    const int4 *q, *qhalf;     // fx: factors and e^{-i pi k/Pc}, k = 0..Pc/2 (q64.cuh)
 };
 cudaError_t launch_face_c2r(const FaceC2R &a, cudaStream_t st);
 

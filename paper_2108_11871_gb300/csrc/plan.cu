@@ -976,7 +976,9 @@ int face_q_pass(idp_plan p, int a_, int nchunk, double2 *part, FaceQPass *q, Fac
     q->gmax = p->gmax[a_ == 2 ? 1 : 0];
     ib->fx = 1; ib->nchunk = nchunk; ib->lgn = q->lgn; ib->ek = p->kq_ek[a_]; ib->gmax = q->gmax;
     const int4 *half;
-    return get_fft_tables(p, 2 * p->P[b], &q->q, &half);
+    const int rc = get_fft_tables(p, 2 * p->P[b], &q->q, &half);
+    ib->q = q->q;
+    return rc;
 }
 
 // boundary values g into the boundary nodes of dst0 (and dst1 if not null).
@@ -1078,6 +1080,8 @@ int boundary(idp_plan p, const double *rho, double *dst0, double *dst1, cudaStre
             c.skip_row_edges = 0; c.skip_col_edges = (face == 2);
             if ((rc = get_fft(p, p->P[other], &t))) return rc;
             c.t = t;
+            c.fx = fx;
+            if ((rc = get_fft_tables(p, p->P[other], &c.q, &c.qhalf))) return rc;
             Mark mk(p, IDP_KERNEL_FACE_C2R, sa);
             IDP_CK(launch_face_c2r(c, sa));
         }
@@ -1137,6 +1141,8 @@ int boundary(idp_plan p, const double *rho, double *dst0, double *dst1, cudaStre
         if ((rc = get_fft(p, p->P[c], &t))) return rc;
         cr.t = t;
         cr.dd = dd;
+        cr.fx = fx;
+        if ((rc = get_fft_tables(p, p->P[c], &cr.q, &cr.qhalf))) return rc;
         Mark mk(p, IDP_KERNEL_FACE_C2R, sa);
         IDP_CK(launch_face_c2r(cr, sa));
     }
