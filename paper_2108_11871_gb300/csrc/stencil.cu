@@ -703,8 +703,11 @@ __global__ void rhs6_e_expand_kernel(const Grid3 gg, const double *__restrict__ 
 // The two expansions from layers in fixed point (layers_combine with gmax): the sums over the
 // axes run in integers, so that the FP64 pipe, which bounded the kernels above (5 and 7
 // instructions a point: 1.71 and 1.59 ms at 513^3), has the conversion of the sum and the
-// products with the tables left (3 and 2): 0.95 and 0.80 ms.  A thread takes one (k1, k2) and
-// ck (even) consecutive k0: its two (four) values of the layers of axis 0 and the factors of
+// products with the tables left (3 and 2): 0.93 and 0.81 ms, of which the bytes need 0.79 and
+// 0.48.  They wait for memory, so warps count: five blocks per SM (48 registers; a loop
+// unrolled by four at 72 registers took 1.37 and 0.93 ms, six blocks with small spills 0.94 and
+// 0.78), and no array indexed by the loop (local memory otherwise).  A thread takes one (k1, k2)
+// and ck (even) consecutive k0: its two (four) values of the layers of axis 0 and the factors of
 // axes 1 and 2 stay in registers.  Eight k0 from 2^20 points on; below that two, which
 // leaves more threads (65^3: 3 us per solve).
 int expand_chunk(const Grid3 &g)
@@ -718,7 +721,8 @@ __device__ __forceinline__ QTo expand_to(const int *gmax)
     return QTo(gm >= Q_GNAN ? Q_NAN : 1098 - gm);
 }
 
-__global__ void gtilde_expand_q_kernel(const Grid3 gg, const long long *__restrict__ Q0, const long long *__restrict__ Q1,
+__global__ void __launch_bounds__(256, 5)
+gtilde_expand_q_kernel(const Grid3 gg, const long long *__restrict__ Q0, const long long *__restrict__ Q1,
                                        const long long *__restrict__ Q2, const int2 *__restrict__ sq,
                                        const int *__restrict__ gmax, const double *__restrict__ tab, const double *add,
                                        double *out, const double *__restrict__ tab2, const double *__restrict__ add2,
@@ -740,12 +744,12 @@ __global__ void gtilde_expand_q_kernel(const Grid3 gg, const long long *__restri
     const long long *q1 = Q1 + (int64_t)((k1 & 1) ? n0 + k0 : k0) * n2 + k2;
     const long long *q2 = Q2 + (int64_t)((k2 & 1) ? n0 + k0 : k0) * n1 + k1;
     int64_t t = k0 * g.is[0] + (int64_t)k1 * g.is[1] + k2;
-#pragma unroll 4
+#pragma unroll 2
     for (int k = k0; k < e0; ++k, q1 += n2, q2 += n1, t += g.is[0]) {
         long long v = q_rmul(*q1, s1.x, s1.y) + q_rmul(*q2, s2.x, s2.y);
         if (g.act[0]) {
             const int2 s0 = sq[k];
-            v += q_rmul(q0[(k - k0) & 1], s0.x, s0.y);   // k0 is even
+            v += q_rmul((k & 1) ? q0[1] : q0[0], s0.x, s0.y);   // k0 is even
         }
         const double x = to(v), tb = tab[t];
         out[t] = add ? fma(tb, x, add[t]) : tb * x;
@@ -753,7 +757,8 @@ __global__ void gtilde_expand_q_kernel(const Grid3 gg, const long long *__restri
     }
 }
 
-__global__ void rhs6_e_expand_q_kernel(const Grid3 gg, const long long *__restrict__ E0, const long long *__restrict__ E1,
+__global__ void __launch_bounds__(256, 5)
+rhs6_e_expand_q_kernel(const Grid3 gg, const long long *__restrict__ E0, const long long *__restrict__ E1,
                                        const long long *__restrict__ E2, const int2 *__restrict__ sq,
                                        const int2 *__restrict__ sq2, const int *__restrict__ gmax,
                                        const double *__restrict__ tab, double *__restrict__ out, int ck)
@@ -778,13 +783,14 @@ __global__ void rhs6_e_expand_q_kernel(const Grid3 gg, const long long *__restri
     const long long *q1 = E1 + (int64_t)k0 * n2 + k2 + ((k1 & 1) ? 2 * p1 : 0);
     const long long *q2 = E2 + (int64_t)k0 * n1 + k1 + ((k2 & 1) ? 2 * p2 : 0);
     int64_t t = k0 * g.is[0] + (int64_t)k1 * g.is[1] + k2;
-#pragma unroll 4
+#pragma unroll 2
     for (int k = k0; k < e0; ++k, q1 += n2, q2 += n1, t += g.is[0]) {
         long long v = q_rmul(q1[0], s1.x, s1.y) + q_rmul(q1[p1], d1.x, d1.y);
         v += q_rmul(q2[0], s2.x, s2.y) + q_rmul(q2[p2], d2.x, d2.y);
         if (g.act[0]) {
             const int2 s0 = sq[k], d0 = sq2[k];
-            v += q_rmul(q0[(k - k0) & 1], s0.x, s0.y) + q_rmul(r0[(k - k0) & 1], d0.x, d0.y);
+            const bool odd = k & 1;   // k0 is even
+            v += q_rmul(odd ? q0[1] : q0[0], s0.x, s0.y) + q_rmul(odd ? r0[1] : r0[0], d0.x, d0.y);
         }
         out[t] = fma(tab[t], to(v), out[t]);
     }
