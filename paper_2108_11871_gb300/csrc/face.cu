@@ -133,8 +133,10 @@ __global__ void __launch_bounds__(FaceQCfg<L>::NT, FaceQCfg<L>::BPS) face_q_kern
             qc v[RL];
 #pragma unroll
             for (int q = 0; q < RL; ++q) v[q] = x[UL % 8 == 0 ? q_slot(q * UL) : q_slot(j + q * UL) - q_slot(j)];
+            if (j != 0) {   // (see q_pass)
 #pragma unroll
-            for (int q = 1; q < RL; ++q) v[q] = q_cmul(v[q], tw[(q - 1) * UL]);
+                for (int q = 1; q < RL; ++q) v[q] = q_cmul(v[q], tw[(q - 1) * UL]);
+            }
             q_dft<RL>(v);
             const int2 *k = ks + ct * KS;
 #pragma unroll
@@ -172,8 +174,11 @@ __global__ void face_kq_kernel(const double *__restrict__ khat, int np, int64_t 
         for (int p = 0; p < npair; ++p) {
             const double k1 = khat[p * per + x], k2 = khat[(np - 1 - p) * per + x];
             const long long s = __double2ll_rn((k1 + k2) * scale), d = __double2ll_rn((k1 - k2) * scale);
-            kq[p * per + x] = make_int2((int)(s >> 31), (int)(s & 0x7fffffff));
-            kq[(npair + p) * per + x] = make_int2((int)(d >> 31), (int)(d & 0x7fffffff));
+            // low words of either sign: what a product drops is then no bias over the slices
+            // (|s| < 2^62 (1 - 1e-9) keeps the high word in range)
+            const int sh = (int)((s + (1LL << 30)) >> 31), dh = (int)((d + (1LL << 30)) >> 31);
+            kq[p * per + x] = make_int2(sh, (int)(s - ((long long)sh << 31)));
+            kq[(npair + p) * per + x] = make_int2(dh, (int)(d - ((long long)dh << 31)));
         }
     }
 }

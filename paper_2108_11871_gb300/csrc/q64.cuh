@@ -202,7 +202,10 @@ __device__ __forceinline__ void q_pass(qc *X, const int4 *__restrict__ tw)
     for (int it = 0; it < IT; ++it) {
         const int b = threadIdx.x + it * NT, line = b / U, j = b - line * U, k = j % Ns;
         if (UNITS % NT != 0 && b >= UNITS) break;
-        if constexpr (Ns > 1) {
+        // no factors at k = 0: the word pairs end 2^-62 below 1, and with it half of such
+        // products would come out one unit low, a bias that DC adds up over the line (noise at
+        // 257^3: boundary values off by 2e-13, against 1e-15 in FP64 and without it)
+        if (Ns > 1 && k != 0) {
             const int4 *w = tw + k;
 #pragma unroll
             for (int q = 1; q < R; ++q) v[it][q] = q_cmul(v[it][q], w[(q - 1) * Ns]);

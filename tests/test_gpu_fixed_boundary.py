@@ -82,3 +82,18 @@ def test_no_charge_gives_zero_and_a_nan_every_node(n):
     rho = _mixed(n)
     rho[tuple(k // 3 for k in n)] = np.nan
     assert np.isnan(_run(idp, n, rho, order=6)).all()
+
+
+def test_rounding_has_no_bias():
+    # a product that rounds one way is a bias, which the lowest frequency adds up over lines and
+    # slices (factors 2^-62 below 1 gave 4e-14 here).  Unbiased: the face pass's unit is 2^-61
+    # of the bound 2 * 128 * 128 on a column's absolute sum, 1e-15 of a coefficient of random
+    # signs (about 13), a few units in all: 1e-14 for the largest error
+    import paper_2108_11871_gb300 as idp
+    n = (129, 129, 129)
+    rho = w.random_interior(n, seed=3)
+    idx = ogreens.boundary_indices(n)
+    t = idx[np.random.default_rng(0).choice(len(idx), 40, replace=False)]
+    ref = ogreens.boundary_direct(rho, _h(n), t)
+    got = _run(idp, n, rho, stage=idp.IDP_STAGE_BOUNDARY)[tuple(t.T)]
+    assert np.abs(got - ref).max() <= 1e-14 * np.abs(ref).max()
