@@ -44,12 +44,12 @@ KERNEL_NAMES = {1: "dst_pass", 2: "rfft", 3: "face", 4: "face_invb", 5: "face_c2
                 7: "rhs6_w", 8: "rhs6_core", 9: "rhs6_extrap", 10: "gtilde_expand", 11: "dst_pass_layers",
                 12: "mixed_pass", 13: "support_flags", 14: "rhs6_expand", 15: "line1d", 16: "pad",
                 17: "validate"}
-# DRAM bytes (read + write) per full-volume launch of the FP64 sine pass, from ncu
+# DRAM bytes (read + write) per full-volume launch of the sine pass, from ncu
 # (dram__bytes_read.sum + dram__bytes_write.sum over the 8 passes of one solve,
 # averaged); a grid not listed reports null
-# (profiles/dst_pass_fp64_257cube_traffic.md: 248.5 MB per launch at 257^3, scaled by the
-# interior points to 513^3)
-DST_TRAFFIC = {(257, 257, 257): 248.5e6, (513, 513, 513): 2.00e9}
+# (profiles/dst_pass_257cube.md: 254 MB per launch at 257^3, scaled by the interior
+# points to 513^3)
+DST_TRAFFIC = {(257, 257, 257): 2.54e8, (513, 513, 513): 2.04e9}
 
 
 def parse():

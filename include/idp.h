@@ -83,7 +83,7 @@ enum {
                                memory and returns, and idp_plan_status reports IDP_ETIMEOUT */
     IDP_KEY_MIXED_BOUNDARY_DF32 = 8, /* value 1: in the tensor-core modes (IDP_PRECISION_MIXED_*) the 3-D
                                boundary convolutions run in double-float arithmetic (48 significant
-                               bits, as in IDP_PRECISION_DF32) instead of FP64; value 0 (default):
+                               bits) instead of FP64; value 0 (default):
                                FP64.  No effect in the other modes.  Setting 1 allocates the
                                double-float copies of the kernel spectra. */
     IDP_KEY_NVTX = 9,       /* value 1: NVTX ranges (NVTX v3, host side, at enqueue time) around every
@@ -110,7 +110,9 @@ enum {
 
 /* values of IDP_KEY_PRECISION */
 enum {
-    IDP_PRECISION_FP64 = 0,        /* FP64 FFT-based sine transforms (default) */
+    IDP_PRECISION_FP64 = 0,        /* FP64-class FFT-based transforms (default): FP64 in and out, the FFTs
+                                      in 64-bit integers on a power-of-two scale per line (errors at or
+                                      below those of FP64 FFTs on smooth densities) */
     IDP_PRECISION_MIXED_BF16X3 = 1, /* the sine transforms of rho, of R and the final inverse become
                                       dense sine-matrix products on the tensor cores: operands split
                                       into three BF16 pieces, six products, FP32 accumulation
@@ -120,11 +122,11 @@ enum {
                                       differences form R) and the transforms of the boundary layers run
                                       in double-float arithmetic (48 significant bits).  Setting it
                                       allocates the pieces of the sine matrices and FP32 temporaries. */
-    IDP_PRECISION_DF32 = 2,        /* the 3-D boundary convolutions (and the direct sine sums of lengths
-                                      without an FFT) in double-float arithmetic (a value is a pair of
-                                      FP32 numbers, ~48 significant bits) on the FP32 pipe, FP64 arrays
-                                      in and out; the sine transforms and all stencils as in FP64.
-                                      Results agree with FP64 to a few 1e-13 relative. */
+    IDP_PRECISION_DF32 = 2,        /* the direct sine sums of lengths without an FFT (exact plans) in
+                                      double-float arithmetic (a value is a pair of FP32 numbers, ~48
+                                      significant bits) on the FP32 pipe; everything else as in FP64.
+                                      Results agree with FP64 to a few 1e-13 relative, bit for bit
+                                      where every length has an FFT. */
     IDP_PRECISION_MIXED_TF32X3 = 3 /* as MIXED_BF16X3, with the operands split into two TF32 pieces
                                       (hi + lo, ~22 significant bits) and three products (hi*hi,
                                       hi*lo, lo*hi; tcgen05 kind::tf32), FP32 accumulation */

@@ -10,6 +10,12 @@
 //   U_{2k} = -Im T_k,   U_{2k+1} = U_{2k-1} + Re T_k,   U_1 = Re Z_0 + Im Z_0
 // (the real-FFT form of the DST-I; T = 4 Y where Y is the real FFT of y), in the
 // block fixed-point arithmetic of q64.cuh, FP64 in and out.
+//
+// What bounds it (257^3, 115 us a pass, of which its bytes need 40): no single unit.  The two
+// integer pipes are busy 36-47 % of the time, the FP64 pipe, which converts, 47-60 %, and
+// shared memory 34-47 %, in turns, because the blocks of an SM are in different phases; half
+// of the warps fit (64 registers).  In FP64 the pass was bound by the FP64 pipe: 250 us at
+// 257^3, 3.9 ms at 513^3 (now 0.98).
 #include "arith.cuh"
 #include "q64.cuh"
 
@@ -291,7 +297,8 @@ cudaError_t launch_cfg(const DstPass &a, int nu, int nv, cudaStream_t st)
 }
 
 // The shapes of a pass: Big (up to 256 threads, C = 8 or 6 pairs a thread), Mid with half
-// its lines, and Thin with up to four times the threads per line, for launches that leave most of the chip idle and so are as long as one block.
+// its lines, and Thin with up to four times the threads per line, for launches that leave most
+// of the chip idle and so are as long as one block.
 template <int K>
 struct DstShapes {
     static constexpr int G = K % 3 == 0 ? K / 6 : K / 8;
@@ -315,9 +322,9 @@ cudaError_t launch_k(const DstPass &a, cudaStream_t st)
     int lines = a.lines > 0 ? a.lines : 0;
     if (!lines) {
         const int64_t all = (int64_t)nu * nv;
-        // Big from twelve of its blocks per SM on (129^3, 508 Big blocks: 250 us per solve
-        // with Big, 235 with Mid; 257^3 and 513^3: Big 3 % and 10 % ahead), Thin below four Mid
-        // blocks per SM (33 x 65 x 97: 117 us per solve with Mid, 77 with Thin)
+        // Big from twelve of its blocks per SM on (passes of a solve, Big and Mid: 129^3,
+        // 508 Big blocks, 197 and 179 us; 257^3 1001 and 1035 us; 513^3 7.8 and 10.8 ms), Thin
+        // below four Mid blocks per SM (33 x 65 x 97: 117 us per solve with Mid, 77 with Thin)
         lines = all >= (int64_t)152 * 12 * S::BIG ? 32 : all >= (int64_t)152 * 4 * S::MID ? 16 : 8;
     }
     if (lines == 32) return launch_cfg<typename S::Big, K>(a, nu, nv, st);

@@ -243,7 +243,7 @@ struct idp_plan_s {
     int *row2 = nullptr, *row1 = nullptr, *sl[3] = {nullptr, nullptr, nullptr};
     double2 *T0 = nullptr, *T1 = nullptr, *part = nullptr, *F = nullptr;
     double *khat[3] = {nullptr, nullptr, nullptr};
-    ddr *khatd[3] = {nullptr, nullptr, nullptr};   // double-float copies (precision DF32)
+    ddr *khatd[3] = {nullptr, nullptr, nullptr};   // double-float copies (IDP_KEY_MIXED_BOUNDARY_DF32)
     int64_t khat_n[3] = {0, 0, 0};
     int2 *kq[3] = {nullptr, nullptr, nullptr};   // fixed-point spectra (FaceQPass) and their exponents
     int *kq_ek[3] = {nullptr, nullptr, nullptr};
