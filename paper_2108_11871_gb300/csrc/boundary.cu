@@ -396,7 +396,7 @@ __global__ void __launch_bounds__(QLineCfg<L, THIN>::T, QLineCfg<L, THIN>::BPS) 
     //    zero and are not read by the first pass
     {
         long long *zl = reinterpret_cast<long long *>(buf + l * LS);
-        const QFrom from(scale, emax);
+        const QFrom from(scale, emax, q_turn(u + blockIdx.x));
 #pragma unroll
         for (int i = 0; i < C; ++i) {
             const int q = g + i * G + 1;   // <= L
@@ -413,7 +413,7 @@ __global__ void __launch_bounds__(QLineCfg<L, THIN>::T, QLineCfg<L, THIN>::BPS) 
     if (ll >= nl) return;
     const qc *zl = buf + ll * LS;
     double2 *ol = outb + (int64_t)ll * osv;
-    const QTo to(s_scale[ll]);
+    const QTo to(s_scale[ll], q_turn(u + blockIdx.x));
 #pragma unroll
     for (int i = 0; i < (L / 2 + G - 1) / G; ++i) {
         const int m = 1 + gg + i * G;   // 1..L/2

@@ -63,7 +63,10 @@ __global__ void __launch_bounds__(FaceQCfg<L>::NT, FaceQCfg<L>::BPS) face_q_kern
     const int chunk = blockIdx.y, diff = blockIdx.z;
     const int npair = (a.np + 1) / 2;
     const int g = *a.gmax;
-    const QFrom from(1102 - min(g, 2100) - a.lgn, g - 31);   // every column's absolute sum below 2^61 units
+    // every column's absolute sum below 2^61 units; signs in turn (q64.cuh) over the blocks and
+    // the pairs of a chunk
+    int turns = blockIdx.x + chunk;
+    QFrom from(1102 - min(g, 2100) - a.lgn, g - 31, q_turn(turns));
     for (int f = threadIdx.x; f < Cfg::TW; f += NT) tws[f] = __ldg(a.q + f);
     const int2 *kq = a.kq + ((int64_t)diff * npair * a.nc + c0) * KS;
 
@@ -143,10 +146,13 @@ __global__ void __launch_bounds__(FaceQCfg<L>::NT, FaceQCfg<L>::BPS) face_q_kern
             for (int q = 0; q < RL; ++q) {
                 const int m = j + q * UL;
                 const int2 w = k[m <= Ph ? m : L - m];
-                acc[it][q].re += q_rmul(v[q].re, w.x, w.y);
-                acc[it][q].im += q_rmul(v[q].im, w.x, w.y);
+                // the sum so far is turned with every pair, as the pair's values are
+                acc[it][q].re = q_rmul(v[q].re, w.x, w.y) - acc[it][q].re;
+                acc[it][q].im = q_rmul(v[q].im, w.x, w.y) - acc[it][q].im;
             }
         }
+        from.flip();
+        ++turns;
         __syncthreads();   // the buffer is free
     }
 #pragma unroll
@@ -154,8 +160,9 @@ __global__ void __launch_bounds__(FaceQCfg<L>::NT, FaceQCfg<L>::BPS) face_q_kern
         const int ct = column(it);
         if (ct >= ncl) continue;
         qc *part = a.part + (((int64_t)chunk * 2 + diff) * a.nc + c0 + ct) * L + freq(it);
+        const bool back = turns & 1;   // the last pair was not turned
 #pragma unroll
-        for (int q = 0; q < RL; ++q) part[q * UL] = acc[it][q];
+        for (int q = 0; q < RL; ++q) part[q * UL] = back ? acc[it][q] : qc{-acc[it][q].re, -acc[it][q].im};
     }
 }
 

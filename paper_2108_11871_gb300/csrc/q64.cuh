@@ -253,10 +253,22 @@ __device__ __forceinline__ unsigned q_weight(double x, int emax)
 }
 __device__ __forceinline__ int q_bits(unsigned S) { return max(32 - __clz((int)S), 21); }
 
-// x 2^s rounded to nearest, |x| 2^s < 2^60
+// Signs in turn.  The parts of a product that are dropped or rounded have a mean that
+// depends on the factor, so that an output of an FFT is off by a few units on average (5 at
+// frequency 1 of length 512), the same ones in every line on the same scale: sums over lines and
+// slices add them up (noise, boundary values: 513^2 off by 4.1e-15, 513 x 33^2 by 3.5e-15, in turns 1.8e-15
+// and 1.5e-15, FP64 1.8e-15 and 1.0e-15).  So every second block of lines goes through its
+// transform with its sign turned, in the exponent word that the conversions change anyway, and its mean
+// errors come out turned as well.  (Not in the sine passes, whose errors are below FP64's without.)
+constexpr unsigned Q_TURN = 0x80000000u;
+__device__ __forceinline__ unsigned q_turn(int k) { return (unsigned)k << 31; }   // odd k
+
+// x 2^s (turn: -x 2^s) rounded to nearest, |x| 2^s < 2^60
 struct QFrom {
     int add, low, s;
-    __device__ __forceinline__ QFrom(int s_, int emax) : add(s_ << 20), s(s_)
+    unsigned turn;
+    __device__ __forceinline__ QFrom(int s_, int emax, unsigned turn_ = 0)
+        : add((int)(((unsigned)s_ << 20) ^ turn_)), s(s_), turn(turn_)
     {
         // values whose exponent field plus s is below 1 give 0 (their half unit is far
         // above them); next to the smallest numbers the general form below runs instead
@@ -279,6 +291,11 @@ struct QFrom {
     {
         return shifted(x, low >= 0 || (__double2hiint(x) & 0x7ff00000) ? 0x100000u : 0u);
     }
+    __device__ __forceinline__ void flip()
+    {
+        add ^= Q_TURN;
+        turn ^= Q_TURN;
+    }
 
 private:
     __device__ __forceinline__ long long shifted(double x, unsigned lead) const
@@ -287,23 +304,27 @@ private:
         const unsigned long long f =
             (((unsigned long long)(((unsigned)h & 0xfffffu) | lead) << 32) | (unsigned)__double2loint(x)) << 10;
         const int r = max(min(1085 - s - q_emax(h & 0x7fffffff), 64), 1);
-        const long long v = (long long)(((f >> (r - 1)) + 1) >> 1), t = h >> 31;
+        const long long v = (long long)(((f >> (r - 1)) + 1) >> 1), t = (int)(h ^ turn) >> 31;
         return (v ^ t) - t;
     }
 };
 constexpr int Q_NAN = 1 << 30;   // scale of a line with a NaN or an infinity
 constexpr int Q_GNAN = 1 << 20;  // emax + bits of such a line in a maximum over lines
-// v 2^-s as FP64
+// v 2^-s (turn: -v 2^-s) as FP64
 struct QTo {
     int sub, s;
     bool fast;   // 2^-s and every |v| keep the result normal
-    __device__ __forceinline__ explicit QTo(int s_) : sub(s_ << 20), s(s_), fast(s_ <= 1022 && s_ >= -960) {}
+    __device__ __forceinline__ explicit QTo(int s_, unsigned turn = 0)
+        : sub((int)(((unsigned)s_ << 20) ^ turn)), s(s_), fast(s_ <= 1022 && s_ >= -960)
+    {
+    }
     __device__ __forceinline__ double operator()(long long v) const
     {
         const double d = __ll2double_rn(v);
         const int h = __double2hiint(d);
         if (fast) return __hiloint2double(h ? h - sub : 0, __double2loint(d));
-        return s == Q_NAN ? __longlong_as_double(0x7ff8000000000000LL) : scalbn(d, -s);
+        if (s == Q_NAN) return __longlong_as_double(0x7ff8000000000000LL);
+        return scalbn(sub != s << 20 ? -d : d, -s);
     }
 };
 
