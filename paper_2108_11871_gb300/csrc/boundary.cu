@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(QLineCfg<L, THIN>::T, QLineCfg<L, THIN>::BPS) 
     qc *buf = smem_q;
     int4 *tws = reinterpret_cast<int4 *>(buf + Cfg::BUF);
     __shared__ int s_high[LB], s_scale[LB], s_any, s_gmax;
-    __shared__ unsigned s_sum[LB];
+    __shared__ unsigned s_sum[LB], s_big[LB];
     int nv;
     int64_t isu, isv, ise, osu, osv, ose;
     if (a.axis == 2) {
@@ -319,6 +319,7 @@ __global__ void __launch_bounds__(QLineCfg<L, THIN>::T, QLineCfg<L, THIN>::BPS) 
     if (threadIdx.x < LB) {
         s_high[threadIdx.x] = 0;
         s_sum[threadIdx.x] = 0;
+        s_big[threadIdx.x] = 0;
     }
     if (threadIdx.x == 0) s_gmax = 0;
     if (mk)
@@ -410,25 +411,56 @@ __global__ void __launch_bounds__(QLineCfg<L, THIN>::T, QLineCfg<L, THIN>::BPS) 
     q_fft<L, Cfg::RM, LB, NT, LS, 1, true>(buf, tws);
     // 5. X'_m = 2 X_m, m = 0..L: G consecutive threads per line
     const int ll = threadIdx.x / G, gg = threadIdx.x % G;
-    if (ll >= nl) return;
-    const qc *zl = buf + ll * LS;
-    double2 *ol = outb + (int64_t)ll * osv;
-    const QTo to(s_scale[ll], q_turn(u + blockIdx.x));
+    unsigned big = 0;   // largest part of an output, in units of 2^32
+    auto part = [&](long long v) {
+        const int h = (int)(v >> 32);
+        big = max(big, (unsigned)(h ^ (h >> 31)));
+        return v;
+    };
+    if (ll < nl) {
+        const qc *zl = buf + ll * LS;
+        double2 *ol = outb + (int64_t)ll * osv;
+        const QTo to(s_scale[ll], q_turn(u + blockIdx.x));
 #pragma unroll
-    for (int i = 0; i < (L / 2 + G - 1) / G; ++i) {
-        const int m = 1 + gg + i * G;   // 1..L/2
-        if ((L / 2) % G != 0 && m > L / 2) break;
-        const qc zm = zl[q_slot(m)], zc = zl[q_slot(L - m)];
-        const long long Er = zm.re + zc.re, Ei = zm.im - zc.im;
-        const qc P = q_cmul(qc{zm.re - zc.re, zm.im + zc.im}, __ldg(a.qhalf + m));   // W O = P; X' = E - i P
-        ol[(int64_t)m * ose] = make_double2(to(Er + P.im), to(Ei - P.re));
-        ol[(int64_t)(L - m) * ose] = make_double2(to(Er - P.im), to(-Ei - P.re));
+        for (int i = 0; i < (L / 2 + G - 1) / G; ++i) {
+            const int m = 1 + gg + i * G;   // 1..L/2
+            if ((L / 2) % G != 0 && m > L / 2) break;
+            const qc zm = zl[q_slot(m)], zc = zl[q_slot(L - m)];
+            const long long Er = zm.re + zc.re, Ei = zm.im - zc.im;
+            const qc P = q_cmul(qc{zm.re - zc.re, zm.im + zc.im}, __ldg(a.qhalf + m));   // W O = P; X' = E - i P
+            ol[(int64_t)m * ose] = make_double2(to(part(Er + P.im)), to(part(Ei - P.re)));
+            ol[(int64_t)(L - m) * ose] = make_double2(to(part(Er - P.im)), to(part(-Ei - P.re)));
+        }
+        if (gg == 0) {
+            const qc z0 = zl[0];
+            const double im = to(0);
+            ol[0] = make_double2(to(part((z0.re + z0.im) << 1)), im);
+            ol[(int64_t)L * ose] = make_double2(to(part((z0.re - z0.im) << 1)), im);
+        }
     }
-    if (gg == 0) {
-        const qc z0 = zl[0];
-        const double im = to(0);
-        ol[0] = make_double2(to((z0.re + z0.im) << 1), im);
-        ol[(int64_t)L * ose] = make_double2(to((z0.re - z0.im) << 1), im);
+    if (!a.sums) return;
+    // 6. the lines' shares of their slices' sums (integers: any order gives the same): half of a
+    //    bound on the line's outputs, its absolute sum or, for rough lines, sqrt(2) times the largest
+    //    part.  (Parts in units of 2^(32 + e + bits - 1102), sums in units of 2^(e + bits - 1064),
+    //    shares in units of 2^(-sh) of that.  With the signs in turn 303 -> 315 us at 257^3.)
+    if constexpr (Cfg::W == 32) big = __reduce_max_sync(0xffffffffu, big);
+    else
+        for (int d = 1; d < Cfg::W; d <<= 1) big = max(big, __shfl_xor_sync(0xffffffffu, big, d));
+    if constexpr (G > 32) {   // the line's warps
+        if ((threadIdx.x & 31) == 0) atomicMax(&s_big[ll], big);
+        __syncthreads();
+        big = s_big[ll];
+    }
+    if (gg == 0 && ll < nl && s_high[ll] > 0) {
+        const unsigned S = s_sum[ll], y = big + 1;
+        const int e = q_emax(s_high[ll]), bits = q_bits(S), sh = (e + bits) & 31;
+        if (e < 0x7ff) {
+            const unsigned long long x = min((unsigned long long)((S >> (bits - 21)) + 1) << sh,
+                                             (((unsigned long long)(y + (y >> 1) + 1) << sh) >> 7) + 1);
+            unsigned long long *w = a.sums + ((e + bits) >> 5) * a.nsum;
+            if (a.sumu >= 0) atomicAdd(w + a.sumu + u, x);
+            atomicAdd(w + a.sumv + v0 + ll, x);
+        }
     }
 }
 
@@ -808,7 +840,7 @@ __global__ void __launch_bounds__(InvbQCfg<L>::T) face_invb_q_kernel(const FaceI
     }
     const int Mb = a.Mb, c0 = blockIdx.x * TC, ncl = min(TC, a.nc - c0);
     const int t = threadIdx.x / G, e = threadIdx.x % G;
-    const int g = *a.gmax, base = 1102 - g - a.lgn;
+    const int g = *a.gmax, base = *a.unit;
     double2 x[2][2];   // [face][frequency e, e + G]
     {
         qc sum[2] = {{0, 0}, {0, 0}}, dif[2] = {{0, 0}, {0, 0}};

@@ -8,12 +8,16 @@
 // sums over the pairs, S and D, give face 0 = S + D and face 1 = S - D.  Against weighing
 // every slice twice this halves the products and reads every spectrum once.
 //
-// Arithmetic (q64.cuh): one scale for all columns and slices of a pass, from a bound on
-// the absolute sum of every line of stage 1; the spectra of each frequency pair (b, c)
-// are fractions of a power of two that bounds their sum over the slices, so that
-// neither a transform nor a sum can overflow.  (One power for all frequencies leaves the
-// products' rounding as white noise over them: measured 1e-12 of g on mixed-sign
-// densities, against 1e-15 with the spectra's decay in the scale.)
+// Arithmetic (q64.cuh): one scale for all columns and slices of a pass, from bounds on the
+// lines of stage 1 summed over each slice (slices x the largest line's bound left a single charged
+// line eight bits short at 257^3: g off by 1.9e-13, with the sums by 2.4e-15, FP64 2.2e-15); the
+// spectra of each frequency pair (b, c) are fractions of a power of two, up to 1 each and up to 4
+// in sum over the slices: a low frequency weighs every slice alike, by a few hundredths at most,
+// and what a product is rounded to counts against that.  So neither a transform nor a sum can
+// overflow: columns are below 2^61 units, S and D below 2^62 and S +- D below 2^63.  (One power
+// for all frequencies leaves the products' rounding as white noise over them: measured 1e-12
+// of g on mixed-sign densities.)  White noise, g off by, with the first bounds and now (FP64): 129^3 5.5e-15 and 1.6e-15
+// (1.5e-15), 257^3 2.5e-14 and 3.8e-15 (2.5e-15), 513^3 8.7e-14 and 4.7e-15 (2.4e-15).
 #include "fft.cuh"
 #include "q64.cuh"
 
@@ -62,12 +66,33 @@ __global__ void __launch_bounds__(FaceQCfg<L>::NT, FaceQCfg<L>::BPS) face_q_kern
     const int c0 = blockIdx.x * TC, ncl = min(TC, a.nc - c0);
     const int chunk = blockIdx.y, diff = blockIdx.z;
     const int npair = (a.np + 1) / 2;
-    const int g = *a.gmax;
-    // every column's absolute sum below 2^61 units; signs in turn (q64.cuh) over the blocks and
-    // the pairs of a chunk
-    int turns = blockIdx.x + chunk;
-    QFrom from(1102 - min(g, 2100) - a.lgn, g - 31, q_turn(turns));
+    const int g = min(*a.gmax, 2100);
     for (int f = threadIdx.x; f < Cfg::TW; f += NT) tws[f] = __ldg(a.q + f);
+    // The unit: every column's absolute sum, at most twice that of the slices' line bounds, below 2^61
+    // units.  b: the largest sum over a pair of slices in units of 2^(32 win - 1064); lines two
+    // windows below the largest one's add up to less than the 1
+    __shared__ int s_bound;
+    if (threadIdx.x == 0) s_bound = 0;
+    __syncthreads();
+    const int win = g >> 5;
+    {
+        float b = 0.0f;
+        for (int pr = threadIdx.x; pr < npair; pr += NT) {
+            const int p2 = a.np - 1 - pr;
+            const unsigned long long *s1 = a.sums + (int64_t)win * a.nsum, *s0 = s1 - a.nsum;
+            const unsigned long long hi = s1[pr] + (p2 > pr ? s1[p2] : 0);
+            const unsigned long long lo = win > 0 ? s0[pr] + (p2 > pr ? s0[p2] : 0) : 0;
+            b = fmaxf(b, __fadd_ru(__ull2float_ru(hi), __fmul_ru(__ull2float_ru(lo), 0x1p-32f)));
+        }
+        const int m = __reduce_max_sync(0xffffffffu, __float_as_int(__fadd_ru(b, 1.0f)));
+        if ((threadIdx.x & 31) == 0) atomicMax(&s_bound, m);
+    }
+    __syncthreads();
+    const int unit = 1124 - ((s_bound >> 23) - 126) - 32 * win;
+    if (threadIdx.x == 0 && blockIdx.x + blockIdx.y + blockIdx.z == 0) *a.unit = unit;
+    // signs in turn (q64.cuh) over the blocks and the pairs of a chunk
+    int turns = blockIdx.x + chunk;
+    QFrom from(unit, g - 31, q_turn(turns));
     const int2 *kq = a.kq + ((int64_t)diff * npair * a.nc + c0) * KS;
 
     // a unit of the last pass: column, frequencies j + q UL
@@ -172,10 +197,13 @@ __global__ void face_kq_kernel(const double *__restrict__ khat, int np, int64_t 
 {
     const int npair = (np + 1) / 2;
     for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < per; x += (int64_t)gridDim.x * blockDim.x) {
-        double sum = 0.0;
-        for (int p = 0; p < np; ++p) sum += fabs(khat[p * per + x]);
+        double sum = 0.0, big = 0.0;
+        for (int p = 0; p < np; ++p) {
+            sum += fabs(khat[p * per + x]);
+            big = fmax(big, fabs(khat[p * per + x]));
+        }
         int e = 0;
-        if (sum > 0.0) frexp(0.5 * sum * (1.0 + 1e-9), &e);
+        if (sum > 0.0) frexp(fmax(0.25 * sum, big) * (1.0 + 1e-9), &e);
         ek[x] = e;
         const double scale = ldexp(0.5, 62 - e);
         for (int p = 0; p < npair; ++p) {

@@ -152,6 +152,10 @@ struct RfftPass {
     int fx;                // 1: fixed-point arithmetic (dd = 0), FP64 in and out
     const int4 *q, *qhalf; // its tables for length P: FFT factors, e^{-i pi m/P}, m = 0..P/2
     int *gmax;             // optional (fx): maximum over the lines of emax + bits (q64.cuh), zero on entry
+    // optional (fx): sums over the lines of a slice (FaceQPass::sums), zero on entry; line (u, v) adds to slices
+    // sumu + u (sumu < 0: not) and sumv + v
+    unsigned long long *sums;
+    int nsum, sumu, sumv;
     double *copy;          // optional: the input is also copied here (same strides)
 };
 cudaError_t launch_rfft_pass(const RfftPass &a, cudaStream_t st);
@@ -184,7 +188,6 @@ struct FaceQPass {
     const double2 *D;          // as FacePass
     int64_t sp, sb, sc;
     int np, Mb, Pb, nc;
-    int lgn;                   // ceil(log2(Mb))
     const int2 *kq;            // [2][(np+1)/2][nc][Pb+1]: (k_p + k_p') / 2 and (k_p - k_p') / 2 as fractions of
                                // 2^ek[c][b]: (bits 62..31, bits 30..0) of the value times 2^(62 - ek)
     qc *part;                  // [nchunk][2][nc][2Pb]
@@ -192,7 +195,13 @@ struct FaceQPass {
     const int4 *q;             // FFT factors of length 2Pb
     const int *sliceflag;      // sliceflag[p] != 0 iff slice p has a non-zero value
     const int *gmax;           // maximum over the lines of D of emax + bits
+    // sums over the lines of slice p (half of each line's bound on its values of D), in windows of 32
+    // exponents: sums[w * nsum + p] in units of 2^(32 w - 1064), w = (emax + bits) / 32 of a line
+    const unsigned long long *sums;
+    int nsum;
+    int *unit;                 // out: the parts are in units of 2^(ek - unit)
 };
+constexpr int FACE_WINDOWS = 66;
 cudaError_t launch_face_q(const FaceQPass &a, cudaStream_t st);
 cudaError_t launch_face_kq(const double *khat, int np, int64_t per, int2 *kq, int *ek, cudaStream_t st);
 cudaError_t face_q_set_attributes();
@@ -218,9 +227,9 @@ struct FaceInvB {
     FftTables t;               // length 2Pb
     int dd;
     int Pb;                    // 0: Mb
-    int fx, lgn;               // 1: parts of FaceQPass, its lgn and ek[nc][Pb+1]
+    int fx;                    // 1: parts of FaceQPass, its unit and ek[nc][Pb+1]
     const int *ek;
-    const int *gmax;
+    const int *gmax, *unit;
     const int4 *q;             // fx: factors of length 2Pb (q64.cuh)
 };
 cudaError_t launch_face_inv_b(const FaceInvB &a, cudaStream_t st);

@@ -238,6 +238,10 @@ struct idp_plan_s {
     double *E0 = nullptr, *E1 = nullptr, *E2 = nullptr, *sin4b = nullptr;   // layers of E = R - R_spec
     double *ld = nullptr;      // per-axis eigenvalues of D2_s (axis s at ldoff[s])
     int64_t ldoff[3] = {0, 0, 0};
+    // zeroed at the start of every solve, one allocation: the slice sums of the face passes
+    // (FaceQPass::sums, slices of axes 0, 1, 2), then the flags
+    unsigned long long *sums = nullptr;
+    int nsum = 0;
     int *flags = nullptr;        // support flags of rho: rows along axes 2 and 1, slices of axes 0, 1, 2
     int64_t nflags = 0;
     int *row2 = nullptr, *row1 = nullptr, *sl[3] = {nullptr, nullptr, nullptr};
@@ -250,6 +254,7 @@ struct idp_plan_s {
     int qchunk[3] = {1, 1, 1};        // chunks of pairs of slices of the fixed-point face passes
     int *gmax[4] = {};                // bounds of the lines along axes 2 and 1 (FaceQPass::gmax), of the layers
                                       // of gtilde and of E; zeroed with the flags
+    int *unit[3] = {};                // units of the parts of the face passes (FaceQPass::unit)
     int2 *sinq = nullptr, *sinq2 = nullptr;   // fixed-point forms of sin4 / 4 and sin4b / 4
     int nchunk[3] = {1, 1, 1}, pchunk[3] = {1, 1, 1};
     int dst_lines = 0;                // lines per block of the full-volume sine passes (0 = default)
@@ -942,13 +947,6 @@ int transform_rho_from_T0(idp_plan p, cudaStream_t st)
     return transform(p, im, p->A, dense(p, p->A), p->tabc2, none, true, st, true, true, dd);
 }
 
-int ceil_log2(int n)
-{
-    int e = 0;
-    while ((1 << e) < n) ++e;
-    return e;
-}
-
 // about n chunks of the np slices of a face pass, no more than pairs: ceil(np / slices per chunk)
 int face_q_chunks(int np, int n)
 {
@@ -968,13 +966,15 @@ int face_q_pass(idp_plan p, int a_, int nchunk, double2 *part, FaceQPass *q, Fac
     q->sb = a_ == 0 ? r2 : a_ == 1 ? p->ni[1] * r2 : p->ni[2] * r1;
     q->sc = 1;
     q->np = p->ni[a_]; q->Mb = p->M[b]; q->Pb = p->P[b]; q->nc = p->P[c] + 1;
-    q->lgn = ceil_log2(p->M[b]);
     q->kq = p->kq[a_];
     q->part = reinterpret_cast<qc *>(part);
     q->nchunk = nchunk;
     q->sliceflag = p->sl[a_];
     q->gmax = p->gmax[a_ == 2 ? 1 : 0];
-    ib->fx = 1; ib->nchunk = nchunk; ib->lgn = q->lgn; ib->ek = p->kq_ek[a_]; ib->gmax = q->gmax;
+    q->sums = p->sums + (a_ == 0 ? 0 : a_ == 1 ? p->ni[0] : p->ni[0] + p->ni[1]);
+    q->nsum = p->nsum;
+    q->unit = p->unit[a_];
+    ib->fx = 1; ib->nchunk = nchunk; ib->ek = p->kq_ek[a_]; ib->gmax = q->gmax; ib->unit = q->unit;
     const int4 *half;
     const int rc = get_fft_tables(p, 2 * p->P[b], &q->q, &half);
     ib->q = q->q;
@@ -998,7 +998,7 @@ int boundary(idp_plan p, const double *rho, double *dst0, double *dst1, cudaStre
     const int dd = boundary_dd(p);
     const int fx = stage ? !dd : boundary_fx(p);
     // support flags of rho: set by the first row transform
-    IDP_CK(cudaMemsetAsync(p->flags, 0, sizeof(int) * p->nflags, st));
+    IDP_CK(cudaMemsetAsync(p->sums, 0, (size_t)((char *)(p->flags + p->nflags) - (char *)p->sums), st));
     // stage 1a: along axis 2 -> T0[i0][i1][m2]; stage 1b: along axis 1 -> T1[i0][i2][m1]
     RfftPass a2{}, a1{};
     a2.in = rho_src ? node_interior(p, rho_src).p : r.p;
@@ -1013,6 +1013,14 @@ int boundary(idp_plan p, const double *rho, double *dst0, double *dst1, cudaStre
     a2.fx = a1.fx = fx;
     a2.gmax = p->gmax[0];
     a1.gmax = p->gmax[1];
+    if (fx && p->d == 3) {
+        a2.sums = a1.sums = p->sums;
+        a2.nsum = a1.nsum = p->nsum;
+        a2.sumu = 0;
+        a2.sumv = p->ni[0];
+        a1.sumu = -1;
+        a1.sumv = p->ni[0] + p->ni[1];
+    }
     if ((rc = get_fft_tables(p, p->P[2], &a2.q, &a2.qhalf))) return rc;
     a2.dd = dd;
     // the pass along axis 2 reads every value of rho once: it also marks which
@@ -1450,8 +1458,11 @@ int plan_setup(idp_plan p)
     }
     {
         const int64_t n0 = p->ni[0], n1 = p->ni[1], n2 = p->ni[2];
-        p->nflags = n0 * n1 + n0 * n2 + n0 + n1 + n2 + 4;
-        if ((rc = p->alloc(&p->flags, p->nflags))) return rc;
+        p->nflags = n0 * n1 + n0 * n2 + n0 + n1 + n2 + 7;
+        p->nsum = (int)(n0 + n1 + n2);
+        const int64_t ns = p->d == 3 ? (int64_t)FACE_WINDOWS * p->nsum : 0;
+        if ((rc = p->alloc(&p->sums, ns + (p->nflags + 1) / 2))) return rc;
+        p->flags = reinterpret_cast<int *>(p->sums + ns);
         p->row2 = p->flags;
         p->row1 = p->row2 + n0 * n1;
         p->sl[0] = p->row1 + n0 * n2;
@@ -1459,6 +1470,7 @@ int plan_setup(idp_plan p)
         p->sl[2] = p->sl[1] + n1;
         p->gmax[0] = p->sl[2] + n2;
         for (int i = 1; i < 4; ++i) p->gmax[i] = p->gmax[0] + i;
+        for (int i = 0; i < 3; ++i) p->unit[i] = p->gmax[3] + 1 + i;
     }
     if ((rc = plan_streams(p))) return rc;
     {

@@ -17,7 +17,7 @@ def _error(n, rho, count):
     idx = ogreens.boundary_indices(n)
     t = idx[np.random.default_rng(0).choice(len(idx), count, replace=False)]
     ref = ogreens.boundary_direct(rho, h, t)
-    plan = idp.create_plan(len(n), n, h, 4)
+    plan = idp.create_plan(len(n), n, h, 4, exact=max(n) == 300)
     r = torch.from_numpy(np.ascontiguousarray(rho)).cuda()
     out = torch.empty_like(r)
     idp.solve_stage(plan, idp.IDP_STAGE_BOUNDARY, r, out)
@@ -30,3 +30,34 @@ def test_mean_errors_do_not_add_up_over_lines(n):
     # the spectra of the kernel, in FP64, are sums of up to 512 terms rounded at 2^-53 each:
     # 23 * 2^-53; errors of the transforms that add up over the lines and slices come on top
     assert _error(n, w.random_interior(n, seed=3), 200) <= 24 * 2.0 ** -53
+
+
+def _density(kind, n):
+    rho = np.zeros(n)
+    noise = w.random_interior(n, seed=3)
+    if kind == "noise":
+        return noise
+    mid = tuple(k // 2 for k in n)
+    if kind == "line":
+        rho[mid[0], mid[1]] = noise[mid[0], mid[1]]
+    elif kind == "points":   # two large charges on faint noise
+        rho = 1e-6 * noise
+        rho[mid], rho[tuple(k // 3 for k in n)] = 1.0, -0.7
+    elif kind == "plane":    # every frequency of one slice next to a face
+        rho[1, 1:-1, 1:-1] = 1.0
+    else:                    # one sign throughout: the sums reach their bounds
+        rho[1:-1, 1:-1, 1:-1] = 1.0
+    return rho
+
+
+@pytest.mark.parametrize("n", [(193, 193, 193), (257, 257, 257), (385, 385, 33), (513, 513, 33), (300, 20, 25)],
+                         ids=lambda n: "x".join(map(str, n)))
+@pytest.mark.parametrize("kind", ["noise", "line", "points", "plane", "constant"])
+def test_the_unit_follows_the_charge(n, kind):
+    # The face passes' unit follows the sum of the line bounds of a pair of slices, within a factor of
+    # two: where few lines are charged, and on noise, whose lines' spectra are far below their absolute sums, it is
+    # no coarser than what FP64 would lose.  64 * 2^-53: the spectra's 23 (above), and as
+    # much again for each of the two transforms.  Points: a point's spectrum does not fall, and the
+    # FP64 spectra of the kernel alone leave 3e-14 of the largest value, 270 * 2^-53
+    tol = (64 if kind != "points" else 400) * 2.0 ** -53
+    assert _error(n, _density(kind, n), 60) <= tol
