@@ -460,6 +460,9 @@ __global__ void __launch_bounds__(QLineCfg<L, THIN>::T, QLineCfg<L, THIN>::BPS) 
             unsigned long long *w = a.sums + ((e + bits) >> 5) * a.nsum;
             if (a.sumu >= 0) atomicAdd(w + a.sumu + u, x);
             atomicAdd(w + a.sumv + v0 + ll, x);
+            // a part of 2^1022 or more: it, or its sum with the mirrored slice's, may have
+            // overflowed, and the face pass converts an infinity to some integer
+            if (32 - __clz((int)big) + e + bits > 2092) atomicMax(a.gmax, Q_GNAN);
         }
     }
 }

@@ -61,3 +61,28 @@ def test_the_unit_follows_the_charge(n, kind):
     # FP64 spectra of the kernel alone leave 3e-14 of the largest value, 270 * 2^-53
     tol = (64 if kind != "points" else 400) * 2.0 ** -53
     assert _error(n, _density(kind, n), 60) <= tol
+
+
+@pytest.mark.parametrize("n", [(33, 49, 17), (65, 65, 65), (49, 65)], ids=lambda n: "x".join(map(str, n)))
+def test_sums_past_the_range_are_not_finite(n):
+    # densities whose transforms overflow: a boundary value is the scaled one or not finite
+    import torch
+    import paper_2108_11871_gb300 as idp
+    plan = idp.create_plan(len(n), n, [1.0 / (max(n) - 1)] * len(n), 4)
+
+    def g(rho):
+        r = torch.from_numpy(rho).cuda()
+        out = torch.empty_like(r)
+        idp.solve_stage(plan, idp.IDP_STAGE_BOUNDARY, r, out)
+        torch.cuda.synchronize()
+        return out.cpu().numpy()
+
+    x = np.meshgrid(*[np.linspace(-1.0, 1.0, k) for k in n], indexing="ij")
+    for rho in (np.maximum(0.0, 1.0 - sum(c * c for c in x)) ** 6, w.random_interior(n, seed=3)):
+        base = g(rho)
+        for power in range(1008, 1024):
+            got = g(np.ldexp(rho, power))
+            with np.errstate(over="ignore"):
+                ref = np.ldexp(base, power)
+            assert (~np.isfinite(got) | (got == ref)).all(), power
+        assert not np.isfinite(got[ogreens.boundary_mask(n)]).any()
