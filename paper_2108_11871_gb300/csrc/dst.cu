@@ -16,7 +16,6 @@
 // shared memory 34-47 %, in turns, because the blocks of an SM are in different phases; half
 // of the warps fit (64 registers).  In FP64 the pass was bound by the FP64 pipe: 250 us at
 // 257^3, 3.9 ms at 513^3 (now 0.98).
-#include "arith.cuh"
 #include "q64.cuh"
 
 namespace idp {
@@ -112,19 +111,20 @@ __global__ void __launch_bounds__(Cfg::T, Cfg::BPS) dst_pass_kernel(const DstPas
             xa[i] = on ? *(mid ? in + (int64_t)(K - 1) * ise : pa) : 0.0;
             xb[i] = on && !mid ? *pb : 0.0;
         }
-        if (a.in_dd) {
-#pragma unroll
-            for (int i = 0; i < C; ++i) {
-                xa[i] = dd_to_bits(*reinterpret_cast<const ddr *>(&xa[i]));
-                xb[i] = dd_to_bits(*reinterpret_cast<const ddr *>(&xb[i]));
-            }
-        }
     }
 
     // 2. the line's scale, from its largest exponent and its absolute sum (q64.cuh)
     int high = 0;
 #pragma unroll
     for (int i = 0; i < C; ++i) high = max(high, max(q_high(xa[i]), q_high(xb[i])));
+    // values that are not finite stay out of the conversions: the line's marker stands for them.
+    // (With many values a thread the compiler mixes the loads and the reductions without a branch
+    // here, 112 -> 123 us a pass at 257^3; short launches are faster without it, 33 x 65 x 97
+    // 142 -> 137 us per solve.)
+    if (C > 4 && high >= 0x7ff00000) {
+#pragma unroll
+        for (int i = 0; i < C; ++i) xa[i] = xb[i] = 0.0;
+    }
     // lanes of one line: G consecutive ones, or those LB apart
     const int d0 = contig ? 1 : LB, d1 = contig ? G : 32;
     for (int d = d0; d < d1; d <<= 1) high = max(high, __shfl_xor_sync(0xffffffffu, high, d));
@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(Cfg::T, Cfg::BPS) dst_pass_kernel(const DstPas
     //    (U_{e+1}); consecutive threads again on consecutive e or on consecutive lines
     int64_t osu, osv, ose;
     view_strides(a.out, a.axis, osu, osv, ose);
-    if (WIDE && contig && !a.tab && !a.add.p) {
+    if (WIDE && contig && !a.tab) {
         // lines along axis 2: a warp writes its lines one after the other, 32 outputs at a time,
         // in half as many pieces of 128-byte lines as the mapping below has: nothing to gain in
         // device memory (257^3: 114.5 us a pass either way), but phi in host memory goes out over
@@ -253,39 +253,32 @@ __global__ void __launch_bounds__(Cfg::T, Cfg::BPS) dst_pass_kernel(const DstPas
         const int e = g + i * G, h = e >> 1;
         return w0[((e & 1) ? 0 : Cfg::OD) + q_slot(h)];
     };
-    if (!a.tab && !a.add.p) {
+    if (!a.tab) {
 #pragma unroll
         for (int i = 0; i < 2 * C; ++i, out += step)
             if (i < 2 * C - 1 || g + i * G < N) *out = to(word(i));
         return;
     }
-    int64_t asu, asv, ase, tsu, tsv, tse;
-    view_strides(a.add, a.axis, asu, asv, ase);
-    // the tables are dense interior arrays n0 x n1 x n2
+    int64_t tsu, tsv, tse;
+    // the table is a dense interior array n0 x n1 x n2
     view_strides(View3{nullptr, (int64_t)a.n1 * a.n2, a.n2, 1}, a.axis, tsu, tsv, tse);
     const double *tab = a.tab + ((int64_t)u * tsu + (int64_t)(v0 + l) * tsv + (int64_t)g * tse);
-    const double *add = a.add.p + ((int64_t)u * asu + (int64_t)(v0 + l) * asv + (int64_t)g * ase);
-    // groups of EG outputs: the table and addend loads of a group go out before
-    // its stores (which, as far as the compiler knows, could alias them)
+    // groups of EG outputs: the table loads of a group go out before its stores (which, as
+    // far as the compiler knows, could alias them)
     constexpr int EG = (2 * C) % 4 == 0 ? 4 : 2;
 #pragma unroll
     for (int i0 = 0; i0 < 2 * C; i0 += EG) {
-        double tv[EG], av[EG];
+        double tv[EG];
 #pragma unroll
         for (int q = 0; q < EG; ++q) {
             const int i = i0 + q;
-            const bool on = i < 2 * C - 1 || g + i * G < N;
-            tv[q] = on && a.tab ? tab[(int64_t)(i * G) * tse] : 1.0;
-            av[q] = on && a.add.p ? add[(int64_t)(i * G) * ase] : 0.0;
+            tv[q] = i < 2 * C - 1 || g + i * G < N ? tab[(int64_t)(i * G) * tse] : 1.0;
         }
 #pragma unroll
         for (int q = 0; q < EG; ++q, out += step) {
             const int i = i0 + q;
             if (i == 2 * C - 1 && g + i * G >= N) break;
-            double y = to(word(i));
-            if (a.tab) y = a.add.p ? fma(tv[q], y, av[q]) : tv[q] * y;
-            else y += av[q];
-            *out = y;
+            *out = tv[q] * to(word(i));
         }
     }
 }

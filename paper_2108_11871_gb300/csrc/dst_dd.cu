@@ -206,9 +206,8 @@ __global__ void __launch_bounds__(NTB) dst_dd_kernel(const DstPass a)
     __syncthreads();
 
     // 6. epilogue and store
-    int64_t osu, osv, ose, asu, asv, ase, tsu, tsv, tse;
+    int64_t osu, osv, ose, tsu, tsv, tse;
     view_strides(a.out, a.axis, osu, osv, ose);
-    view_strides(a.add, a.axis, asu, asv, ase);
     {
         // the tables are dense interior arrays n0 x n1 x n2
         const View3 tv{nullptr, (int64_t)a.n1 * a.n2, a.n2, 1};
@@ -216,9 +215,8 @@ __global__ void __launch_bounds__(NTB) dst_dd_kernel(const DstPass a)
     }
     const int64_t outb = (int64_t)u * osu + (int64_t)v0 * osv;
     const int64_t tabb = (int64_t)u * tsu + (int64_t)v0 * tsv;
-    const int64_t addb = (int64_t)u * asu + (int64_t)v0 * asv;
     const bool has_tab = a.tab || a.tabd;
-    if (!has_tab && !a.add.p) {
+    if (!has_tab) {
         for (int f = threadIdx.x; f < LB * N; f += NT) {
             int l, e;
             if (contig) { l = f / N; e = f - l * N; }
@@ -228,25 +226,22 @@ __global__ void __launch_bounds__(NTB) dst_dd_kernel(const DstPass a)
         }
         return;
     }
-    // groups of EG outputs: the table and addend loads of a group go out before
-    // its stores (which, as far as the compiler knows, could alias them)
+    // groups of EG outputs: the table loads of a group go out before its stores
+    // (which, as far as the compiler knows, could alias them)
     constexpr int EG = 4;
     for (int f0 = threadIdx.x; f0 < LB * N; f0 += EG * NT) {
-        R tv[EG], av[EG];
+        R tv[EG];
 #pragma unroll
         for (int g = 0; g < EG; ++g) {
             const int f = f0 + g * NT;
             tv[g] = A::zero();
-            av[g] = A::zero();
             if (f >= LB * N) continue;
             int l, e;
             if (contig) { l = f / N; e = f - l * N; }
             else { e = f / LB; l = f - e * LB; }
             if (l >= nl) continue;
             const int64_t ti = tabb + (int64_t)l * tsv + (int64_t)e * tse;
-            const int64_t ai = addb + (int64_t)l * asv + (int64_t)e * ase;
-            if (has_tab) tv[g] = Io<R>::ld(a.tabd ? (const void *)a.tabd : (const void *)a.tab, ti, a.tabd != nullptr);
-            if (a.add.p) av[g] = Io<R>::ld(a.add.p, ai, a.add_dd);
+            tv[g] = Io<R>::ld(a.tabd ? (const void *)a.tabd : (const void *)a.tab, ti, a.tabd != nullptr);
         }
 #pragma unroll
         for (int g = 0; g < EG; ++g) {
@@ -256,14 +251,7 @@ __global__ void __launch_bounds__(NTB) dst_dd_kernel(const DstPass a)
             if (contig) { l = f / N; e = f - l * N; }
             else { e = f / LB; l = f - e * LB; }
             if (l >= nl) continue;
-            R y = o[l * M + e];
-            if (has_tab) {
-                if (a.add.p) y = A::fma(tv[g], y, av[g]);
-                else y = A::mul(tv[g], y);
-            } else {
-                y = A::add(y, av[g]);
-            }
-            Io<R>::st(a.out.p, outb + (int64_t)l * osv + (int64_t)e * ose, y, a.out_dd);
+            Io<R>::st(a.out.p, outb + (int64_t)l * osv + (int64_t)e * ose, A::mul(tv[g], o[l * M + e]), a.out_dd);
         }
     }
 }
@@ -315,16 +303,14 @@ __global__ void __launch_bounds__(NT) dst_direct_kernel(const DstPass a)
             for (int l = 0; l < LBD; ++l) acc[j][l] = A::fma(sv, xs[l * N + i], acc[j][l]);
         }
     }
-    int64_t osu, osv, ose, asu, asv, ase, tsu, tsv, tse;
+    int64_t osu, osv, ose, tsu, tsv, tse;
     view_strides(a.out, a.axis, osu, osv, ose);
-    view_strides(a.add, a.axis, asu, asv, ase);
     {
         const View3 tv{nullptr, (int64_t)a.n1 * a.n2, a.n2, 1};
         view_strides(tv, a.axis, tsu, tsv, tse);
     }
     const int64_t outb = (int64_t)u * osu + (int64_t)v0 * osv;
     const int64_t tabb = (int64_t)u * tsu + (int64_t)v0 * tsv;
-    const int64_t addb = (int64_t)u * asu + (int64_t)v0 * asv;
     const bool has_tab = a.tab || a.tabd;
 #pragma unroll
     for (int j = 0; j < DMAX; ++j) {
@@ -335,14 +321,8 @@ __global__ void __launch_bounds__(NT) dst_direct_kernel(const DstPass a)
             if (l >= nl) break;
             R y = times4_exact(acc[j][l]);
             const int64_t ti = tabb + (int64_t)l * tsv + (int64_t)e * tse;
-            const int64_t ai = addb + (int64_t)l * asv + (int64_t)e * ase;
-            if (has_tab) {
-                const R t = Io<R>::ld(a.tabd ? (const void *)a.tabd : (const void *)a.tab, ti, a.tabd != nullptr);
-                if (a.add.p) y = A::fma(t, y, Io<R>::ld(a.add.p, ai, a.add_dd));
-                else y = A::mul(t, y);
-            } else if (a.add.p) {
-                y = A::add(y, Io<R>::ld(a.add.p, ai, a.add_dd));
-            }
+            if (has_tab)
+                y = A::mul(Io<R>::ld(a.tabd ? (const void *)a.tabd : (const void *)a.tab, ti, a.tabd != nullptr), y);
             Io<R>::st(a.out.p, outb + (int64_t)l * osv + (int64_t)e * ose, y, a.out_dd);
         }
     }

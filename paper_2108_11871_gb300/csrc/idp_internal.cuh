@@ -41,10 +41,10 @@ struct View3 {
 // One sine-transform pass along `axis` of an interior-index box n0 x n1 x n2
 // (every extent along `axis` equals M-1).  Each line x -> U with U = 4 * S x,
 // S_{k,i} = sin(pi k i / M); then the epilogue
-//     out = (tab ? tab * U : U) + (add ? add : 0)
-// with tab laid out densely over the box and `add` a strided view.
+//     out = tab ? tab * U : U
+// with tab laid out densely over the box.
 struct DstPass {
-    View3 in, out, add;
+    View3 in, out;
     const double *tab;
     int n0, n1, n2;
     int axis;
@@ -52,14 +52,13 @@ struct DstPass {
     // fixed-point tables (q64.cuh): the factors of the complex FFT of
     // length K = M/2 pass by pass, e^{-i pi k/K} (k = 0..K/2), sin(pi j/M) (j = 0..K-1)
     const int4 *qtab;
-    int in_dd;             // the input holds double-float pairs
     int *gmax;             // optional (fixed-point passes): maximum over the lines of emax + bits (q64.cuh), which
                            // bounds every output by 2^(gmax - 1041); zero on entry
     int lines;   // lines per block: 0 = by size, 8 = fewest, 16, 32 = most
-    // double-float variant (dd = 1): arithmetic on the FP32 pipe; in/out/add
-    // may hold FP64 values or double-float pairs (in_dd / out_dd / add_dd)
+    // double-float variant (dd = 1): arithmetic on the FP32 pipe; in and out
+    // may hold FP64 values or double-float pairs (in_dd / out_dd)
     int dd;
-    int out_dd, add_dd;
+    int in_dd, out_dd;
     const ddr *tabd;       // tab as double-float pairs (if not null, used instead of tab)
     const TwD *twd;        // twiddles for the complex FFT of length M/2
     const ddc *halfd;      // half-step twiddles for length M/2 (e^{-i pi k/(M/2)})

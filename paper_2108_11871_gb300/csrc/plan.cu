@@ -705,7 +705,7 @@ int get_mp_image(idp_plan p, int M, int variant, const void **out)
 
 // Sine transform of all active axes with the tensor-core pass (mixed.cu).
 // The passes rotate the axes: (a,b,c) -> (c',a,b) -> (b',c',a) -> (a',b',c').
-int transform_mixed(idp_plan p, View3 in, View3 out, const double *tab, View3 add, int sidx, cudaStream_t st)
+int transform_mixed(idp_plan p, View3 in, View3 out, const double *tab, int sidx, cudaStream_t st)
 {
     const int n0 = p->ni[0], n1 = p->ni[1], n2 = p->ni[2];
     float *ta = p->t32[sidx][0], *tb = p->t32[sidx][1];
@@ -737,12 +737,11 @@ int transform_mixed(idp_plan p, View3 in, View3 out, const double *tab, View3 ad
     }
     // last pass: FP64 output in the original layout with the epilogue
     const int s0 = p->d == 3 ? 0 : 1;   // output axis of the modes
-    const int64_t os[3] = {out.s0, out.s1, out.s2}, as[3] = {add.s0, add.s1, add.s2};
+    const int64_t os[3] = {out.s0, out.s1, out.s2};
     const int64_t ts[3] = {p->is[0], p->is[1], p->is[2]};
     a.out = out.p; a.out_f64 = 1;
     a.os_m = os[s0]; a.os_p = p->d == 3 ? os[1] : 0; a.os_q = os[2];
     a.tab = tab; a.ts_m = ts[s0]; a.ts_p = p->d == 3 ? ts[1] : 0; a.ts_q = ts[2];
-    a.add = add.p; a.as_m = as[s0]; a.as_p = p->d == 3 ? as[1] : 0; a.as_q = as[2];
     ps.push_back(a);
     // pass i transforms axis 2, 1, 0 (3-D) / 2, 1 (2-D) of the original array
     const int axes3[3] = {2, 1, 0}, axes2[2] = {2, 1};
@@ -761,18 +760,18 @@ int transform_mixed(idp_plan p, View3 in, View3 out, const double *tab, View3 ad
 }
 
 // one full sine transform (all active axes); `first` pass reads `in`, the
-// last pass applies the epilogue (tab, add) and writes `out`; intermediate
+// last pass applies the epilogue (tab) and writes `out`; intermediate
 // passes run in place on `work`.
 // allow_reduced = false: FP64 passes in every precision mode except that
 // fp64_only = false lets the tensor-core modes run them as double-float passes
 // (the transform producing u1: FP64-class there, never the tensor cores)
-int transform(idp_plan p, View3 in, double *work, View3 out, const double *tab, View3 add, bool forward,
-              cudaStream_t st, bool allow_reduced = true, bool skip_axis2 = false, int in_dd0 = 0,
+int transform(idp_plan p, View3 in, double *work, View3 out, const double *tab, bool forward, cudaStream_t st,
+              bool allow_reduced = true, bool skip_axis2 = false, int in_dd0 = 0,
               bool fp64_only = true)
 {
     Range rg(p, forward ? "idp:sine transform (forward)" : "idp:sine transform (inverse)");
     if (tensor_mode(p) && allow_reduced && p->mixed_path == 0)
-        return transform_mixed(p, in, out, tab, add, st == p->side ? 1 : 0, st);
+        return transform_mixed(p, in, out, tab, st == p->side ? 1 : 0, st);
     // df32 passes: precision DF32, or precision MIXED when the autotuner found the
     // double-float FFT faster than the matrix pass (it is also more accurate), or the
     // double-float transform of u1 in the tensor-core modes
@@ -792,7 +791,6 @@ int transform(idp_plan p, View3 in, double *work, View3 out, const double *tab, 
         a.lines = p->dst_lines;
         a.in = (q == 0) ? in : dense(p, work);
         a.out = (q == na - 1) ? out : dense(p, work);
-        a.add = (q == na - 1) ? add : View3{nullptr, 0, 0, 0};
         a.tab = (q == na - 1) ? tab : nullptr;
         a.n0 = p->ni[0]; a.n1 = p->ni[1]; a.n2 = p->ni[2];
         a.axis = s;
@@ -843,7 +841,7 @@ int dst_box(idp_plan p, double *x, int b0, int b1, int b2, int M2, int M1, cudaS
         if (Ms[q] <= 0) continue;
         DstPass a{};
         const View3 v{x, (int64_t)b1 * b2, b2, 1};
-        a.in = v; a.out = v; a.add = View3{nullptr, 0, 0, 0}; a.tab = nullptr;
+        a.in = v; a.out = v; a.tab = nullptr;
         a.n0 = b0; a.n1 = b1; a.n2 = b2;
         a.axis = axes[q];
         a.M = Ms[q];
@@ -940,11 +938,10 @@ int e_layers(idp_plan p, cudaStream_t st, bool conc)
 // on that data and the factor -2 is in tabc2.
 int transform_rho_from_T0(idp_plan p, cudaStream_t st)
 {
-    const View3 none{nullptr, 0, 0, 0};
     const int64_t row = 2 * (int64_t)(p->P[2] + 1);   // doubles per T0 row
     const View3 im{reinterpret_cast<double *>(p->T0) + 3, (int64_t)p->ni[1] * row, row, 2};
     const int dd = boundary_dd(p);   // T0 holds pairs
-    return transform(p, im, p->A, dense(p, p->A), p->tabc2, none, true, st, true, true, dd);
+    return transform(p, im, p->A, dense(p, p->A), p->tabc2, true, st, true, true, dd);
 }
 
 // about n chunks of the np slices of a face pass, no more than pairs: ceil(np / slices per chunk)
@@ -1170,7 +1167,6 @@ enum { RUN_PHI = 0 };
 // the two ends and the straight line through them added inside
 int enqueue_1d(idp_plan p, const double *rho, double *phi, int stop, cudaStream_t st)
 {
-    const View3 none{nullptr, 0, 0, 0};
     const size_t node_bytes = sizeof(double) * p->nodes;
     const int M = p->M[2];
     if (stop == 0 && p->hio_rho)
@@ -1183,8 +1179,8 @@ int enqueue_1d(idp_plan p, const double *rho, double *phi, int stop, cudaStream_
     if (stop != 0 && stop != IDP_STAGE_PHISTAR) return IDP_ESUPPORT;
     int rc;
     if (stop == IDP_STAGE_PHISTAR) IDP_CK(cudaMemsetAsync(phi, 0, node_bytes, st));
-    if ((rc = transform(p, node_interior(p, rho), p->A, dense(p, p->A), p->tabc, none, true, st))) return rc;
-    if ((rc = transform(p, dense(p, p->A), p->A, node_interior(p, phi), nullptr, none, false, st))) return rc;
+    if ((rc = transform(p, node_interior(p, rho), p->A, dense(p, p->A), p->tabc, true, st))) return rc;
+    if ((rc = transform(p, dense(p, p->A), p->A, node_interior(p, phi), nullptr, false, st))) return rc;
     if (stop == IDP_STAGE_PHISTAR) return IDP_OK;
     Mark mk(p, IDP_KERNEL_LINE1D, st);
     IDP_CK(launch_line1d(rho, phi, M, p->h[2], LINE1D_ADD, st));
@@ -1255,7 +1251,6 @@ int enqueue_grid(idp_plan p, const double *rho, double *phi, int stop, cudaStrea
 {
     if (p->d == 1) return enqueue_1d(p, rho, phi, stop, st);
     int rc;
-    const View3 none{nullptr, 0, 0, 0};
     const size_t node_bytes = sizeof(double) * p->nodes;
     if (stop == IDP_STAGE_BOUNDARY) {
         IDP_CK(cudaMemsetAsync(phi, 0, node_bytes, st));
@@ -1263,8 +1258,8 @@ int enqueue_grid(idp_plan p, const double *rho, double *phi, int stop, cudaStrea
     }
     if (stop == IDP_STAGE_PHISTAR) {
         IDP_CK(cudaMemsetAsync(phi, 0, node_bytes, st));
-        if ((rc = transform(p, node_interior(p, rho), p->A, dense(p, p->A), p->tabc, none, true, st))) return rc;
-        return transform(p, dense(p, p->A), p->A, node_interior(p, phi), nullptr, none, false, st);
+        if ((rc = transform(p, node_interior(p, rho), p->A, dense(p, p->A), p->tabc, true, st))) return rc;
+        return transform(p, dense(p, p->A), p->A, node_interior(p, phi), nullptr, false, st);
     }
     // 0. the forward transform of rho does not depend on the boundary values:
     //    queue it on the side stream so it overlaps the boundary convolutions
@@ -1288,7 +1283,7 @@ int enqueue_grid(idp_plan p, const double *rho, double *phi, int stop, cudaStrea
     if (overlap_rho && !rho_from_T0) {
         IDP_CK(cudaEventRecord(p->fork, st));
         IDP_CK(cudaStreamWaitEvent(p->side, p->fork, 0));
-        if ((rc = transform(p, node_interior(p, rho), p->A, dense(p, p->A), nullptr, none, true, p->side)))
+        if ((rc = transform(p, node_interior(p, rho), p->A, dense(p, p->A), nullptr, true, p->side)))
             return rc;
         IDP_CK(cudaEventRecord(p->join, p->side));
     }
@@ -1307,7 +1302,7 @@ int enqueue_grid(idp_plan p, const double *rho, double *phi, int stop, cudaStrea
     if (stop == 0 && !overlap_rho) {
         if (rho_from_T0) {
             if ((rc = transform_rho_from_T0(p, st))) return rc;
-        } else if ((rc = transform(p, node_interior(p, rho), p->A, dense(p, p->A), nullptr, none, true, st))) {
+        } else if ((rc = transform(p, node_interior(p, rho), p->A, dense(p, p->A), nullptr, true, st))) {
             return rc;
         }
     }
@@ -1321,7 +1316,7 @@ int enqueue_grid(idp_plan p, const double *rho, double *phi, int stop, cudaStrea
                                 : launch_gtilde_expand(p->grid, p->Q0, p->Q1, p->Q2, p->sin4, p->tab4, p->A, p->A,
                                                        st, nullptr, nullptr, nullptr, 0, ascale));
         }
-        return transform(p, dense(p, p->A), p->A, node_interior(p, phi), nullptr, none, false, st);
+        return transform(p, dense(p, p->A), p->A, node_interior(p, phi), nullptr, false, st);
     }
     // 4. u1 = S B, B = tab4 * S gtilde; in a full solve also C = A + tabR * S gtilde,
     //    the solution coefficients less the layer correction (R_spec's share)
@@ -1338,7 +1333,7 @@ int enqueue_grid(idp_plan p, const double *rho, double *phi, int stop, cudaStrea
     // u1 feeds the sixth differences of R, which amplify its rounding by ~1e4-1e7:
     // this inverse transform stays FP64 in the FP64 and DF32 modes, and is a
     // double-float one (48 bits, never the tensor cores) in the tensor-core modes
-    if ((rc = transform(p, dense(p, p->B), p->B, node_interior(p, p->U), nullptr, none, false, st, false, false, 0,
+    if ((rc = transform(p, dense(p, p->B), p->B, node_interior(p, p->U), nullptr, false, st, false, false, 0,
                         false)))
         return rc;
     if (stop == IDP_STAGE_U1) {
@@ -1370,7 +1365,7 @@ int enqueue_grid(idp_plan p, const double *rho, double *phi, int stop, cudaStrea
                                                        p->C, st));
         }
         IDP_CK(launch_rhs6_symbol(p->grid, p->ld, p->ldoff[1], p->ldoff[2], p->C, st));
-        if ((rc = transform(p, dense(p, p->C), p->C, dense(p, phi), nullptr, none, false, st, false))) return rc;
+        if ((rc = transform(p, dense(p, p->C), p->C, dense(p, phi), nullptr, false, st, false))) return rc;
         IDP_CK(launch_rhs6_e_scatter(p->grid, p->E0, p->E1, p->E2, phi, st));
         return IDP_OK;
     }
@@ -1383,7 +1378,7 @@ int enqueue_grid(idp_plan p, const double *rho, double *phi, int stop, cudaStrea
                             : launch_rhs6_e_expand(p->grid, p->E0, p->E1, p->E2, p->sin4, p->sin4b, p->tab4, p->C,
                                                    st));
     }
-    return transform(p, dense(p, p->C), p->C, node_interior(p, phi), nullptr, none, false, st);
+    return transform(p, dense(p, p->C), p->C, node_interior(p, phi), nullptr, false, st);
 }
 
 // the plan's streams and events (graph capture forks and joins through them)
@@ -1807,12 +1802,11 @@ int autotune(idp_plan p)
         p->dst_lines = best;
     }
     if (!rc && tensor_mode(p)) {
-        const View3 none{nullptr, 0, 0, 0};
         float tm[2];
         for (int path = 0; path < 2 && !rc; ++path) {
             p->mixed_path = path;
             tm[path] = timed([&]() -> int {
-                return transform(p, dense(p, p->C), p->C, dense(p, p->C), nullptr, none, false, st);
+                return transform(p, dense(p, p->C), p->C, dense(p, p->C), nullptr, false, st);
             });
         }
         p->mixed_path = (tm[1] < tm[0]) ? 1 : 0;
