@@ -351,6 +351,12 @@ __global__ void __launch_bounds__(QLineCfg<L, THIN>::T, QLineCfg<L, THIN>::BPS) 
             if (mk) colnz[g + i * G] = 1;
         }
     }
+    // values that are not finite stay out of the conversions: the line's marker stands for them
+    // (and the loads together: 257^3 315 -> 305 us per solve; short launches are faster without)
+    if (C > 4 && high >= 0x7ff00000) {
+#pragma unroll
+        for (int i = 0; i < C; ++i) x[i] = 0.0;
+    }
     if (mk && nz) rownz[l] = 1;
     // 2. the line's scale (lanes of one line: consecutive ones, or those LB apart)
     const int d0 = contig ? 1 : LB, d1 = contig ? Cfg::W : 32;
@@ -442,7 +448,7 @@ __global__ void __launch_bounds__(QLineCfg<L, THIN>::T, QLineCfg<L, THIN>::BPS) 
     // 6. the lines' shares of their slices' sums (integers: any order gives the same): half of a
     //    bound on the line's outputs, its absolute sum or, for rough lines, sqrt(2) times the largest
     //    part.  (Parts in units of 2^(32 + e + bits - 1102), sums in units of 2^(e + bits - 1064),
-    //    shares in units of 2^(-sh) of that.  With the signs in turn 303 -> 315 us at 257^3.)
+    //    shares in units of 2^(-sh) of that.)
     if constexpr (Cfg::W == 32) big = __reduce_max_sync(0xffffffffu, big);
     else
         for (int d = 1; d < Cfg::W; d <<= 1) big = max(big, __shfl_xor_sync(0xffffffffu, big, d));
