@@ -1762,13 +1762,13 @@ int autotune(idp_plan p)
         }
     }
     if (!rc) {
-        // block shape of the full-volume sine passes: the default, 8 lines on 256
-        // threads, 8 lines on 128 threads (M = 128), 32 lines (M = 128), 16
-        // lines (M = 256) or 4 lines on 128 threads (M = 256, 512); shapes that do
-        // not apply to a length fall back to the default.  Timed in whole solves: the transform of rho runs beside the
-        // boundary stages, so what a shape costs depends on what runs next to it
-        // (a shape can win alone and lose in the solve).  The density is a smooth
-        // bump over the middle of the box, zero near the boundary.
+        // block shape of the full-volume sine passes: the default, most lines per block (32),
+        // half of them (16) or few (8); in the tensor-core modes, whose double-float passes
+        // have shapes of their own, also 8 and 4 lines on 128 threads (-8: M = 128, 4: M = 256,
+        // 512).  Shapes that do not apply to a length fall back to the default.  Timed in
+        // whole solves: the transform of rho runs beside the boundary stages, so what a shape
+        // costs depends on what runs next to it (a shape can win alone and lose in the
+        // solve).  The density is a smooth bump over the middle of the box, zero near the boundary.
         std::vector<double> hr((size_t)p->nodes, 0.0);
         for (int i0 = 0; i0 < p->n[0]; ++i0)
             for (int i1 = 0; i1 < p->n[1]; ++i1)
@@ -1788,10 +1788,11 @@ int autotune(idp_plan p)
         if (e == cudaSuccess) e = cudaMalloc(&tphi, sizeof(double) * p->nodes);
         if (e == cudaSuccess) e = cudaMemcpy(trho, hr.data(), sizeof(double) * p->nodes, cudaMemcpyHostToDevice);
         if (e != cudaSuccess) rc = cuda_fail(e, "autotune buffers");
-        const int opts[6] = {0, 8, -8, 32, 16, 4};
+        const int opts[6] = {0, 8, 32, 16, -8, 4};
+        const int nopt = tensor_mode(p) ? 6 : 4;   // (-8 and 4 are 0 and 8 to the fixed-point pass)
         int best = 0;
         float bt = 1e30f;
-        for (int i = 0; i < 6 && !rc; ++i) {
+        for (int i = 0; i < nopt && !rc; ++i) {
             p->dst_lines = opts[i];
             const float t = timed([&]() -> int { return enqueue_grid(p, trho, tphi, 0, st); });
             if (t < bt) { bt = t; best = opts[i]; }
