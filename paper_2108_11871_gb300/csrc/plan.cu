@@ -7,6 +7,7 @@
 #include <atomic>
 #include <mutex>
 #include <new>
+#include <tuple>
 #include <algorithm>
 #include <vector>
 
@@ -229,6 +230,7 @@ struct idp_plan_s {
     static constexpr unsigned char GUARD_BYTE = 0xA5;
     std::vector<std::pair<char *, size_t>> guarded;   // allocation base, payload bytes
     int64_t bytes = 0;
+    bool released_dirty = false;                      // a guard of a released buffer was overwritten
 
     double *A = nullptr, *B = nullptr, *C = nullptr, *U = nullptr, *W = nullptr;
     double *tabc = nullptr, *tab4 = nullptr;
@@ -329,8 +331,38 @@ struct idp_plan_s {
         allocs.push_back(q);
         guarded.emplace_back(c, payload);
         if (e != cudaSuccess) return cuda_fail(e, "cudaMemset (guards)");
-        bytes += (int64_t)b;
+        bytes += (int64_t)payload;
         *p = (T *)(c + GUARD);
+        return IDP_OK;
+    }
+
+    // frees a buffer of alloc() (synchronises the device); its guards are looked at first
+    int release(void *q)
+    {
+        char *c = static_cast<char *>(q) - GUARD;
+        for (size_t i = 0; i < guarded.size(); ++i)
+            if (guarded[i].first == c) {
+                int rc = IDP_OK;
+                bool intact = true;
+                if ((rc = guards_intact(guarded[i], &intact))) return rc;
+                released_dirty = released_dirty || !intact;
+                bytes -= (int64_t)guarded[i].second;
+                guarded.erase(guarded.begin() + i);
+                allocs.erase(std::find(allocs.begin(), allocs.end(), (void *)c));
+                const cudaError_t e = cudaFree(c);
+                return e == cudaSuccess ? IDP_OK : cuda_fail(e, "cudaFree");
+            }
+        return IDP_EINVAL;
+    }
+
+    static int guards_intact(const std::pair<char *, size_t> &g, bool *intact)
+    {
+        unsigned char h[GUARD];
+        for (int side = 0; side < 2; ++side) {
+            const cudaError_t e = cudaMemcpy(h, side ? g.first + GUARD + g.second : g.first, GUARD, cudaMemcpyDeviceToHost);
+            if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpy (guards)");
+            for (unsigned char v : h) *intact = *intact && v == GUARD_BYTE;
+        }
         return IDP_OK;
     }
 };
@@ -1413,6 +1445,18 @@ int plan_setup_1d(idp_plan p)
     return plan_streams(p);
 }
 
+// the first face axis whose kernel spectra are those of axis a_
+int spectra_like(idp_plan p, int a_)
+{
+    auto key = [&](int s) {
+        const int b = s == 0 ? 1 : 0, c = s == 2 ? 1 : 2;
+        return std::make_tuple(p->ni[s], p->P[b], p->P[c], p->h[s], p->h[b], p->h[c]);
+    };
+    int s = 0;
+    while (key(s) != key(a_)) ++s;
+    return s;
+}
+
 int plan_setup(idp_plan p)
 {
     int rc;
@@ -1561,12 +1605,26 @@ int plan_setup(idp_plan p)
             IDP_CK(cudaMemcpy(tb, cb.data(), sizeof(double) * cb.size(), cudaMemcpyHostToDevice));
             IDP_CK(launch_gemm_batched(np, Mb + 1, Mb + 1, kb, Mb + 1, 0, tb, Mb + 1, 0, p->khat[face], Mb + 1, 0,
                                        1, 0));
+            if ((rc = p->release(kb)) || (rc = p->release(tb))) return rc;
             fmax = std::max<int64_t>(fmax, 2 * (Mb + 1));
         }
         if ((rc = p->alloc(&p->F, 2 * fmax))) return rc;
         p->f_cap = fmax;
     } else {
         int64_t pmax = 0, fmax = 0;
+        // temporaries of the spectra, built in slabs of slices that bound them: the kernel's
+        // values and their transform along c, the two cosine tables; one buffer for all axes
+        auto slab_of = [](int np, int64_t per) { return (int)std::max<int64_t>(1, std::min<int64_t>(np, (64 << 20) / (per * 8))); };
+        int64_t tslab = 0, ttab = 0;
+        for (int a_ = 0; a_ < 3; ++a_) {
+            const int b = a_ == 0 ? 1 : 0, c = a_ == 2 ? 1 : 2;
+            const int64_t per = (int64_t)(p->P[b] + 1) * (p->P[c] + 1);
+            tslab = std::max(tslab, (slab_of(p->ni[a_], per) * per + 31) / 32 * 32);
+            ttab = std::max(ttab, ((int64_t)(p->P[a_] + 1) * (p->P[a_] + 1) + 31) / 32 * 32);
+        }
+        double *kb;
+        if ((rc = p->alloc(&kb, 2 * (tslab + ttab)))) return rc;
+        double *yb = kb + tslab, *tcb = yb + tslab, *tbb = tcb + ttab;
         for (int a_ = 0; a_ < 3; ++a_) {
             const int b = a_ == 0 ? 1 : 0;
             const int c = a_ == 2 ? 1 : 2;
@@ -1594,14 +1652,18 @@ int plan_setup(idp_plan p)
             pmax = std::max<int64_t>(pmax, (int64_t)p->qchunk[a_] * 2 * L * (Mc + 1));
             fmax = std::max<int64_t>(fmax, (int64_t)2 * (Mb + 1) * (Mc + 1));
             const int64_t per = (int64_t)(Mb + 1) * (Mc + 1);
-            if ((rc = p->alloc(&p->khat[a_], (int64_t)np * per))) return rc;
             p->khat_n[a_] = (int64_t)np * per;
-            // build in slabs of slices to bound the temporaries
-            const int slab = std::max(1, (int)std::min<int64_t>(np, (int64_t)(64 << 20) / (per * 8)));
-            double *kb, *yb, *tcb, *tbb;
-            if ((rc = p->alloc(&kb, (int64_t)slab * per)) || (rc = p->alloc(&yb, (int64_t)slab * per)) ||
-                (rc = p->alloc(&tcb, (int64_t)(Mc + 1) * (Mc + 1))) || (rc = p->alloc(&tbb, (int64_t)(Mb + 1) * (Mb + 1))))
-                return rc;
+            // axes with the same lengths and mesh sizes have the same spectra (all three of a
+            // cube): kept once
+            const int like = spectra_like(p, a_);
+            if (like < a_) {
+                p->khat[a_] = p->khat[like];
+                p->kq[a_] = p->kq[like];
+                p->kq_ek[a_] = p->kq_ek[like];
+                continue;
+            }
+            if ((rc = p->alloc(&p->khat[a_], (int64_t)np * per))) return rc;
+            const int slab = slab_of(np, per);
             // the spectra are stored transposed, [slice][frequency c][frequency b]:
             //   khat^T = Cc^T K^T Cb^T  with  K^T[t_c][t_b] = G(d_p, t_b h_b, t_c h_c)
             std::vector<double> cct((size_t)(Mc + 1) * (Mc + 1)), cbt((size_t)(Mb + 1) * (Mb + 1));
@@ -1631,6 +1693,7 @@ int plan_setup(idp_plan p)
             if ((rc = p->alloc(&p->kq[a_], 2 * (int64_t)npair * per)) || (rc = p->alloc(&p->kq_ek[a_], per))) return rc;
             IDP_CK(launch_face_kq(p->khat[a_], np, per, p->kq[a_], p->kq_ek[a_], 0));
         }
+        if ((rc = p->release(kb))) return rc;
         if ((rc = p->alloc(&p->part, 3 * pmax)) || (rc = p->alloc(&p->F, 3 * fmax))) return rc;
         p->part_cap = pmax;
         p->f_cap = fmax;
@@ -2029,11 +2092,18 @@ int idp_plan_set(idp_plan p, int key, int64_t value)
         if (value != 0 && value != 1) return IDP_EINVAL;
         if (value && p->d == 3 && !p->khatd[0]) {
             int rc;
+            ddr *d[3];
             for (int a_ = 0; a_ < 3; ++a_) {
-                if ((rc = p->alloc(&p->khatd[a_], p->khat_n[a_]))) return rc;
-                IDP_CK(launch_to_dd(p->khat[a_], p->khatd[a_], p->khat_n[a_], 0));
+                const int like = spectra_like(p, a_);
+                if (like < a_) {
+                    d[a_] = d[like];
+                    continue;
+                }
+                if ((rc = p->alloc(&d[a_], p->khat_n[a_]))) return rc;
+                IDP_CK(launch_to_dd(p->khat[a_], d[a_], p->khat_n[a_], 0));
             }
             IDP_CK(cudaDeviceSynchronize());
+            for (int a_ = 0; a_ < 3; ++a_) p->khatd[a_] = d[a_];
         }
         if (p->mixed_bdd != (int)value) {
             p->mixed_bdd = (int)value;
@@ -2288,16 +2358,11 @@ int idp_plan_check_guards(idp_plan p)
 {
     if (!p) return IDP_EINVAL;
     IDP_CK(cudaDeviceSynchronize());
-    std::vector<unsigned char> h(idp_plan_s::GUARD);
-    for (const auto &g : p->guarded) {
-        for (int side = 0; side < 2; ++side) {
-            const char *src = side ? g.first + idp_plan_s::GUARD + g.second : g.first;
-            IDP_CK(cudaMemcpy(h.data(), src, idp_plan_s::GUARD, cudaMemcpyDeviceToHost));
-            for (unsigned char v : h)
-                if (v != idp_plan_s::GUARD_BYTE) return IDP_EGUARD;
-        }
-    }
-    return IDP_OK;
+    bool intact = !p->released_dirty;
+    int rc;
+    for (const auto &g : p->guarded)
+        if ((rc = idp_plan_s::guards_intact(g, &intact))) return rc;
+    return intact ? IDP_OK : IDP_EGUARD;
 }
 
 int idp_plan_grid(idp_plan p, int64_t n_solved[], int64_t offset[])
