@@ -134,7 +134,11 @@ enum {
 
 /* stages for idp_solve_stage */
 enum {
-    IDP_STAGE_BOUNDARY = 1, /* out: node array, g on the boundary, 0 inside (section 4) */
+    IDP_STAGE_BOUNDARY = 1, /* out: node array, g on the boundary, 0 inside (section 4).  Of a plan in a
+                               tensor-core mode with the FP64 boundary: the bits of an FP64 plan, from
+                               fixed-point FFTs; its solves and other stages take g from FP64 FFTs
+                               (rounding errors apart, a few 1e-15), and have it on the boundary
+                               nodes of phi and of IDP_STAGE_U1 */
     IDP_STAGE_GTILDE = 2,   /* out: interior array prod(n[s]-2), gtilde (eq. harmonic4thOrderNH2D) */
     IDP_STAGE_PHISTAR = 3,  /* out: node array, phi* (section 3), 0 on the boundary */
     IDP_STAGE_U1 = 4,       /* out: node array, u1 inside, g on the boundary (section 5) */
@@ -250,7 +254,8 @@ int idp_profile_solve(idp_plan plan, const double *rho, double *phi, void *strea
 
 /* Settings chosen by IDP_KEY_AUTOTUNE (or the defaults): out[0] = 1 if tuned,
  * out[1] = mixed path (0 tensor-core matrix, 1 double-float FFT), out[2..4] =
- * slice chunks of the face passes of axes 0..2, out[5..7] = slices per chunk,
+ * slice chunks of the face passes of axes 0..2, out[5..7] = slices per chunk (the
+ * chunks of a fixed-point pass take every out[2..4]-th pair of mirrored slices),
  * out[8] = block shape of the full-volume sine passes (IDP_KEY_DST_SHAPE values). */
 int idp_plan_tuning(idp_plan plan, int64_t out[9]);
 
