@@ -1605,7 +1605,7 @@ int plan_setup(idp_plan p)
             IDP_CK(cudaMemcpy(tb, cb.data(), sizeof(double) * cb.size(), cudaMemcpyHostToDevice));
             IDP_CK(launch_gemm_batched(np, Mb + 1, Mb + 1, kb, Mb + 1, 0, tb, Mb + 1, 0, p->khat[face], Mb + 1, 0,
                                        1, 0));
-            if ((rc = p->release(kb)) || (rc = p->release(tb))) return rc;
+            // (kb and tb stay: a few MB, and giving them back takes a tenth of the set-up)
             fmax = std::max<int64_t>(fmax, 2 * (Mb + 1));
         }
         if ((rc = p->alloc(&p->F, 2 * fmax))) return rc;

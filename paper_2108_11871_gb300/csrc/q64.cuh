@@ -204,7 +204,8 @@ __device__ __forceinline__ void q_pass(qc *X, const int4 *__restrict__ tw)
         if (UNITS % NT != 0 && b >= UNITS) break;
         // no factors at k = 0: the word pairs end 2^-62 below 1, and with it half of such
         // products would come out one unit low, a bias that DC adds up over the line (noise at
-        // 257^3: boundary values off by 2e-13, against 1e-15 in FP64 and without it)
+        // 257^3: boundary values off by 2.6e-13 with these products, 2.1e-14 without, before the
+        // signs in turn and the slice sums of face.cu)
         if (Ns > 1 && k != 0) {
             const int4 *w = tw + k;
 #pragma unroll

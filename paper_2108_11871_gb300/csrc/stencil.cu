@@ -639,7 +639,10 @@ __global__ void rhs6_e_kernel(const Grid3 gg, const StencilCoef c, const double 
 __global__ void layers_combine_kernel(double *__restrict__ P0, int pl0, double *__restrict__ P1, int pl1,
                                       double *__restrict__ P2, int pl2, int nl, const int *__restrict__ gmax)
 {
-    // gmax: fixed-point results, |a +- b| < 2^(gmax - 1040), so below 2^60 units
+    // gmax: fixed-point results, |a +- b| < 2^(gmax - 1040), so below 2^60 units.  One unit for
+    // the layers of all axes, which scale like 1 / h_s^2: on a stretched mesh the weak axis has
+    // fewer bits, which the eigenvalues take back (2-D 129^2, u1 against 80 bits: mesh ratio 100 off by
+    // 2.0e-14, with FP64 layers 1.8e-14; ratio 1e4 1.6e-14 both)
     const int gm = gmax ? min(*gmax, 2100) : 0;
     const QFrom from(1100 - gm, gm - 31);
     // 32-bit index arithmetic: at most 2 * 3 * 511^2 entries
