@@ -17,7 +17,7 @@
 // overflow: columns are below 2^61 units, S and D below 2^62 and S +- D below 2^63.  (One power
 // for all frequencies leaves the products' rounding as white noise over them: measured 1e-12
 // of g on mixed-sign densities.)  White noise, g off by, with the first bounds and now (FP64): 129^3 5.5e-15 and 1.6e-15
-// (1.5e-15), 257^3 2.5e-14 and 3.8e-15 (2.5e-15), 513^3 8.7e-14 and 4.7e-15 (2.4e-15).
+// (1.5e-15), 257^3 2.5e-14 and 4.5e-15 (2.5e-15), 513^3 8.7e-14 and 5.1e-15 (2.4e-15).
 #include "fft.cuh"
 #include "q64.cuh"
 
@@ -53,7 +53,11 @@ __device__ __forceinline__ void cp_async8(void *dst, const void *src)
                  : "memory");
 }
 
-template <int L>
+// Signs in turn (q64.cuh) over the pairs and the column blocks, by the pair's number, so that
+// the sums are the same integers for every chunk count.  ALT: an odd number of chunks, where
+// the pairs of a chunk alternate and the sum so far is turned with each of them (r - sum in place
+// of sum + r); with an even number all pairs of a chunk have one sign.
+template <int L, bool ALT>
 __global__ void __launch_bounds__(FaceQCfg<L>::NT, FaceQCfg<L>::BPS) face_q_kernel(const FaceQPass a)
 {
     using Cfg = FaceQCfg<L>;
@@ -90,7 +94,6 @@ __global__ void __launch_bounds__(FaceQCfg<L>::NT, FaceQCfg<L>::BPS) face_q_kern
     __syncthreads();
     const int unit = 1124 - ((s_bound >> 23) - 126) - 32 * win;
     if (threadIdx.x == 0 && blockIdx.x + blockIdx.y + blockIdx.z == 0) *a.unit = unit;
-    // signs in turn (q64.cuh) over the blocks and the pairs of a chunk
     int turns = blockIdx.x + chunk;
     QFrom from(unit, g - 31, q_turn(turns));
     const int2 *kq = a.kq + ((int64_t)diff * npair * a.nc + c0) * KS;
@@ -108,7 +111,17 @@ __global__ void __launch_bounds__(FaceQCfg<L>::NT, FaceQCfg<L>::BPS) face_q_kern
         const int p2 = a.np - 1 - pr;
         const bool two = pr != p2;
         // slices of zeros contribute nothing; the middle slice has no difference
-        if (!(a.sliceflag[pr] | a.sliceflag[p2]) || (!two && diff)) continue;
+        if (!(a.sliceflag[pr] | a.sliceflag[p2]) || (!two && diff)) {
+            if constexpr (ALT) {
+                from.flip();
+                ++turns;
+#pragma unroll
+                for (int it = 0; it < IL; ++it)
+#pragma unroll
+                    for (int q = 0; q < RL; ++q) acc[it][q] = qc{-acc[it][q].re, -acc[it][q].im};
+            }
+            continue;
+        }
         {
             const int2 *src = kq + (int64_t)pr * a.nc * KS;
             for (int f = threadIdx.x; f < ncl * KS; f += NT) cp_async8(ks + f, src + f);
@@ -171,13 +184,19 @@ __global__ void __launch_bounds__(FaceQCfg<L>::NT, FaceQCfg<L>::BPS) face_q_kern
             for (int q = 0; q < RL; ++q) {
                 const int m = j + q * UL;
                 const int2 w = k[m <= Ph ? m : L - m];
-                // the sum so far is turned with every pair, as the pair's values are
-                acc[it][q].re = q_rmul(v[q].re, w.x, w.y) - acc[it][q].re;
-                acc[it][q].im = q_rmul(v[q].im, w.x, w.y) - acc[it][q].im;
+                if constexpr (ALT) {
+                    acc[it][q].re = q_rmul(v[q].re, w.x, w.y) - acc[it][q].re;
+                    acc[it][q].im = q_rmul(v[q].im, w.x, w.y) - acc[it][q].im;
+                } else {
+                    acc[it][q].re += q_rmul(v[q].re, w.x, w.y);
+                    acc[it][q].im += q_rmul(v[q].im, w.x, w.y);
+                }
             }
         }
-        from.flip();
-        ++turns;
+        if constexpr (ALT) {
+            from.flip();
+            ++turns;
+        }
         __syncthreads();   // the buffer is free
     }
 #pragma unroll
@@ -185,7 +204,7 @@ __global__ void __launch_bounds__(FaceQCfg<L>::NT, FaceQCfg<L>::BPS) face_q_kern
         const int ct = column(it);
         if (ct >= ncl) continue;
         qc *part = a.part + (((int64_t)chunk * 2 + diff) * a.nc + c0 + ct) * L + freq(it);
-        const bool back = turns & 1;   // the last pair was not turned
+        const bool back = ((turns ^ (ALT ? 0 : 1)) & 1) != 0;   // the last pair was not turned
 #pragma unroll
         for (int q = 0; q < RL; ++q) part[q * UL] = back ? acc[it][q] : qc{-acc[it][q].re, -acc[it][q].im};
     }
@@ -236,7 +255,11 @@ __global__ void face_kq_kernel(const double *__restrict__ khat, int np, int64_t 
 template <int L>
 cudaError_t face_attr()
 {
-    return cudaFuncSetAttribute(face_q_kernel<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FaceQCfg<L>::SMEM);
+    const cudaError_t e = cudaFuncSetAttribute(face_q_kernel<L, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)FaceQCfg<L>::SMEM);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(face_q_kernel<L, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)FaceQCfg<L>::SMEM);
 }
 
 }  // namespace
@@ -254,7 +277,9 @@ cudaError_t launch_face_q(const FaceQPass &a, cudaStream_t st)
 {
     IDP_FACE_SWITCH(2 * a.Pb, {
         using Cfg = FaceQCfg<L>;
-        face_q_kernel<L><<<dim3((a.nc + Cfg::TC - 1) / Cfg::TC, a.nchunk, 2), Cfg::NT, Cfg::SMEM, st>>>(a);
+        const dim3 grid((a.nc + Cfg::TC - 1) / Cfg::TC, a.nchunk, 2);
+        if (a.nchunk & 1) face_q_kernel<L, true><<<grid, Cfg::NT, Cfg::SMEM, st>>>(a);
+        else face_q_kernel<L, false><<<grid, Cfg::NT, Cfg::SMEM, st>>>(a);
         return cudaGetLastError();
     })
 }

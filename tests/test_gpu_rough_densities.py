@@ -86,3 +86,31 @@ def test_sums_past_the_range_are_not_finite(n):
                 ref = np.ldexp(base, power)
             assert (~np.isfinite(got) | (got == ref)).all(), power
         assert not np.isfinite(got[ogreens.boundary_mask(n)]).any()
+
+
+@pytest.mark.parametrize("n", [(129, 129, 129), (97, 65, 129), (193, 33, 65), (65, 65, 65)],
+                         ids=lambda n: "x".join(map(str, n)))
+@pytest.mark.parametrize("kind", ["noise", "sparse"])
+def test_autotuning_leaves_the_bits(n, kind):
+    # the sums over slices are the same integers for every number of chunks (odd or even), with
+    # slices of zeros among them
+    import torch
+    import paper_2108_11871_gb300 as idp
+    rho = w.random_interior(n, seed=3)
+    if kind == "sparse":
+        rho[5:9] = 0.0
+        rho[20] = 0.0
+        rho[:, 11:14] = 0.0
+        rho[:, :, 7] = 0.0
+    r = torch.from_numpy(rho).cuda()
+    bits, chunks = set(), set()
+    for tune in (0, 1):
+        plan = idp.create_plan(3, n, [1.0 / (max(n) - 1)] * 3, 6)
+        idp.plan_set(plan, idp.IDP_KEY_AUTOTUNE, tune)
+        chunks.add(tuple(idp.plan_tuning(plan)["face_chunks"]))
+        out = torch.empty_like(r)
+        idp.solve(plan, r, out)
+        torch.cuda.synchronize()
+        bits.add(out.cpu().numpy().tobytes())
+    print(n, chunks)
+    assert len(bits) == 1
