@@ -47,9 +47,9 @@ KERNEL_NAMES = {1: "dst_pass", 2: "rfft", 3: "face", 4: "face_invb", 5: "face_c2
 # DRAM bytes (read + write) per full-volume launch of the sine pass, from ncu
 # (dram__bytes_read.sum + dram__bytes_write.sum over the 8 passes of one solve,
 # averaged); a grid not listed reports null
-# (profiles/dst_pass_257cube.md: 254 MB per launch at 257^3, scaled by the interior
-# points to 513^3)
-DST_TRAFFIC = {(257, 257, 257): 2.54e8, (513, 513, 513): 2.04e9}
+# (profiles/dst_pass_257cube.md: 249 MB per launch at 257^3, scaled by the interior
+# points to 513^3, where the plan is too large to capture: not a measurement there)
+DST_TRAFFIC = {(257, 257, 257): 2.49e8, (513, 513, 513): 2.00e9}
 
 
 def parse():

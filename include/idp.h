@@ -112,7 +112,8 @@ enum {
 enum {
     IDP_PRECISION_FP64 = 0,        /* FP64-class FFT-based transforms (default): FP64 in and out, the FFTs
                                       in 64-bit integers on a power-of-two scale per line (errors at or
-                                      below those of FP64 FFTs on smooth densities) */
+                                      below those of FP64 FFTs on smooth densities, at their level on
+                                      rough ones) */
     IDP_PRECISION_MIXED_BF16X3 = 1, /* the sine transforms of rho, of R and the final inverse become
                                       dense sine-matrix products on the tensor cores: operands split
                                       into three BF16 pieces, six products, FP32 accumulation
