@@ -70,14 +70,16 @@ __global__ void __launch_bounds__(FaceQCfg<L>::NT, FaceQCfg<L>::BPS) face_q_kern
     const int c0 = blockIdx.x * TC, ncl = min(TC, a.nc - c0);
     const int chunk = blockIdx.y, diff = blockIdx.z;
     const int npair = (a.np + 1) / 2;
+    // (the factors come in while the unit is found)
+    for (int f = threadIdx.x; f < Cfg::TW; f += NT)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(tws + f)),
+                     "l"(a.q + f)
+                     : "memory");
     const int g = min(*a.gmax, 2100);
-    for (int f = threadIdx.x; f < Cfg::TW; f += NT) tws[f] = __ldg(a.q + f);
     // The unit: every column's absolute sum, at most twice that of the slices' line bounds, below 2^61
     // units.  b: the largest sum over a pair of slices in units of 2^(32 win - 1064); lines two
     // windows below the largest one's add up to less than the 1
-    __shared__ int s_bound;
-    if (threadIdx.x == 0) s_bound = 0;
-    __syncthreads();
+    __shared__ int s_bound[NT / 32];
     const int win = g >> 5;
     {
         float b = 0.0f;
@@ -89,10 +91,14 @@ __global__ void __launch_bounds__(FaceQCfg<L>::NT, FaceQCfg<L>::BPS) face_q_kern
             b = fmaxf(b, __fadd_ru(__ull2float_ru(hi), __fmul_ru(__ull2float_ru(lo), 0x1p-32f)));
         }
         const int m = __reduce_max_sync(0xffffffffu, __float_as_int(__fadd_ru(b, 1.0f)));
-        if ((threadIdx.x & 31) == 0) atomicMax(&s_bound, m);
+        if ((threadIdx.x & 31) == 0) s_bound[threadIdx.x >> 5] = m;
     }
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
     __syncthreads();
-    const int unit = 1124 - ((s_bound >> 23) - 126) - 32 * win;
+    int bound = 0;
+#pragma unroll
+    for (int i = 0; i < NT / 32; ++i) bound = max(bound, s_bound[i]);
+    const int unit = 1124 - ((bound >> 23) - 126) - 32 * win;
     if (threadIdx.x == 0 && blockIdx.x + blockIdx.y + blockIdx.z == 0) *a.unit = unit;
     int turns = blockIdx.x + chunk;
     QFrom from(unit, g - 31, q_turn(turns));
